@@ -45,9 +45,22 @@ constexpr int EPI_THREADS = 128;
 constexpr int EPI_WARPS = EPI_THREADS / 32;
 constexpr int MAX_BANDS = 128;
 
+// A launch that leaves most of the chip's warps empty takes 256 or 512 threads
+// per row (NT): a row is one chain of dependent loads, and spreading its
+// nodes, filter samples and pixels over more warps shortens the chain (64 rows
+// of the paper-scale photometric fit: epilogue stage 28.7 -> 16.4 us, step 54.1 ->
+// 37.7 us; 301 rows with a 1111-pixel spectrum: 59.4 -> 28.7 us).  Every sum keeps the
+// 128-thread instance's terms and order, so a row's result does not depend on
+// the instance that computed it: the samples' interpolated values and the
+// pixels' residuals go through shared memory, and the sums over them run as
+// lanes of a warp per band and as EPI_THREADS threads over the pixels.
+// EPI_MISSED marks an excluded pixel there (a NaN no arithmetic produces).
+constexpr uint32_t EPI_MISSED = 0x7fa00001u;
+
 // dynamic shared memory: {lam, F/lam^2} and F over the row's window, the
-// included pixels' mu/sigma for the calibration moments, and, with emission
-// lines, per line ln(lam_obs) (an FP32 pair), F_l, A_l and 1/s_l
+// included pixels' mu/sigma for the calibration moments, with emission lines,
+// per line ln(lam_obs) (an FP32 pair), F_l, A_l and 1/s_l, and, with more than
+// EPI_THREADS threads, the samples' values and the pixels' residuals
 size_t epilogue_lines_off(const EpiArgs& a) {   // in floats, even (float2 alignment)
   const int np = a.row_model ? a.smem_pix : a.md.n_pix;
   const size_t W = (size_t)(a.row_model ? a.smem_win : a.md.win_max);
@@ -55,9 +68,13 @@ size_t epilogue_lines_off(const EpiArgs& a) {   // in floats, even (float2 align
   const size_t f = 2 * W + (np > 0 ? W : 0) + (calib ? (size_t)np : 0);
   return (f + 1) & ~(size_t)1;
 }
-size_t epilogue_smem(const EpiArgs& a) {
+size_t epilogue_terms_off(const EpiArgs& a) {   // in floats
   const bool lines = a.row_model ? a.g.n_line > 0 : a.md.use_lines != 0;
-  return (epilogue_lines_off(a) + (lines ? (size_t)5 * a.g.n_line : 0)) * sizeof(float);
+  return epilogue_lines_off(a) + (lines ? (size_t)5 * a.g.n_line : 0);
+}
+size_t epilogue_smem(const EpiArgs& a, int nt) {
+  const size_t terms = a.row_model ? (size_t)a.smem_samp + a.smem_pix : (size_t)a.md.n_samp + a.md.n_pix;
+  return (epilogue_terms_off(a) + (nt > EPI_THREADS ? terms : 0)) * sizeof(float);
 }
 
 // MULTI: rows of several fits (serving), row r reads model mtab[row_model[r]];
@@ -65,8 +82,8 @@ size_t epilogue_smem(const EpiArgs& a) {
 // instance with the emission lines (the one without keeps its code free of them).
 // VAR: 1 the age-binned attenuation (one Y per attenuated block), 2 the
 // nebular age axis (per-age ionising weights); 0 neither.
-template <bool MULTI, bool LINES, int VAR = 0>
-__global__ void __launch_bounds__(EPI_THREADS, 7) k_epilogue(const __grid_constant__ EpiArgs a) {
+template <bool MULTI, bool LINES, int VAR, int NT>
+__global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilogue(const __grid_constant__ EpiArgs a) {
   pdl_enter();
   const int r = blockIdx.x;
   const ModelDev& md = MULTI ? a.mtab[a.row_model[a.rs[r].orig]] : a.md;
@@ -124,7 +141,7 @@ __global__ void __launch_bounds__(EPI_THREADS, 7) k_epilogue(const __grid_consta
   // not unrolled: measured faster than unrolling by 2, 4 or 8 (1024-row
   // photometric step 0.0892 against 0.0906, 0.0927 and 0.0947 ms)
 #pragma unroll 1
-  for (int k = k_lo + tid; k <= k_hi; k += EPI_THREADS) {
+  for (int k = k_lo + tid; k <= k_hi; k += NT) {
     const float4 c = g.att4[k];
     const float ys = a.lam8 ? rs.y_scale * a.lam8[k] : 1.f;
     const float o = O2r ? Or[k] + O2r[k] : Or[k];
@@ -152,23 +169,57 @@ __global__ void __launch_bounds__(EPI_THREADS, 7) k_epilogue(const __grid_consta
   float* ln_F = reinterpret_cast<float*>(ln_x + NLn);
   float* ln_A = ln_F + NLn;
   float* ln_is = ln_A + NLn;
-  for (int l = tid; l < NLn; l += EPI_THREADS) line_setup(md, g, rs, eb, l, ln_F, ln_A, ln_is, ln_x);
+  for (int l = tid; l < NLn; l += NT) line_setup(md, g, rs, eb, l, ln_F, ln_A, ln_is, ln_x);
   __syncthreads();
   if (LINES && a.lines_out) {   // the lines' fluxes only (sed_line_fluxes)
-    for (int l = tid; l < NLn; l += EPI_THREADS) a.lines_out[(size_t)ro * NLn + l] = ln_F[l];
+    for (int l = tid; l < NLn; l += NT) a.lines_out[(size_t)ro * NLn + l] = ln_F[l];
     if (!a.lnl && !a.phot_out && !a.spec_out) return;
   }
 
-  // ---- photometry, one band per warp.  Consecutive lanes take consecutive
-  //      filter samples (coalesced loads, eight in flight per lane); each
-  //      sample's bracket starts from the index table over ln(lambda) at the
-  //      sample's rest-frame wavelength and is corrected by a walk within the
-  //      row's window in shared memory (any start gives the same bracket, so a
-  //      fast logarithm serves).  Lane-strided sums and a fixed shuffle tree
-  //      keep the order of the band sum fixed.
+  // ---- photometry.  Each sample's bracket starts from the index table over
+  //      ln(lambda) at the sample's rest-frame wavelength and is corrected by a
+  //      walk within the row's window in shared memory (any start gives the same
+  //      bracket, so a fast logarithm serves).
   const float lam0 = g.lam_f[0], lamN = g.lam_f[N - 1];
-  {
-    const int kmin = k_lo, kmax = k_hi - 1;
+  const int kmin = k_lo, kmax = k_hi - 1;
+  auto sample_start = [&](float lam_obs) {
+    int q = (int)((__logf(fmaxf(lam_obs * rs.inv1pz, lam0)) - g.lut_x0) * g.lut_inv_h);
+    q = q < 0 ? 0 : (q >= g.lut_n ? g.lut_n - 1 : q);
+    return g.lut[q];
+  };
+  // F/lam^2 at the rest-frame wavelength x, from the start k
+  auto sample_value = [&](float x, int k) {
+    int kc = min(max(k, kmin), kmax);
+#pragma unroll 1
+    while (kc < kmax && LG[kc + 1].x <= x) ++kc;
+#pragma unroll 1
+    while (kc > kmin && LG[kc].x > x) --kc;
+    const float2 p0 = LG[kc], p1 = LG[kc + 1];
+    const float t = __fdividef(x - p0.x, p1.x - p0.x);
+    return p0.y + t * (p1.y - p0.y);
+  };
+  // the band's flux from its lanes' sample sums, plus the lines in it (one line
+  // per lane); a fixed shuffle tree keeps the order of the sum fixed
+  auto band_finish = [&](int b, float acc) {
+#pragma unroll
+    for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    float lsum = 0.f;
+    if (LINES && NLn) {
+      for (int l = lane; l < NLn; l += 32) lsum += line_in_band(md, g, rs, b, l, ln_F[l]);
+#pragma unroll
+      for (int o = 16; o; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+    }
+    if (lane == 0) {
+      const float mb = LINES && NLn ? fmaf(rs.p_phot, acc, lsum) : rs.p_phot * acc;
+      if (a.phot_out) a.phot_out[(size_t)ro * md.n_filt + b] = mb;
+      mb_s[b] = mb;
+    }
+  };
+  float* v_s = reinterpret_cast<float*>(smem4) + a.terms_off;   // NT > EPI_THREADS: the samples' values,
+  float* rn_s = v_s + md.n_samp;                                // then the pixels' residuals
+  if constexpr (NT == EPI_THREADS) {
+    // one band per warp: consecutive lanes take consecutive samples (coalesced
+    // loads, eight in flight per lane)
     for (int b = warp; b < md.n_filt; b += EPI_WARPS) {
       const int j1 = md.band_start[b + 1];
       float acc = 0.f;
@@ -178,39 +229,28 @@ __global__ void __launch_bounds__(EPI_THREADS, 7) k_epilogue(const __grid_consta
 #pragma unroll
         for (int u = 0; u < 8; ++u) sp[u] = j0 + 32 * u < j1 ? md.samp2[j0 + 32 * u] : make_float2(0.f, 0.f);
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          int q = (int)((__logf(fmaxf(sp[u].x * rs.inv1pz, lam0)) - g.lut_x0) * g.lut_inv_h);
-          q = q < 0 ? 0 : (q >= g.lut_n ? g.lut_n - 1 : q);
-          kg[u] = g.lut[q];
-        }
+        for (int u = 0; u < 8; ++u) kg[u] = sample_start(sp[u].x);
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
           const float x = sp[u].x * rs.inv1pz;
-          if (x >= lam0 && x <= lamN) {
-            int kc = min(max(kg[u], kmin), kmax);
-#pragma unroll 1
-            while (kc < kmax && LG[kc + 1].x <= x) ++kc;
-#pragma unroll 1
-            while (kc > kmin && LG[kc].x > x) --kc;
-            const float2 p0 = LG[kc], p1 = LG[kc + 1];
-            const float t = __fdividef(x - p0.x, p1.x - p0.x);
-            acc = fmaf(sp[u].y, p0.y + t * (p1.y - p0.y), acc);
-          }
+          if (x >= lam0 && x <= lamN) acc = fmaf(sp[u].y, sample_value(x, kg[u]), acc);
         }
       }
+      band_finish(b, acc);
+    }
+  } else {
+    for (int j0 = tid; j0 < md.n_samp; j0 += 4 * NT) {
+      float x[4];
+      int kg[4];
 #pragma unroll
-      for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      // the lines in this band, one line per lane
-      float lsum = 0.f;
-      if (LINES && NLn) {
-        for (int l = lane; l < NLn; l += 32) lsum += line_in_band(md, g, rs, b, l, ln_F[l]);
+      for (int u = 0; u < 4; ++u) x[u] = j0 + u * NT < md.n_samp ? md.samp2[j0 + u * NT].x : 0.f;
 #pragma unroll
-        for (int o = 16; o; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-      }
-      if (lane == 0) {
-        const float mb = LINES && NLn ? fmaf(rs.p_phot, acc, lsum) : rs.p_phot * acc;
-        if (a.phot_out) a.phot_out[(size_t)ro * md.n_filt + b] = mb;
-        mb_s[b] = mb;
+      for (int u = 0; u < 4; ++u) kg[u] = sample_start(x[u]);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (j0 + u * NT >= md.n_samp) break;
+        const float xr = x[u] * rs.inv1pz;
+        v_s[j0 + u * NT] = xr >= lam0 && xr <= lamN ? sample_value(xr, kg[u]) : 0.f;
       }
     }
   }
@@ -221,7 +261,14 @@ __global__ void __launch_bounds__(EPI_THREADS, 7) k_epilogue(const __grid_consta
   double part = 0.0;
   float chi = 0.f;
   const float ll0 = g.lnl_hi[0], llN = g.lnl_hi[N - 1];
-  for (int i = tid; i < md.n_pix; i += blockDim.x) {
+  // an included pixel's term of the running sum: the residual squared, or twice
+  // minus the term with the noise floor (sigma_eff of Eq. app_noise_floor)
+  auto add_term = [&](float t, int i) {
+    if (md.floor_bits[1]) chi -= 0.5f * t;
+    else chi = fmaf(-0.5f * t, t, chi);
+    part += md.spec_nlog[i];
+  };
+  for (int i = tid; i < md.n_pix; i += NT) {
     float xh, xl;
     ln_rest(md.pix_ln2[i], rs.ln1pz_hi, rs.ln1pz_lo, xh, xl);
     float v = 0.f;
@@ -265,29 +312,46 @@ __global__ void __launch_bounds__(EPI_THREADS, 7) k_epilogue(const __grid_consta
     const float isf = md.spec_isf[i];
     const bool inc = valid && isf != 0.f;
     const float ms = inc ? mi * isf : 0.f;   // mu / sigma
-    if (inc) {
-      const float dn = md.spec_dn[i], rn = dn - ms;   // (d - mu) / sigma
-      if (md.floor_bits[1]) {                         // sigma_eff of Eq. app_noise_floor
-        const float q = floor_q(rs.fl[1], ms, dn, rs.fl[1][3] * isf);
-        chi -= 0.5f * (rn * rn / q + logf(q));
-      } else {
-        chi = fmaf(-0.5f * rn, rn, chi);
-      }
-      part += md.spec_nlog[i];
+    const float dn = md.spec_dn[i];
+    float t = dn - ms;                       // (d - mu) / sigma
+    if (inc && md.floor_bits[1]) {
+      const float q = floor_q(rs.fl[1], ms, dn, rs.fl[1][3] * isf);
+      t = t * t / q + logf(q);
+    }
+    if constexpr (NT == EPI_THREADS) {
+      if (inc) add_term(t, i);
+    } else {
+      rn_s[i] = inc ? t : __uint_as_float(EPI_MISSED);
     }
     if (md.calib_n) mu_s[i] = ms;
   }
+  if constexpr (NT > EPI_THREADS) {
+    __syncthreads();
+    for (int b = NT / 32 - 1 - warp; b < md.n_filt; b += NT / 32) {   // the first warps have the pixels' sums below
+      float acc = 0.f;
+#pragma unroll 8
+      for (int j = md.band_start[b] + lane; j < md.band_start[b + 1]; j += 32) acc = fmaf(md.samp2[j].y, v_s[j], acc);
+      band_finish(b, acc);
+    }
+    if (tid < EPI_THREADS)
+      for (int i = tid; i < md.n_pix; i += EPI_THREADS) {
+        const float t = rn_s[i];
+        if (__float_as_uint(t) != EPI_MISSED) add_term(t, i);
+      }
+  }
   part += (double)chi;
   // calibration moments over this thread's own pixels (no barrier needed),
-  // in three blocks of sums (S_0..12, S_13..24, b_0..12), each summed per warp
-  if (md.calib_n) {
+  // in three blocks of sums (S_0..12, S_13..24, b_0..12), each summed per warp;
+  // the first EPI_WARPS warps own the pixels in every instance
+  const bool own = NT == EPI_THREADS || tid < EPI_THREADS;
+  if (md.calib_n && own) {
     calib_block<0, 0, EPI_THREADS>(md, mu_s, cal_c, tid, lane, warp, &cal_part[0][0]);
     calib_block<SED_MAX_CALIB, 0, EPI_THREADS>(md, mu_s, cal_c, tid, lane, warp, &cal_part[0][0]);
     calib_block<0, 1, EPI_THREADS>(md, mu_s, cal_c, tid, lane, warp, &cal_part[0][0]);
   }
 #pragma unroll
   for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-  if (lane == 0) red[warp] = part;
+  if (lane == 0 && own) red[warp] = part;
   __syncthreads();
   if (md.calib_n) {
     // sum the warps' moments in warp order into row 0, factor M and solve for
@@ -298,7 +362,7 @@ __global__ void __launch_bounds__(EPI_THREADS, 7) k_epilogue(const __grid_consta
       if (lane == 0) cal_fix = f;
     }
     __syncthreads();
-    calib_block<0, 2, EPI_THREADS>(md, mu_s, cal_c, tid, lane, warp, &cal_part[0][0]);
+    if (own) calib_block<0, 2, EPI_THREADS>(md, mu_s, cal_c, tid, lane, warp, &cal_part[0][0]);
     __syncthreads();
     if (warp == 0) {
       const double f = calib_refine(md, &cal_part[0][0], EPI_WARPS, cal_L, cal_D, cal_c, lane);
@@ -306,7 +370,7 @@ __global__ void __launch_bounds__(EPI_THREADS, 7) k_epilogue(const __grid_consta
     }
     __syncthreads();
     float cpf = 0.f;
-    for (int i = tid; i < md.n_pix; i += EPI_THREADS) {
+    for (int i = own ? tid : md.n_pix; i < md.n_pix; i += EPI_THREADS) {
       const float ms = mu_s[i];
       if (ms == 0.f) continue;
       cpf += calib_pixel_term(md.spec_dn[i] - ms, ms, calib_poly(cal_c, md.calib_n, md.pix_cx[i]));
@@ -314,7 +378,7 @@ __global__ void __launch_bounds__(EPI_THREADS, 7) k_epilogue(const __grid_consta
     double cp = (double)cpf;
 #pragma unroll
     for (int o = 16; o; o >>= 1) cp += __shfl_xor_sync(0xffffffffu, cp, o);
-    if (lane == 0) red[warp] += cp;
+    if (lane == 0 && own) red[warp] += cp;
     __syncthreads();
   }
   // photometric terms in FP64, one band per lane of warp 0 (GB300's FP64 pipe
@@ -350,23 +414,35 @@ __global__ void __launch_bounds__(EPI_THREADS, 7) k_epilogue(const __grid_consta
   }
 }
 
-cudaError_t launch_epilogue(const EpiArgs& a_in, cudaStream_t s) {
-  EpiArgs a = a_in;
-  a.lines_off = (int)epilogue_lines_off(a);
-  const size_t smem = epilogue_smem(a);
+template <int NT>
+cudaError_t launch_epilogue_nt(const EpiArgs& a, cudaStream_t s) {
+  const size_t smem = epilogue_smem(a, NT);
   static DynSmemCache set_for[6];
   const bool lines = a.row_model ? a.g.n_line > 0 : a.md.use_lines != 0;
   // age-binned dust and the nebular age axis: neither served nor with lines
   const bool bins = !a.row_model && a.md.n_bin > 0, axis = !a.row_model && a.qneb;
   const int m = bins ? 4 : axis ? 5 : (a.row_model ? 1 : 0) + (lines ? 2 : 0);
-  auto k = m == 0 ? k_epilogue<false, false>
-         : m == 1 ? k_epilogue<true, false>
-         : m == 2 ? k_epilogue<false, true>
-         : m == 3 ? k_epilogue<true, true>
-         : m == 4 ? k_epilogue<false, false, 1> : k_epilogue<false, false, 2>;
+  auto k = m == 0 ? k_epilogue<false, false, 0, NT>
+         : m == 1 ? k_epilogue<true, false, 0, NT>
+         : m == 2 ? k_epilogue<false, true, 0, NT>
+         : m == 3 ? k_epilogue<true, true, 0, NT>
+         : m == 4 ? k_epilogue<false, false, 1, NT> : k_epilogue<false, false, 2, NT>;
   cudaError_t e = ensure_dyn_smem(k, smem, &set_for[m]);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k, dim3(a.n), dim3(EPI_THREADS), smem, s, a);
+  return launch_pdl(k, dim3(a.n), dim3(NT), smem, s, a);
+}
+
+cudaError_t launch_epilogue(const EpiArgs& a_in, cudaStream_t s) {
+  EpiArgs a = a_in;
+  a.lines_off = (int)epilogue_lines_off(a);
+  a.terms_off = (int)epilogue_terms_off(a);
+  // Threads per row: as many as keep every row of the launch resident at once
+  // (1024 threads per SM at 64 registers), where their shared memory fits.
+  const int sm = device_sm_count();
+  const size_t room = (size_t)220 * 1024;
+  if (a.n <= 2 * sm && 2 * epilogue_smem(a, 512) <= room) return launch_epilogue_nt<512>(a, s);
+  if (a.n <= 4 * sm && 4 * epilogue_smem(a, 256) <= room) return launch_epilogue_nt<256>(a, s);
+  return launch_epilogue_nt<EPI_THREADS>(a, s);
 }
 
 }  // namespace sed
