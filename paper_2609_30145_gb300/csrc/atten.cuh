@@ -29,38 +29,48 @@ __device__ __forceinline__ float dust_shape(const ModelDev& md, const float4& c,
   return md.dust_law == SED_DUST_POWER_LAW ? pw : (c.y + eb * c.z) * pw;
 }
 
+// A node's four template corners: the cell's float4 where the grid keeps them
+// together, else one load per corner.
+__device__ __forceinline__ float4 neb_corners(const RowScal& rs, const GridDev& g, int k) {
+  if (g.neb4) return __ldg(g.neb4 + rs.neb_cell + k);
+  return make_float4(g.neb_tab[rs.neb_off[0] + k], g.neb_tab[rs.neb_off[1] + k], g.neb_tab[rs.neb_off[2] + k],
+                     g.neb_tab[rs.neb_off[3] + k]);
+}
+__device__ __forceinline__ float neb_log10(const RowScal& rs, const float4& t) {
+  return rs.neb_w[0] * t.x + rs.neb_w[1] * t.y + rs.neb_w[2] * t.z + rs.neb_w[3] * t.w;
+}
 __device__ __forceinline__ float neb_log10(const RowScal& rs, const float* tab, int k) {
-  return rs.neb_w[0] * tab[rs.neb_off[0] + k] + rs.neb_w[1] * tab[rs.neb_off[1] + k] +
-         rs.neb_w[2] * tab[rs.neb_off[2] + k] + rs.neb_w[3] * tab[rs.neb_off[3] + k];
+  return neb_log10(rs, make_float4(tab[rs.neb_off[0] + k], tab[rs.neb_off[1] + k], tab[rs.neb_off[2] + k],
+                                   tab[rs.neb_off[3] + k]));
 }
 
 // Nebular emission at node k (device units): Q_young 10^template, or with a
 // nebular age axis (App. C) the sum over the nebular SSP ages of q_a 10^(the
-// cube at that age), qa the row's q_a (NULL without an axis).
+// cube at that age), qa the row's q_a.
+__device__ __forceinline__ float neb_emission(const RowScal& rs, const float4& t) {
+  return ex2_approx(rs.log2_qy + 3.3219280948873623f * neb_log10(rs, t));
+}
 __device__ __forceinline__ float neb_emission(const RowScal& rs, const GridDev& g, const float* qa, int k) {
-  if (qa) {
-    const size_t plane = (size_t)g.neb_nu * g.neb_nz * g.n_lam;
-    float acc = 0.f;
-    for (int i = 0; i < g.neb_na; ++i) {
-      const float q = qa[i];
-      if (q != 0.f) acc = fmaf(q, ex2_approx(3.3219280948873623f * neb_log10(rs, g.neb_tab + i * plane, k)), acc);
-    }
-    return acc;
+  const size_t plane = (size_t)g.neb_nu * g.neb_nz * g.n_lam;
+  float acc = 0.f;
+  for (int i = 0; i < g.neb_na; ++i) {
+    const float q = qa[i];
+    if (q != 0.f) acc = fmaf(q, ex2_approx(3.3219280948873623f * neb_log10(rs, g.neb_tab + i * plane, k)), acc);
   }
-  return ex2_approx(rs.log2_qy + 3.3219280948873623f * neb_log10(rs, g.neb_tab, k));
+  return acc;
 }
 
-// c = {ln(lam/5500), k'/4.05, Drude/4.05, 1/lam^2}; eb = 0.85 - 1.9 delta
+// c = {ln(lam/5500), k'/4.05, Drude/4.05, 1/lam^2}; eb = 0.85 - 1.9 delta; nb the
+// node's nebular emission (0 without)
 __device__ __forceinline__ float attenuated(const ModelDev& md, const RowScal& rs, const float4& c, float eb, float y,
-                                           float o, const GridDev& g, const float* qa, int k) {
+                                           float o, float nb, int k) {
   const float tbc = rs.tau_bc * __expf(rs.alpha_bc * c.x);
   const float pw = __expf(rs.delta * c.x);
   const float td = rs.tau_d * dust_shape(md, c, eb, pw);
   if (md.fesc_geom == SED_FESC_NONE) {
-    if (md.use_neb) y += neb_emission(rs, g, qa, k);
+    if (md.use_neb) y += nb;
     return __expf(-td) * (__expf(-tbc) * y + o);
   }
-  const float nb = md.use_neb ? neb_emission(rs, g, qa, k) : 0.f;
   const bool lyc = md.use_neb && k < md.n_lyc;
   const float ys = lyc ? 0.f : y, f = rs.fob, ed = __expf(-td), ebc = __expf(-tbc);
   if (md.fesc_geom == SED_FESC_PICKET) return f * y + ed * ((1.f - f) * ebc * (ys + nb) + o);
@@ -81,12 +91,12 @@ __device__ __forceinline__ float bin_shape(int law, const float4& c, float slope
 }
 
 __device__ __forceinline__ float attenuated_bins(const ModelDev& md, const RowScal& rs, const float4& c, float eb,
-                                                const float* y, float o, const float* neb_tab, int k) {
+                                                const float* y, float o, const GridDev& g, int k) {
   float kap[MAX_DUST_BIN];
 #pragma unroll
   for (int b = 0; b < MAX_DUST_BIN; ++b)
     kap[b] = b < md.n_bin ? rs.bin_tau[b] * bin_shape(md.bin_law[b], c, rs.bin_slope[b]) : 0.f;
-  const float lg = md.use_neb ? 3.3219280948873623f * neb_log10(rs, neb_tab, k) : 0.f;
+  const float lg = md.use_neb ? 3.3219280948873623f * neb_log10(rs, neb_corners(rs, g, k)) : 0.f;
   float acc = o;
   if (md.use_neb) acc += ex2_approx(rs.log2_qs[MAX_SEG] + lg);
 #pragma unroll

@@ -193,9 +193,10 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
       float yv[MAX_SEG];
 #pragma unroll
       for (int sg = 0; sg < MAX_SEG; ++sg) yv[sg] = sg < md.n_seg ? Yr[sg * a.seg_stride + k] : 0.f;
-      Fs[k] = attenuated_bins(md, rs, g.att4[k], eb_kc, yv, O2r ? Or[k] + O2r[k] : Or[k], g.neb_tab, k);
+      Fs[k] = attenuated_bins(md, rs, g.att4[k], eb_kc, yv, O2r ? Or[k] + O2r[k] : Or[k], g, k);
     } else {
-      Fs[k] = attenuated(md, rs, g.att4[k], eb_kc, Yr[k], O2r ? Or[k] + O2r[k] : Or[k], g, qa, k);
+      const float nb = !md.use_neb ? 0.f : VAR == 2 ? neb_emission(rs, g, qa, k) : neb_emission(rs, neb_corners(rs, g, k));
+      Fs[k] = attenuated(md, rs, g.att4[k], eb_kc, Yr[k], O2r ? Or[k] + O2r[k] : Or[k], nb, k);
     }
     if (md.use_igm && g.lam_f[k] < IGM_LYA) {   // the IGM transmission (the forward epilogue's)
       float tau, dtau;
@@ -743,7 +744,7 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
       const float ed = __expf(-rs.tau_d * shape);
       float lg = 0.f, nbu = 0.f;   // log10 and value of the nebular template per unit Q
       if (md.use_neb) {
-        lg = neb_log10(rs, g.neb_tab, k);
+        lg = neb_log10(rs, neb_corners(rs, g, k));
         nbu = ex2_approx(3.3219280948873623f * lg);
       }
       // with the IGM, F = T F0: dlnL/dF0 = T dlnL/dF, and ln T = -f tau moves with f and z
@@ -837,7 +838,7 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
       if (qa) {
         nb = neb_emission(rs, g, qa, k);
       } else {
-        lg = neb_log10(rs, g.neb_tab, k);
+        lg = neb_log10(rs, neb_corners(rs, g, k));
         nb = ex2_approx(rs.log2_qy + 3.3219280948873623f * lg);
       }
     }

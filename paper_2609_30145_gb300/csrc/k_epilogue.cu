@@ -40,7 +40,12 @@ namespace sed {
 // the kernel is bound by the latency of its gathers, so rows in flight is what
 // sets its speed, and the 72 registers that 7 CTAs leave a thread (against 64
 // at 8) keep more of each thread's loads in flight (measured 0.0988 against
-// 0.1029 ms per 1024-row step).
+// 0.1029 ms per 1024-row step).  Of a 1024-row photometric launch the row's
+// fixed part takes about 6 us, its nodes 11 us and its samples 6 us; copying Y
+// and O of all nodes at once, one load for the nebular corners, samples without
+// walks and shared-memory words without the pairs' bank conflicts took the
+// epilogue stage from 34.8 to 26.6 us (1024 rows) and 116.7 to 79.9 us (4096
+// rows, BF16).
 constexpr int EPI_THREADS = 128;
 constexpr int EPI_WARPS = EPI_THREADS / 32;
 constexpr int MAX_BANDS = 128;
@@ -56,8 +61,12 @@ constexpr int MAX_BANDS = 128;
 // lanes of a warp per band and as EPI_THREADS threads over the pixels.
 // EPI_MISSED marks an excluded pixel there (a NaN no arithmetic produces).
 constexpr uint32_t EPI_MISSED = 0x7fa00001u;
+// From this many threads on, a band's samples are spread over all of them; below
+// it a warp takes a band (no shared memory for the samples' values, which would
+// cost the 256-thread instance with a spectrum its fourth CTA per SM).
+constexpr int EPI_FLAT = 512;
 
-// dynamic shared memory: {lam, F/lam^2} and F over the row's window, the
+// dynamic shared memory: lam, F/lam^2 and F over the row's window, the
 // included pixels' mu/sigma for the calibration moments, with emission lines,
 // per line ln(lam_obs) (an FP32 pair), F_l, A_l and 1/s_l, and, with more than
 // EPI_THREADS threads, the samples' values and the pixels' residuals
@@ -73,9 +82,30 @@ size_t epilogue_terms_off(const EpiArgs& a) {   // in floats
   return epilogue_lines_off(a) + (lines ? (size_t)5 * a.g.n_line : 0);
 }
 size_t epilogue_smem(const EpiArgs& a, int nt) {
-  const size_t terms = a.row_model ? (size_t)a.smem_samp + a.smem_pix : (size_t)a.md.n_samp + a.md.n_pix;
-  return (epilogue_terms_off(a) + (nt > EPI_THREADS ? terms : 0)) * sizeof(float);
+  const size_t pix = a.row_model ? a.smem_pix : a.md.n_pix;
+  const size_t samp = 32 * (size_t)(a.row_model ? a.smem_samp : a.md.n_samp32);
+  return (epilogue_terms_off(a) + (nt > EPI_THREADS ? pix : 0) + (nt >= EPI_FLAT ? samp : 0)) * sizeof(float);
 }
+
+// a / b by the hardware's reciprocal, subnormals as zero (a and b here are
+// differences of wavelengths: zero or far above the subnormals)
+__device__ __forceinline__ float div_approx(float a, float b) {
+  float q;
+  asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(q) : "f"(a), "f"(b));
+  return q;
+}
+
+__device__ __forceinline__ float lg2_approx(float x) {
+  float y;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// four bytes of global memory to shared memory without a register (the thread
+// itself reads them after cp_async_wait_all)
+__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // MULTI: rows of several fits (serving), row r reads model mtab[row_model[r]];
 // otherwise every row reads the model in the kernel parameters.  LINES: an
@@ -84,8 +114,8 @@ size_t epilogue_smem(const EpiArgs& a, int nt) {
 // nebular age axis (per-age ionising weights); 0 neither.
 template <bool MULTI, bool LINES, int VAR, int NT>
 __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilogue(const __grid_constant__ EpiArgs a) {
-  pdl_enter();
   const int r = blockIdx.x;
+  if constexpr (MULTI) pdl_enter();
   const ModelDev& md = MULTI ? a.mtab[a.row_model[a.rs[r].orig]] : a.md;
   const GridDev& g = a.g;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -100,6 +130,15 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
   __shared__ float cal_part[EPI_WARPS][CAL_NV];    // per-warp calibration sums
   __shared__ float cal_L[SED_MAX_CALIB * SED_MAX_CALIB], cal_D[SED_MAX_CALIB], cal_c[SED_MAX_CALIB];  // M = L L^T, 1/L_ii, c*
   __shared__ double cal_fix;                       // the row's lnL terms that do not sum over pixels
+
+  // the bands' extents and data, read in the shadow of the kernel before
+  __shared__ int b32_s[MAX_BANDS + 1];
+  __shared__ double3 band_s[MAX_BANDS];   // {datum, 1/sigma, -ln(2 pi sigma^2)/2}
+  for (int b = tid; b <= md.n_filt && md.n_filt > 0; b += NT) {
+    b32_s[b] = md.band32[b];
+    if (b < md.n_filt) band_s[b] = make_double3(md.phot_d[b], md.phot_isig[b], md.phot_nlog[b]);
+  }
+  if constexpr (!MULTI) pdl_enter();
 
   if (a.win_reset && r == 0) empty_windows(a.win_reset, a.win_mt);
   RowScal rs = a.rs[r];
@@ -135,24 +174,47 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
   }
   const bool spec = md.n_pix > 0;
   const int k_lo = rs.k_lo, k_hi = min(rs.k_hi, rs.k_lo + WIN - 1);   // nodes [k_lo, k_hi] are the only ones read below
-  float2* LG = reinterpret_cast<float2*>(smem4) - k_lo;               // {rest-frame lambda, F / lam^2}
-  float* Fs = reinterpret_cast<float*>(reinterpret_cast<float2*>(smem4) + WIN) - k_lo;   // F (spectral arm only)
-  float* mu_s = reinterpret_cast<float*>(reinterpret_cast<float2*>(smem4) + WIN) + WIN;  // calibration: included pixels' mu/sigma (0 elsewhere)
-  // not unrolled: measured faster than unrolling by 2, 4 or 8 (1024-row
-  // photometric step 0.0892 against 0.0906, 0.0927 and 0.0947 ms)
+  // Rest-frame lambda and F / lam^2, as two arrays: a warp's samples lie one to
+  // two nodes apart, so one word per node makes half the bank conflicts of a pair
+  float* Ls = reinterpret_cast<float*>(smem4) - k_lo;
+  float* Gs = Ls + WIN;
+  float* Fs = Gs + WIN;                                                // F (spectral arm only)
+  float* mu_s = reinterpret_cast<float*>(smem4) + 3 * WIN;             // calibration: included pixels' mu/sigma (0 elsewhere)
+  // Y and O of all the thread's nodes are copied to the nodes' own places in the
+  // two arrays at once; the other loads of the next node are issued before this
+  // node's arithmetic (the loop, not unrolled, waits on L2 otherwise)
+  if constexpr (VAR != 1)
+    for (int k = k_lo + tid; k <= k_hi; k += NT) {
+      cp_async4(Ls + k, Yr + k);
+      cp_async4(Gs + k, Or + k);
+    }
+  struct Node { float o2; float4 c, nt; };
+  auto load_node = [&](int k, Node& v) {
+    if (k > k_hi) return;
+    v.c = __ldg(g.att4 + k);
+    v.o2 = VAR == 1 ? Or[k] : O2r ? O2r[k] : 0.f;
+    if (VAR == 1 && O2r) v.o2 = v.o2 + O2r[k];
+    if (VAR == 0 && md.use_neb) v.nt = neb_corners(rs, g, k);
+  };
+  Node nx{};
+  load_node(k_lo + tid, nx);
+  cp_async_wait_all();
 #pragma unroll 1
   for (int k = k_lo + tid; k <= k_hi; k += NT) {
-    const float4 c = g.att4[k];
+    const Node v = nx;
+    load_node(k + NT, nx);
+    const float4 c = v.c;
     const float ys = a.lam8 ? rs.y_scale * a.lam8[k] : 1.f;
-    const float o = O2r ? Or[k] + O2r[k] : Or[k];
     float F;
     if constexpr (VAR == 1) {
       float yv[MAX_SEG];
 #pragma unroll
       for (int sg = 0; sg < MAX_SEG; ++sg) yv[sg] = sg < md.n_seg ? Yr[sg * a.seg_stride + k] * ys : 0.f;
-      F = attenuated_bins(md, rs, c, eb, yv, o * ys, g.neb_tab, k);
+      F = attenuated_bins(md, rs, c, eb, yv, v.o2 * ys, g, k);
     } else {
-      F = attenuated(md, rs, c, eb, Yr[k] * ys, o * ys, g, qa, k);
+      const float o = O2r ? Gs[k] + v.o2 : Gs[k];
+      const float nb = !md.use_neb ? 0.f : VAR == 2 ? neb_emission(rs, g, qa, k) : neb_emission(rs, v.nt);
+      F = attenuated(md, rs, c, eb, Ls[k] * ys, o * ys, nb, k);
     }
     if (md.use_igm && c.w < IGM_LYA) {   // the IGM transmission at the node's observed wavelength
       float tau, dtau;
@@ -160,7 +222,8 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
       F *= __expf(-rs.igm_f * tau);
     }
     if (spec) Fs[k] = F;
-    LG[k] = make_float2(c.w, __fdividef(F, c.w * c.w));
+    Ls[k] = c.w;
+    Gs[k] = __fdividef(F, c.w * c.w);
   }
   // emission lines: ln(lam_obs) pairs, fluxes F_l, profile peaks A_l = F_l /
   // (sqrt(2 pi) s_l) and 1/s_l in the tail of the dynamic shared memory
@@ -177,26 +240,47 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
   }
 
   // ---- photometry.  Each sample's bracket starts from the index table over
-  //      ln(lambda) at the sample's rest-frame wavelength and is corrected by a
-  //      walk within the row's window in shared memory (any start gives the same
-  //      bracket, so a fast logarithm serves).
+  //      ln(lambda) at its rest-frame wavelength and is corrected within the
+  //      row's window in shared memory; any start gives the same bracket.
   const float lam0 = g.lam_f[0], lamN = g.lam_f[N - 1];
   const int kmin = k_lo, kmax = k_hi - 1;
-  auto sample_start = [&](float lam_obs) {
-    int q = (int)((__logf(fmaxf(lam_obs * rs.inv1pz, lam0)) - g.lut_x0) * g.lut_inv_h);
-    q = q < 0 ? 0 : (q >= g.lut_n ? g.lut_n - 1 : q);
-    return g.lut[q];
+  // A table cell is half the smallest node spacing wide, and a sample's place in
+  // it carries an error below 8e-6 in ln(lambda) (lg2's 2^-22 of its value,
+  // 2.6e-6, and the roundings of ln lambda, 1/h and the place, 2.1e-6 together): with that
+  // taken off the place, the table's node is the bracket or the one before it as
+  // long as the slack stays below a quarter of a cell.  With every sample inside
+  // the grid (the window then holds all the nodes) such a sample needs no walk and
+  // no clamping but at the grid's end: it tests the next node and takes its
+  // bracket, so that a lane's samples run side by side.  The phase is bound by
+  // the wavefronts of its loads (the samples, the table, two words of each
+  // bracket node), not by arithmetic.
+  const float slack = 8e-6f * g.lut_inv_h;
+  const bool pick = slack <= 0.25f && k_hi - k_lo >= 2 && md.samp_lam_min * rs.inv1pz >= lam0 &&
+                    md.samp_lam_max * rs.inv1pz <= lamN;
+  const float q_mul = 0.6931471805599453f * g.lut_inv_h, q_add = fmaf(-g.lut_x0, g.lut_inv_h, -slack);
+  auto lerp_at = [&](float x, float l0, float l1, float g0, float g1) {
+    const float t = div_approx(x - l0, l1 - l0);
+    return g0 + t * (g1 - g0);
   };
-  // F/lam^2 at the rest-frame wavelength x, from the start k
-  auto sample_value = [&](float x, int k) {
-    int kc = min(max(k, kmin), kmax);
+  // place in the table, and F/lam^2, at the rest-frame wavelength x
+  auto sample_start = [&](float x) { return (int)__ldg(g.lut + (int)fmaf(lg2_approx(x), q_mul, q_add)); };
+  auto sample_pick = [&](float x, int k) {
+    k = min(k, kmax - 1);
+    const float l1 = Ls[k + 1];
+    const bool up = l1 <= x;
+    const float lx = Ls[up ? k + 2 : k];
+    const float* G = Gs + (up ? k + 1 : k);
+    return lerp_at(x, up ? l1 : lx, up ? lx : l1, G[0], G[1]);
+  };
+  auto sample_walk = [&](float x) {
+    if (!(x >= lam0 && x <= lamN)) return 0.f;
+    int kc = g.lut[min(max((int)fmaf(lg2_approx(x), q_mul, q_add), 0), g.lut_n - 1)];
+    kc = min(max(kc, kmin), kmax);
 #pragma unroll 1
-    while (kc < kmax && LG[kc + 1].x <= x) ++kc;
+    while (kc < kmax && Ls[kc + 1] <= x) ++kc;
 #pragma unroll 1
-    while (kc > kmin && LG[kc].x > x) --kc;
-    const float2 p0 = LG[kc], p1 = LG[kc + 1];
-    const float t = __fdividef(x - p0.x, p1.x - p0.x);
-    return p0.y + t * (p1.y - p0.y);
+    while (kc > kmin && Ls[kc] > x) --kc;
+    return lerp_at(x, Ls[kc], Ls[kc + 1], Gs[kc], Gs[kc + 1]);
   };
   // the band's flux from its lanes' sample sums, plus the lines in it (one line
   // per lane); a fixed shuffle tree keeps the order of the sum fixed
@@ -215,43 +299,59 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
       mb_s[b] = mb;
     }
   };
-  float* v_s = reinterpret_cast<float*>(smem4) + a.terms_off;   // NT > EPI_THREADS: the samples' values,
-  float* rn_s = v_s + md.n_samp;                                // then the pixels' residuals
-  if constexpr (NT == EPI_THREADS) {
+  float* rn_s = reinterpret_cast<float*>(smem4) + a.terms_off;   // NT > EPI_THREADS: the pixels' residuals,
+  float* v_s = rn_s + md.n_pix;                                 // NT >= EPI_FLAT: the samples' values
+  if constexpr (NT < EPI_FLAT) {
     // one band per warp: consecutive lanes take consecutive samples (coalesced
-    // loads, eight in flight per lane)
-    for (int b = warp; b < md.n_filt; b += EPI_WARPS) {
-      const int j1 = md.band_start[b + 1];
+    // loads, eight in flight per lane); a sample outside the grid adds zero
+    for (int b = warp; b < md.n_filt; b += NT / 32) {
       float acc = 0.f;
-      for (int j0 = md.band_start[b] + lane; j0 < j1; j0 += 256) {
-        float2 sp[8];   // {lambda_obs, weight}; past the band's end x = 0 < lam0
-        int kg[8];
+      const float2* s2 = md.samp32 + 32 * b32_s[b] + lane;
+      for (int n32 = b32_s[b + 1] - b32_s[b]; n32 > 0; n32 -= 8, s2 += 256) {
+        if (pick) {
+          float2 sp[8];
+          int kg[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) sp[u] = j0 + 32 * u < j1 ? md.samp2[j0 + 32 * u] : make_float2(0.f, 0.f);
+          for (int u = 0; u < 8; ++u)
+            if (u < n32) sp[u] = __ldg(s2 + 32 * u);
 #pragma unroll
-        for (int u = 0; u < 8; ++u) kg[u] = sample_start(sp[u].x);
+          for (int u = 0; u < 8; ++u)
+            if (u < n32) {
+              sp[u].x *= rs.inv1pz;
+              kg[u] = sample_start(sp[u].x);
+            }
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const float x = sp[u].x * rs.inv1pz;
-          if (x >= lam0 && x <= lamN) acc = fmaf(sp[u].y, sample_value(x, kg[u]), acc);
+          for (int u = 0; u < 8; ++u)
+            if (u < n32) acc = fmaf(sp[u].y, sample_pick(sp[u].x, kg[u]), acc);
+        } else {
+#pragma unroll 1
+          for (int u = 0; u < min(n32, 8); ++u) {
+            const float2 sp = __ldg(s2 + 32 * u);
+            acc = fmaf(sp.y, sample_walk(sp.x * rs.inv1pz), acc);
+          }
         }
       }
       band_finish(b, acc);
     }
   } else {
-    for (int j0 = tid; j0 < md.n_samp; j0 += 4 * NT) {
-      float x[4];
-      int kg[4];
+    const int ns = 32 * md.n_samp32;
+    if (pick) {
+      for (int j0 = tid; j0 < ns; j0 += 4 * NT) {
+        float x[4];
+        int kg[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) x[u] = j0 + u * NT < md.n_samp ? md.samp2[j0 + u * NT].x : 0.f;
+        for (int u = 0; u < 4; ++u)
+          if (j0 + u * NT < ns) x[u] = __ldg(&md.samp32[j0 + u * NT].x) * rs.inv1pz;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) kg[u] = sample_start(x[u]);
+        for (int u = 0; u < 4; ++u)
+          if (j0 + u * NT < ns) kg[u] = sample_start(x[u]);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (j0 + u * NT >= md.n_samp) break;
-        const float xr = x[u] * rs.inv1pz;
-        v_s[j0 + u * NT] = xr >= lam0 && xr <= lamN ? sample_value(xr, kg[u]) : 0.f;
+        for (int u = 0; u < 4; ++u)
+          if (j0 + u * NT < ns) v_s[j0 + u * NT] = sample_pick(x[u], kg[u]);
       }
+    } else {
+#pragma unroll 1
+      for (int j = tid; j < ns; j += NT) v_s[j] = sample_walk(__ldg(&md.samp32[j].x) * rs.inv1pz);
     }
   }
 
@@ -327,10 +427,11 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
   }
   if constexpr (NT > EPI_THREADS) {
     __syncthreads();
+    if (NT >= EPI_FLAT)
     for (int b = NT / 32 - 1 - warp; b < md.n_filt; b += NT / 32) {   // the first warps have the pixels' sums below
       float acc = 0.f;
 #pragma unroll 8
-      for (int j = md.band_start[b] + lane; j < md.band_start[b + 1]; j += 32) acc = fmaf(md.samp2[j].y, v_s[j], acc);
+      for (int j = 32 * b32_s[b] + lane; j < 32 * b32_s[b + 1]; j += 32) acc = fmaf(__ldg(&md.samp32[j].y), v_s[j], acc);
       band_finish(b, acc);
     }
     if (tid < EPI_THREADS)
@@ -339,19 +440,22 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
         if (__float_as_uint(t) != EPI_MISSED) add_term(t, i);
       }
   }
-  part += (double)chi;
+  // the first EPI_WARPS warps own the pixels in every instance; without pixels
+  // there is nothing to sum (the FP64 pipe serves the whole SM)
+  const bool own = md.n_pix > 0 && (NT == EPI_THREADS || tid < EPI_THREADS);
+  if (own) part += (double)chi;
   // calibration moments over this thread's own pixels (no barrier needed),
-  // in three blocks of sums (S_0..12, S_13..24, b_0..12), each summed per warp;
-  // the first EPI_WARPS warps own the pixels in every instance
-  const bool own = NT == EPI_THREADS || tid < EPI_THREADS;
+  // in three blocks of sums (S_0..12, S_13..24, b_0..12), each summed per warp
   if (md.calib_n && own) {
     calib_block<0, 0, EPI_THREADS>(md, mu_s, cal_c, tid, lane, warp, &cal_part[0][0]);
     calib_block<SED_MAX_CALIB, 0, EPI_THREADS>(md, mu_s, cal_c, tid, lane, warp, &cal_part[0][0]);
     calib_block<0, 1, EPI_THREADS>(md, mu_s, cal_c, tid, lane, warp, &cal_part[0][0]);
   }
+  if (own) {
 #pragma unroll
-  for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-  if (lane == 0 && own) red[warp] = part;
+    for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+    if (lane == 0) red[warp] = part;
+  }
   __syncthreads();
   if (md.calib_n) {
     // sum the warps' moments in warp order into row 0, factor M and solve for
@@ -386,14 +490,15 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
   if (warp == 0) {
     double pv = 0.0;
     for (int b = lane; b < md.n_filt; b += 32) {
-      if (md.phot_isig[b] != 0.0) {
-        const double is = md.phot_isig[b], mn = (double)mb_s[b] * is, dn = md.phot_d[b] * is;
+      const double is = band_s[b].y;
+      if (is != 0.0) {
+        const double mn = (double)mb_s[b] * is, dn = band_s[b].x * is;
         const double rr = phot_resid(md, b, dn, mn);
         if (md.floor_bits[0]) {   // sigma_eff of Eq. app_noise_floor
           const double q = floor_q(rs.fl[0], mn, dn, (double)rs.fl[0][3] * is);
-          pv += -0.5 * (rr * rr / q + log(q)) + md.phot_nlog[b];
+          pv += -0.5 * (rr * rr / q + log(q)) + band_s[b].z;
         } else {
-          pv += -0.5 * rr * rr + md.phot_nlog[b];
+          pv += -0.5 * rr * rr + band_s[b].z;
         }
       }
     }
@@ -404,7 +509,7 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
     for (int o = 16; o; o >>= 1) pv += __shfl_xor_sync(0xffffffffu, pv, o);
     if (lane == 0) {
       double tot = pv;
-      for (int w = 0; w < EPI_WARPS; ++w) tot += red[w];
+      for (int w = 0; w < EPI_WARPS && md.n_pix > 0; ++w) tot += red[w];
       if (md.calib_n) tot += cal_fix;
       uint32_t st = 0;
       if (!isfinite(tot)) { st = SED_ROW_NONFINITE; tot = -INFINITY; }

@@ -114,6 +114,38 @@ sed_status ensure_f8_layout(sed_ctx* ctx, Grid* g, Layout* L);
 }  // namespace
 
 namespace sed {
+__global__ void k_neb4(const float* __restrict__ tab, int nu, int nz, int nl, float4* __restrict__ out) {
+  const int cz = max(nz - 1, 1), cell = blockIdx.y, u = cell / cz, z = cell - u * cz;
+  const int u1 = min(u + 1, nu - 1), z1 = min(z + 1, nz - 1);
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nl; k += gridDim.x * blockDim.x)
+    out[(size_t)cell * nl + k] = make_float4(tab[(size_t)(u * nz + z) * nl + k], tab[(size_t)(u * nz + z1) * nl + k],
+                                             tab[(size_t)(u1 * nz + z) * nl + k], tab[(size_t)(u1 * nz + z1) * nl + k]);
+}
+void ensure_neb4(sed_ctx* ctx, Grid* g, cudaStream_t s) {
+  if (g->neb4_tried.load(std::memory_order_acquire) || !g->dv.neb_tab || g->neb_na > 0) return;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return;
+  }
+  std::lock_guard<std::mutex> lk(ctx->mu);
+  if (g->neb4_tried.load(std::memory_order_relaxed)) return;
+  const int cells = std::max(g->neb_nu - 1, 1) * std::max(g->neb_nz - 1, 1);
+  const size_t bytes = (size_t)cells * g->n_lam * sizeof(float4);
+  if (bytes <= NEB4_MAX_BYTES && (!ctx->budget || ctx->used.load() + 8 * bytes <= ctx->budget)) {
+    const std::string kept = ctx->last_error;
+    float4* p = nullptr;
+    if (dalloc(ctx, (void**)&p, bytes, &g->allocs, &g->bytes) == SED_OK) {
+      k_neb4<<<dim3((g->n_lam + 255) / 256, cells), 256, 0, s>>>(g->dv.neb_tab, g->neb_nu, g->neb_nz, g->n_lam, p);
+      // other streams may read it as soon as it is published
+      if (cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(s) == cudaSuccess)
+        g->neb4.store(p, std::memory_order_release);
+    } else {
+      ctx->last_error = kept;
+    }
+  }
+  g->neb4_tried.store(true, std::memory_order_release);
+}
 sed_status ensure_f8_layout_shared(sed_ctx* ctx, Grid* g, Layout* L) { return ensure_f8_layout(ctx, g, L); }
 }  // namespace sed
 
@@ -338,13 +370,13 @@ sed_status sed_load_grid(sed_ctx* ctx, const sed_grid_desc* d, sed_grid_id* out)
     delete g;
     return fail(ctx, SED_ERANGE, "wavelength axis too unevenly spaced for the index table");
   }
-  std::vector<int> lut(lut_n);
+  std::vector<uint16_t> lut(lut_n);
   {
     size_t k = 0;
     for (int q = 0; q < lut_n; q++) {
       const double xq = x0 + q * h;
       while (k + 1 < nl && (double)lh[k + 1] <= xq) k++;
-      lut[q] = (int)k;
+      lut[q] = (uint16_t)k;
     }
   }
   // linear-time Voronoi cells (App. B step scheme)
@@ -363,13 +395,13 @@ sed_status sed_load_grid(sed_ctx* ctx, const sed_grid_desc* d, sed_grid_id* out)
   GridDev& dv = g->dv;
   dv.n_age = g->n_age; dv.n_feh = g->n_feh; dv.n_afe = g->n_afe; dv.n_lam = g->n_lam;
   float* p;
-  int* pi;
+  uint16_t* pu;
 #define UPF(field, vec)                                                   \
   if (!st) { st = upload(ctx, &p, vec.data(), vec.size(), &g->allocs, &g->bytes); dv.field = p; }
   UPF(lam_f, lam_f) UPF(inv_lam2, inv_lam2) UPF(inv_dlam, idl) UPF(lnp, lnp) UPF(kprime, kp) UPF(drude, dr)
   UPF(lnl_hi, lh) UPF(lnl_lo, lo) UPF(cell_lo, clo) UPF(cell_hi, chi) UPF(age_t, at) UPF(age_dl, adl)
 #undef UPF
-  if (!st) { st = upload(ctx, &pi, lut.data(), lut.size(), &g->allocs, &g->bytes); dv.lut = pi; }
+  if (!st) { st = upload(ctx, &pu, lut.data(), lut.size(), &g->allocs, &g->bytes); dv.lut = pu; }
   if (!st) {
     std::vector<float4> a4(nl);
     for (size_t k = 0; k < nl; k++)
@@ -1065,6 +1097,20 @@ sed_status sed_create_model(sed_ctx* ctx, const sed_model_desc* d, sed_model_id*
     for (int j = 0; j < S; j++) s2[j] = make_float2(sl[j], sw[j]);
     float2* p2;
     if (!st) { st = upload(ctx, &p2, s2.data(), s2.size(), &M->allocs, &M->bytes); dv.samp2 = p2; }
+    if (!st) {   // the samples in whole warps per band
+      std::vector<int> b32(d->n_filt + 1, 0);
+      for (int b = 0; b < d->n_filt; b++) b32[b + 1] = b32[b] + (bs[b + 1] - bs[b] + 31) / 32;
+      std::vector<float2> sp((size_t)b32[d->n_filt] * 32);
+      for (int b = 0; b < d->n_filt; b++)
+        for (int q = 32 * b32[b]; q < 32 * b32[b + 1]; q++) {
+          const int j = bs[b] + q - 32 * b32[b], jj = std::min(j, bs[b + 1] - 1);
+          sp[q] = make_float2(sl[jj], j == jj ? sw[jj] : 0.f);
+        }
+      st = upload(ctx, &p2, sp.data(), sp.size(), &M->allocs, &M->bytes);
+      dv.samp32 = p2;
+      if (!st) { st = upload(ctx, &pi, b32.data(), b32.size(), &M->allocs, &M->bytes); dv.band32 = pi; }
+      dv.n_samp32 = b32[d->n_filt];
+    }
     if (!st && d->use_lines) {   // a line's photometry: R / Z_b at the samples
       float* pr;
       st = upload(ctx, &pr, srz.data(), srz.size(), &M->allocs, &M->bytes);
@@ -1361,6 +1407,7 @@ sed_status run_forward_core(sed_ctx* ctx, Model* M, Workspace* w, const float* t
     w->have_stats = true;
     w->last_grad = false;
   }
+  if (M->dv.use_neb) ensure_neb4(ctx, g, s);
   if (sed_status ps = prof_mark(ctx, w, 0, s)) return ps;
   PrepArgs pa{};
   pa.theta = theta; pa.n = n; pa.ld = ld;
@@ -1478,7 +1525,7 @@ sed_status sed_forward(sed_ctx* ctx, sed_model_id id, const float* theta, int n,
   EpiArgs ea{};
   ea.n = n; ea.ldn = w->ldn; ea.Y = w->Y; ea.O = w->O; ea.rs = w->rs;
   ea.O2 = w->O2; ea.split = precision == SED_PREC_FP32 ? w->err + 8 : nullptr;   // the 3xTF32 launch's split choice
-  ea.md = M->dv; ea.g = M->g->dv;
+  ea.md = M->dv; ea.g = grid_view(M->g);
   ea.seg_stride = (size_t)w->cap_rows * w->ldn;
   ea.qneb = M->dv.use_neb && M->g->neb_na > 0 ? w->qneb : nullptr;
   ea.win_reset = w->tile_win; ea.win_mt = (n + 127) / 128;   // read by the contraction, emptied for the next call
@@ -1508,7 +1555,7 @@ sed_status sed_line_fluxes(sed_ctx* ctx, sed_model_id id, const float* theta, in
   EpiArgs ea{};
   ea.n = n; ea.ldn = w->ldn; ea.Y = w->Y; ea.O = w->O; ea.rs = w->rs;
   ea.O2 = w->O2; ea.split = precision == SED_PREC_FP32 ? w->err + 8 : nullptr;   // the 3xTF32 launch's split choice
-  ea.md = M->dv; ea.g = M->g->dv;
+  ea.md = M->dv; ea.g = grid_view(M->g);
   ea.seg_stride = (size_t)w->cap_rows * w->ldn;
   ea.qneb = M->dv.use_neb && M->g->neb_na > 0 ? w->qneb : nullptr;
   ea.win_reset = w->tile_win; ea.win_mt = (n + 127) / 128;   // read by the contraction, emptied for the next call
@@ -1537,7 +1584,7 @@ static sed_status loglike_impl(sed_ctx* ctx, sed_model_id id, const float* theta
   EpiArgs ea{};
   ea.n = n; ea.ldn = w->ldn; ea.Y = w->Y; ea.O = w->O; ea.rs = w->rs;
   ea.O2 = w->O2; ea.split = precision == SED_PREC_FP32 ? w->err + 8 : nullptr;   // the 3xTF32 launch's split choice
-  ea.md = M->dv; ea.g = M->g->dv;
+  ea.md = M->dv; ea.g = grid_view(M->g);
   ea.seg_stride = (size_t)w->cap_rows * w->ldn;
   ea.qneb = M->dv.use_neb && M->g->neb_na > 0 ? w->qneb : nullptr;
   ea.win_reset = w->tile_win; ea.win_mt = (n + 127) / 128;   // read by the contraction, emptied for the next call
@@ -1656,7 +1703,7 @@ sed_status sed_loglike_grad(sed_ctx* ctx, sed_model_id id, const float* theta, i
   EpiBwdArgs eb{};
   eb.n = n; eb.ldn = w->ldn; eb.Y = w->Y; eb.O = w->O; eb.rs = w->rs;
   eb.O2 = w->O2; eb.o2_split = precision == SED_PREC_FP32 ? w->err + 8 : nullptr;
-  eb.md = M->dv; eb.g = g->dv; eb.split = f32 ? 1 : 0;
+  eb.md = M->dv; eb.g = grid_view(g); eb.split = f32 ? 1 : 0;
   eb.gy_hi = w->G_hi; eb.gy_lo = w->G_lo; eb.go_hi = w->GO_hi; eb.go_lo = w->GO_lo;
   eb.rgrad = w->rgrad; eb.lnl = lnl_out; eb.status = row_status; eb.err = w->err;
   eb.seg_stride = (size_t)w->cap_rows * w->ldn;

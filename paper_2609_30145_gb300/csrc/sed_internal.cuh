@@ -36,6 +36,7 @@ constexpr int KMASK_WORDS = 8;
 constexpr int MAX_LINES = 128;   // emission lines of a nebular grid
 constexpr int MAX_DUST_BIN = SED_MAX_DUST_BIN;   // age-binned attenuation laws
 constexpr int MAX_SEG = SED_MAX_DUST_SEG;        // attenuated K blocks (runs of ages with one non-zero row of M)
+constexpr size_t NEB4_MAX_BYTES = (size_t)64 << 20;   // largest table of nebular template corners (GridDev::neb4)
 constexpr int MAX_NEB_AGE = 32;  // SSP ages a nebular age axis spans
 
 // Physical constants (cgs unless noted).
@@ -63,6 +64,7 @@ struct RowScal {
   float log2_qy;    // log2(Q_young, device units) (-inf when Q_young = 0)
   float neb_w[4];   // bilinear weights of the nebular template corners
   int neb_off[4];   // corner offsets (rows of the template)
+  int neb_cell;     // offset of the cell's row of corners (GridDev::neb4)
   float neb_dwu[4]; // d neb_w / d gas_logu (adjoint)
   float neb_dwz[4]; // d neb_w / d gas_logz (adjoint)
   float dlnp_dz;    // d ln(p_phot)/dz (adjoint)
@@ -107,7 +109,7 @@ struct GridDev {
   const float* drude;      // Drude profile with E_b = 1
   const float* lnl_hi;     // ln(lambda) split in two floats
   const float* lnl_lo;
-  const int* lut;          // lut[q] = last node with ln(lambda) <= x0 + q/inv_h
+  const uint16_t* lut;     // lut[q] = last node with ln(lambda) <= x0 + q/inv_h (n_lam <= MAX_LAM < 2^16)
   int lut_n;
   float lut_x0, lut_inv_h;
   float dln_max;           // largest ln(lambda[k+1] / lambda[k])
@@ -117,6 +119,9 @@ struct GridDev {
   const float* age_dl;     // ln(t_{a+1} / t_a) (last entry unused)
   const float* neb_tab;    // [nu][nz][n_lam] log10 template + device-unit offset; with an age axis
                            // [neb_na][nu][nz][n_lam], plane i the cube at SSP age neb_a0 + i
+  const float4* neb4;      // the template's four corners {(u,z), (u,z+1), (u+1,z), (u+1,z+1)} of each cell of its
+                           // axes, [cells in u][cells in z][n_lam]: a node's corners in one load.  NULL in a grid's
+                           // own view (grid_view() fills it in); where it is NULL neb_tab is read instead
   int neb_nu, neb_nz;
   int neb_a0, neb_na;      // nebular age axis: the SSP ages [neb_a0, neb_a0 + neb_na) (neb_na = 0: none)
   // emission-line cube: per line {ln(lam/5500), k'/4.05, Drude/4.05, lam},
@@ -159,6 +164,11 @@ struct ModelDev {
   int n_filt, n_samp;
   const int* band_start;   // [n_filt + 1]
   const float2* samp2;     // [n_samp] {observed-frame lambda (A), weight R lam dlam / Z_b}
+  // the samples as the forward epilogue reads them: samp2 with each band padded to whole warps by its
+  // last sample at weight 0; band b's are [32 band32[b], 32 band32[b+1])
+  const float2* samp32;
+  const int* band32;       // [n_filt + 1]
+  int n_samp32;            // padded samples / 32
   const double* phot_d;    // [n_filt]
   const double* phot_isig; // [n_filt] 1/sigma (0 when masked out)
   const double* phot_nlog; // [n_filt] -1/2 ln(2 pi sigma^2) (0 when masked out)
@@ -285,6 +295,8 @@ struct Grid {
   GridDev dv{};
   int neb_nu = 0, neb_nz = 0;
   int neb_a0 = 0, neb_na = 0;  // nebular age axis: the SSP ages it spans (neb_na = 0: none)
+  std::atomic<const float4*> neb4{nullptr};   // GridDev::neb4, built by the first call that reads it
+  std::atomic<bool> neb4_tried{false};
   std::vector<double> neb_logu, neb_logz;
   std::vector<Layout*> layouts;
   std::vector<void*> allocs;
@@ -500,8 +512,11 @@ __device__ __forceinline__ void ln_rest(float2 p, float z_hi, float z_lo, float&
 // those of plain stream order.  Under stream capture the attribute is left off:
 // a graph replay already launches back to back, and measured slower with it.
 // Without the attribute the wait returns at once.
+// What a kernel does before the wait touches only the model's and the grid's
+// constant tables, which no kernel writes.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_enter() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_wait();
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
@@ -632,8 +647,8 @@ struct EpiArgs {
   const RowScal* rs;
   ModelDev md; GridDev g;
   const ModelDev* mtab;    // as in PrepArgs; with row_model set, smem_samp / smem_pix give the
-  const int* row_model;    // largest n_samp / n_pix of the launch's models
-  int smem_samp, smem_pix, smem_win;
+  const int* row_model;    // largest n_samp32 / n_pix of the launch's models
+  int smem_samp, smem_pix, smem_win;   // samples in units of 32
   float* phot_out; float* spec_out;
   float* lines_out;    // [n][n_line] observer-frame line fluxes (erg/s/cm^2), or NULL
   double* lnl; uint32_t* status;
@@ -689,6 +704,17 @@ struct PrepBwdArgs {
   float* grad;          // [n][ld]
 };
 cudaError_t launch_prep_bwd(const PrepBwdArgs& a, cudaStream_t s);
+
+// The table of nebular template corners (GridDev::neb4), built on the first call
+// of a model with nebular emission: kept to NEB4_MAX_BYTES, left out for an age
+// axis, under stream capture, or where memory or the budget is short (a call
+// then reads neb_tab; the results are the same).
+void ensure_neb4(sed_ctx* ctx, Grid* g, cudaStream_t s);
+inline GridDev grid_view(const Grid* g) {
+  GridDev d = g->dv;
+  d.neb4 = g->neb4.load(std::memory_order_acquire);
+  return d;
+}
 
 // Build the FP8 copy of a layout (caller holds ctx->mu).
 sed_status ensure_f8_layout_shared(sed_ctx* ctx, Grid* g, Layout* L);
