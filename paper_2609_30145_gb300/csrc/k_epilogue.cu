@@ -56,10 +56,11 @@ constexpr int MAX_BANDS = 128;
 // of the paper-scale photometric fit: epilogue stage 28.7 -> 16.4 us, step 54.1 ->
 // 37.7 us; 301 rows with a 1111-pixel spectrum: 59.4 -> 28.7 us).  Every sum keeps the
 // 128-thread instance's terms and order, so a row's result does not depend on
-// the instance that computed it: the samples' interpolated values and the
-// pixels' residuals go through shared memory, and the sums over them run as
-// lanes of a warp per band and as EPI_THREADS threads over the pixels.
-// EPI_MISSED marks an excluded pixel there (a NaN no arithmetic produces).
+// the instance that computed it: the samples' interpolated values go through
+// shared memory where they are spread over all threads, the pixels' residuals
+// always do, and the sums over them run as lanes of a warp per band and as
+// EPI_THREADS threads over the pixels.  EPI_MISSED marks an excluded pixel there
+// (a NaN no arithmetic produces).
 constexpr uint32_t EPI_MISSED = 0x7fa00001u;
 // From this many threads on, a band's samples are spread over all of them; below
 // it a warp takes a band (no shared memory for the samples' values, which would
@@ -68,8 +69,8 @@ constexpr int EPI_FLAT = 512;
 
 // dynamic shared memory: lam, F/lam^2 and F over the row's window, the
 // included pixels' mu/sigma for the calibration moments, with emission lines,
-// per line ln(lam_obs) (an FP32 pair), F_l, A_l and 1/s_l, and, with more than
-// EPI_THREADS threads, the samples' values and the pixels' residuals
+// per line ln(lam_obs) (an FP32 pair), F_l, A_l and 1/s_l, the pixels' residuals
+// and, from EPI_FLAT threads on, the samples' values
 size_t epilogue_lines_off(const EpiArgs& a) {   // in floats, even (float2 alignment)
   const int np = a.row_model ? a.smem_pix : a.md.n_pix;
   const size_t W = (size_t)(a.row_model ? a.smem_win : a.md.win_max);
@@ -77,14 +78,19 @@ size_t epilogue_lines_off(const EpiArgs& a) {   // in floats, even (float2 align
   const size_t f = 2 * W + (np > 0 ? W : 0) + (calib ? (size_t)np : 0);
   return (f + 1) & ~(size_t)1;
 }
-size_t epilogue_terms_off(const EpiArgs& a) {   // in floats
+size_t epilogue_samp_off(const EpiArgs& a) {   // in floats
   const bool lines = a.row_model ? a.g.n_line > 0 : a.md.use_lines != 0;
   return epilogue_lines_off(a) + (lines ? (size_t)5 * a.g.n_line : 0);
 }
+// the pixels' residuals: over lam and F/lam^2, which the spectrum does not read,
+// where they fit there
+bool epilogue_res_alias(const EpiArgs& a) {
+  return (a.row_model ? a.smem_pix : a.md.n_pix) <= 2 * (a.row_model ? a.smem_win : a.md.win_max);
+}
 size_t epilogue_smem(const EpiArgs& a, int nt) {
-  const size_t pix = a.row_model ? a.smem_pix : a.md.n_pix;
+  const size_t pix = epilogue_res_alias(a) ? 0 : (size_t)(a.row_model ? a.smem_pix : a.md.n_pix);
   const size_t samp = 32 * (size_t)(a.row_model ? a.smem_samp : a.md.n_samp32);
-  return (epilogue_terms_off(a) + (nt > EPI_THREADS ? pix : 0) + (nt >= EPI_FLAT ? samp : 0)) * sizeof(float);
+  return (epilogue_samp_off(a) + pix + (nt >= EPI_FLAT ? samp : 0)) * sizeof(float);
 }
 
 // a / b by the hardware's reciprocal, subnormals as zero (a and b here are
@@ -99,6 +105,12 @@ __device__ __forceinline__ float lg2_approx(float x) {
   float y;
   asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
+}
+// e^(-u^2/2) (2^x by the hardware; used for u^2 <= 25, far from the subnormals)
+__device__ __forceinline__ float gauss_w(float u2) {
+  float w;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(w) : "f"(u2 * (-0.5f * 1.4426950408889634f)));
+  return w;
 }
 // four bytes of global memory to shared memory without a register (the thread
 // itself reads them after cp_async_wait_all)
@@ -299,8 +311,8 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
       mb_s[b] = mb;
     }
   };
-  float* rn_s = reinterpret_cast<float*>(smem4) + a.terms_off;   // NT > EPI_THREADS: the pixels' residuals,
-  float* v_s = rn_s + md.n_pix;                                 // NT >= EPI_FLAT: the samples' values
+  float* rn_s = reinterpret_cast<float*>(smem4) + a.res_off;    // the pixels' residuals
+  float* v_s = reinterpret_cast<float*>(smem4) + a.samp_off;    // NT >= EPI_FLAT: the samples' values
   if constexpr (NT < EPI_FLAT) {
     // one band per warp: consecutive lanes take consecutive samples (coalesced
     // loads, eight in flight per lane); a sample outside the grid adds zero
@@ -355,97 +367,127 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
     }
   }
 
-  // ---- spectrum: one thread per pixel
-  // per-pixel terms in FP32 on the normalised residual (d - mu)/sigma; the
-  // constants -1/2 ln(2 pi sigma^2) in FP64
-  double part = 0.0;
-  float chi = 0.f;
-  const float ll0 = g.lnl_hi[0], llN = g.lnl_hi[N - 1];
-  // an included pixel's term of the running sum: the residual squared, or twice
-  // minus the term with the noise floor (sigma_eff of Eq. app_noise_floor)
-  auto add_term = [&](float t, int i) {
-    if (md.floor_bits[1]) chi -= 0.5f * t;
-    else chi = fmaf(-0.5f * t, t, chi);
-    part += md.spec_nlog[i];
-  };
-  for (int i = tid; i < md.n_pix; i += NT) {
-    float xh, xl;
-    ln_rest(md.pix_ln2[i], rs.ln1pz_hi, rs.ln1pz_lo, xh, xl);
-    float v = 0.f;
-    bool valid = false;
-    if (xh >= ll0 && xh <= llN) {
-      // total dispersion: fixed, or sigma_fix composed with the row's sigma_gal (Eq. one_kernel)
-      const float s = md.sample_sgal ? sqrtf(md.pix_fix2[i] + rs.sg_ln * rs.sg_ln) : md.pix_s[i];
-      const int k = locate_ln(g, xh, g.lnl_hi);
-      const float dln = (g.lnl_hi[k + 1] - g.lnl_hi[k]) + (g.lnl_lo[k + 1] - g.lnl_lo[k]);
-      if (s < 0.5f * dln) {
-        const float t = ((xh - g.lnl_hi[k]) + (xl - g.lnl_lo[k])) / dln;
-        v = Fs[k] + t * (Fs[k + 1] - Fs[k]);
-        valid = true;
-      } else {
-        // the nodes within 5 dispersions: a superset of them from the index
-        // table alone (each entry within one node of the exact bracket; the
-        // margins cover that), clamped to the row's window, which holds every
-        // node within 5 dispersions of a pixel; a node past 5 dispersions
-        // weighs exactly 0, so the sums are those over the nodes inside, in
-        // the same order, and the loop carries no branch (its loads pipeline)
-        const float inv_s = 1.f / s;
-        int qa = (int)((fmaxf(xh - 5.f * s, ll0) - g.lut_x0) * g.lut_inv_h);
-        int qb = (int)((fminf(xh + 5.f * s, llN) - g.lut_x0) * g.lut_inv_h);
-        qa = min(max(qa, 0), g.lut_n - 1);
-        qb = min(max(qb, 0), g.lut_n - 1);
-        const int jlo = max(g.lut[qa] - 1, k_lo), jhi = min(g.lut[qb] + 3, k_hi);
-        float sw = 0.f, sf = 0.f;
-#pragma unroll 4
-        for (int j = jlo; j <= jhi; ++j) {
-          const float d = (g.lnl_hi[j] - xh) + (g.lnl_lo[j] - xl);
-          const float u = d * inv_s;
-          const float w = fabsf(u) <= 5.f ? __expf(-0.5f * u * u) : 0.f;
-          sw += w;
-          sf = fmaf(w, Fs[j], sf);
-        }
-        if (sw > 0.f) { v = sf / sw; valid = true; }
-      }
-    }
-    const float mi = LINES && NLn ? fmaf(rs.s_spec, v, lines_at_pixel(md, i, NLn, ln_A, ln_is, ln_x)) : rs.s_spec * v;
-    if (a.spec_out) a.spec_out[(size_t)ro * md.n_pix + i] = mi;
-    const float isf = md.spec_isf[i];
-    const bool inc = valid && isf != 0.f;
-    const float ms = inc ? mi * isf : 0.f;   // mu / sigma
-    const float dn = md.spec_dn[i];
-    float t = dn - ms;                       // (d - mu) / sigma
-    if (inc && md.floor_bits[1]) {
-      const float q = floor_q(rs.fl[1], ms, dn, rs.fl[1][3] * isf);
-      t = t * t / q + logf(q);
-    }
-    if constexpr (NT == EPI_THREADS) {
-      if (inc) add_term(t, i);
-    } else {
-      rn_s[i] = inc ? t : __uint_as_float(EPI_MISSED);
-    }
-    if (md.calib_n) mu_s[i] = ms;
-  }
-  if constexpr (NT > EPI_THREADS) {
+  if constexpr (NT >= EPI_FLAT) {
     __syncthreads();
-    if (NT >= EPI_FLAT)
-    for (int b = NT / 32 - 1 - warp; b < md.n_filt; b += NT / 32) {   // the first warps have the pixels' sums below
+    for (int b = warp; b < md.n_filt; b += NT / 32) {
       float acc = 0.f;
 #pragma unroll 8
       for (int j = 32 * b32_s[b] + lane; j < 32 * b32_s[b + 1]; j += 32) acc = fmaf(__ldg(&md.samp32[j].y), v_s[j], acc);
       band_finish(b, acc);
     }
-    if (tid < EPI_THREADS)
+  }
+
+  // ---- spectrum: two neighbouring pixels per thread, which share most of their
+  //      nodes, so that a node's position and flux are loaded once for both.  (The
+  //      loop over the nodes is bound by instruction issue: 12.5 per pixel and
+  //      node against 23 with one pixel per thread.  Epilogue stage of 1024 rows of
+  //      1500 pixels with 30 lines 104.5 -> 79.9 us, of 512 calibrated rows 65.5 ->
+  //      53.2 us.)  Per-pixel terms in FP32 on
+  //      the normalised residual (d - mu)/sigma; the constants
+  //      -1/2 ln(2 pi sigma^2) in FP64.
+  double part = 0.0;
+  float chi = 0.f;
+  if (md.n_pix > 0) {
+    if (a.res_off < 2 * WIN) __syncthreads();   // the residuals go over lam and F/lam^2
+    const float ll0 = g.lnl_hi[0], llN = g.lnl_hi[N - 1];
+    const int last = md.n_pix - 1;
+    for (int ib = 2 * 32 * warp; ib < md.n_pix; ib += 2 * NT) {
+      float2 pl[2];
+      float v[2], xh[2], xl[2], inv_s[2], sw[2] = {0.f, 0.f}, sf[2] = {0.f, 0.f};
+      bool gauss[2], valid[2];
+      int jl = k_hi, jh = k_lo - 1;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int i = min(ib + 2 * lane + q, last);
+        pl[q] = md.pix_ln2[i];
+        ln_rest(pl[q], rs.ln1pz_hi, rs.ln1pz_lo, xh[q], xl[q]);
+        v[q] = 0.f;
+        valid[q] = gauss[q] = false;
+        inv_s[q] = 0.f;
+        if (xh[q] >= ll0 && xh[q] <= llN) {
+          // total dispersion: fixed, or sigma_fix composed with the row's sigma_gal (Eq. one_kernel)
+          const float s = md.sample_sgal ? sqrtf(md.pix_fix2[i] + rs.sg_ln * rs.sg_ln) : md.pix_s[i];
+          const int k = locate_ln(g, xh[q], g.lnl_hi);
+          const float2 n0 = __ldg(g.lnl2 + k), n1 = __ldg(g.lnl2 + k + 1);
+          const float dln = (n1.x - n0.x) + (n1.y - n0.y);
+          if (s < 0.5f * dln) {
+            const float t = ((xh[q] - n0.x) + (xl[q] - n0.y)) / dln;
+            v[q] = Fs[k] + t * (Fs[k + 1] - Fs[k]);
+            valid[q] = true;
+          } else {
+            // the nodes within 5 dispersions: a superset of them from the index
+            // table alone (each entry within one node of the exact bracket; the
+            // margins cover that), clamped to the row's window, which holds every
+            // node within 5 dispersions of a pixel; a node past 5 dispersions is
+            // left out by predication, so the loop carries no branch (its loads
+            // pipeline)
+            gauss[q] = true;
+            inv_s[q] = 1.f / s;
+            int qa = (int)((fmaxf(xh[q] - 5.f * s, ll0) - g.lut_x0) * g.lut_inv_h);
+            int qb = (int)((fminf(xh[q] + 5.f * s, llN) - g.lut_x0) * g.lut_inv_h);
+            qa = min(max(qa, 0), g.lut_n - 1);
+            qb = min(max(qb, 0), g.lut_n - 1);
+            jl = min(jl, max(g.lut[qa] - 1, k_lo));
+            jh = max(jh, min(g.lut[qb] + 3, k_hi));
+          }
+        }
+      }
+#pragma unroll 4
+      for (int j = jl; j <= jh; ++j) {
+        const float2 n = __ldg(g.lnl2 + j);
+        const float f = Fs[j];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const float u = ((n.x - xh[q]) + (n.y - xl[q])) * inv_s[q];
+          const float u2 = u * u, w = gauss_w(u2);
+          if (u2 <= 25.f) {   // predicated: a node past 5 dispersions is left out
+            sw[q] += w;
+            sf[q] = fmaf(w, f, sf[q]);
+          }
+        }
+      }
+      float la[2] = {0.f, 0.f};
+      if (LINES && NLn)
+        lines_at_pixels(NLn, ln_A, ln_is, ln_x, pl[0], pl[1], __shfl_sync(0xffffffffu, pl[0].x, 0),
+                        __shfl_sync(0xffffffffu, pl[1].x, 31), lane, la[0], la[1]);
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int i = ib + 2 * lane + q;
+        if (i > last) break;
+        if (gauss[q] && sw[q] > 0.f) { v[q] = sf[q] / sw[q]; valid[q] = true; }
+        const float mi = LINES && NLn ? fmaf(rs.s_spec, v[q], la[q] * md.pix_lamc[i]) : rs.s_spec * v[q];
+        if (a.spec_out) a.spec_out[(size_t)ro * md.n_pix + i] = mi;
+        const float isf = md.spec_isf[i];
+        const bool inc = valid[q] && isf != 0.f;
+        const float ms = inc ? mi * isf : 0.f;   // mu / sigma
+        const float dn = md.spec_dn[i];
+        float t = dn - ms;                       // (d - mu) / sigma
+        if (inc && md.floor_bits[1]) {           // sigma_eff of Eq. app_noise_floor
+          const float qf = floor_q(rs.fl[1], ms, dn, rs.fl[1][3] * isf);
+          t = t * t / qf + logf(qf);
+        }
+        rn_s[i] = inc ? t : __uint_as_float(EPI_MISSED);
+        if (md.calib_n) mu_s[i] = ms;
+      }
+    }
+    __syncthreads();
+    if (NT == EPI_THREADS || tid < EPI_THREADS)
       for (int i = tid; i < md.n_pix; i += EPI_THREADS) {
+        // an included pixel's term: the residual squared, or twice minus the term
+        // with the noise floor
         const float t = rn_s[i];
-        if (__float_as_uint(t) != EPI_MISSED) add_term(t, i);
+        if (__float_as_uint(t) == EPI_MISSED) continue;
+        if (md.floor_bits[1]) chi -= 0.5f * t;
+        else chi = fmaf(-0.5f * t, t, chi);
+        part += md.spec_nlog[i];
       }
   }
   // the first EPI_WARPS warps own the pixels in every instance; without pixels
   // there is nothing to sum (the FP64 pipe serves the whole SM)
   const bool own = md.n_pix > 0 && (NT == EPI_THREADS || tid < EPI_THREADS);
   if (own) part += (double)chi;
-  // calibration moments over this thread's own pixels (no barrier needed),
-  // in three blocks of sums (S_0..12, S_13..24, b_0..12), each summed per warp
+  // calibration moments over each thread's pixels in three blocks of sums
+  // (S_0..12, S_13..24, b_0..12), each summed per warp
   if (md.calib_n && own) {
     calib_block<0, 0, EPI_THREADS>(md, mu_s, cal_c, tid, lane, warp, &cal_part[0][0]);
     calib_block<SED_MAX_CALIB, 0, EPI_THREADS>(md, mu_s, cal_c, tid, lane, warp, &cal_part[0][0]);
@@ -520,8 +562,9 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
 }
 
 template <int NT>
-cudaError_t launch_epilogue_nt(const EpiArgs& a, cudaStream_t s) {
+cudaError_t launch_epilogue_nt(EpiArgs a, cudaStream_t s) {
   const size_t smem = epilogue_smem(a, NT);
+  if (!epilogue_res_alias(a)) a.res_off = a.samp_off + (NT >= EPI_FLAT ? 32 * (a.row_model ? a.smem_samp : a.md.n_samp32) : 0);
   static DynSmemCache set_for[6];
   const bool lines = a.row_model ? a.g.n_line > 0 : a.md.use_lines != 0;
   // age-binned dust and the nebular age axis: neither served nor with lines
@@ -540,7 +583,8 @@ cudaError_t launch_epilogue_nt(const EpiArgs& a, cudaStream_t s) {
 cudaError_t launch_epilogue(const EpiArgs& a_in, cudaStream_t s) {
   EpiArgs a = a_in;
   a.lines_off = (int)epilogue_lines_off(a);
-  a.terms_off = (int)epilogue_terms_off(a);
+  a.samp_off = (int)epilogue_samp_off(a);
+  a.res_off = 0;
   // Threads per row: as many as keep every row of the launch resident at once
   // (1024 threads per SM at 64 registers), where their shared memory fits.
   const int sm = device_sm_count();

@@ -90,6 +90,31 @@ __device__ __forceinline__ float lines_at_pixel(const ModelDev& md, int i, int N
   return acc * md.pix_lamc[i];
 }
 
+// The same sum for a warp's two pixels per lane (ln(lambda) in p0, p1; the
+// warp's pixels ascend from xmin to xmax): most lines reach none of them, so
+// each lane first tests one line against the warp's range, and only the lines
+// found are gone through, in index order.
+__device__ __forceinline__ void lines_at_pixels(int NLn, const float* A_s, const float* is_s, const float2* x_s,
+                                                float2 p0, float2 p1, float xmin, float xmax, int lane, float& a0,
+                                                float& a1) {
+  a0 = a1 = 0.f;
+  for (int l0 = 0; l0 < NLn; l0 += 32) {
+    bool near = false;
+    if (l0 + lane < NLn && is_s[l0 + lane] > 0.f) {   // a line without width has no profile (A_l = 0)
+      const float x = x_s[l0 + lane].x, reach = 5.01f / is_s[l0 + lane] + 1e-5f;
+      near = x + reach >= xmin && x - reach <= xmax;
+    }
+    for (unsigned m = __ballot_sync(0xffffffffu, near); m; m &= m - 1) {
+      const int l = l0 + __ffs(m) - 1;
+      const float2 x = x_s[l];
+      const float is = is_s[l], A = A_s[l];
+      const float u0 = ((p0.x - x.x) + (p0.y - x.y)) * is, u1 = ((p1.x - x.x) + (p1.y - x.y)) * is;
+      if (fabsf(u0) <= 5.f) a0 = fmaf(A, __expf(-0.5f * u0 * u0), a0);
+      if (fabsf(u1) <= 5.f) a1 = fmaf(A, __expf(-0.5f * u1 * u1), a1);
+    }
+  }
+}
+
 // Band b's response to a line at observed wavelength x: rz = R_b(x) / Z_b, R_b
 // linear between the band's samples (0 outside them), and its slope drz in x.
 // The bracket (the last sample at or below x; the last interval at the band's

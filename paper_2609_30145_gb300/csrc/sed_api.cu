@@ -401,6 +401,13 @@ sed_status sed_load_grid(sed_ctx* ctx, const sed_grid_desc* d, sed_grid_id* out)
   UPF(lam_f, lam_f) UPF(inv_lam2, inv_lam2) UPF(inv_dlam, idl) UPF(lnp, lnp) UPF(kprime, kp) UPF(drude, dr)
   UPF(lnl_hi, lh) UPF(lnl_lo, lo) UPF(cell_lo, clo) UPF(cell_hi, chi) UPF(age_t, at) UPF(age_dl, adl)
 #undef UPF
+  if (!st) {
+    std::vector<float2> l2(nl);
+    for (size_t k = 0; k < nl; k++) l2[k] = make_float2(lh[k], lo[k]);
+    float2* p2;
+    st = upload(ctx, &p2, l2.data(), nl, &g->allocs, &g->bytes);
+    dv.lnl2 = p2;
+  }
   if (!st) { st = upload(ctx, &pu, lut.data(), lut.size(), &g->allocs, &g->bytes); dv.lut = pu; }
   if (!st) {
     std::vector<float4> a4(nl);

@@ -109,6 +109,7 @@ struct GridDev {
   const float* drude;      // Drude profile with E_b = 1
   const float* lnl_hi;     // ln(lambda) split in two floats
   const float* lnl_lo;
+  const float2* lnl2;      // {lnl_hi, lnl_lo}
   const uint16_t* lut;     // lut[q] = last node with ln(lambda) <= x0 + q/inv_h (n_lam <= MAX_LAM < 2^16)
   int lut_n;
   float lut_x0, lut_inv_h;
@@ -655,7 +656,7 @@ struct EpiArgs {
   const int* err;      // device error word of the contraction (row status SED_ROW_DEVICE_TIMEOUT)
   const float* lam8;   // FP8 path: [n_lam] 2^-f_l multiplying Y and O; NULL otherwise
   int lines_off;       // set by launch_epilogue: float offsets of the emission lines' shared arrays and of
-  int terms_off;       //   the samples' and pixels' terms
+  int samp_off, res_off;   //   the samples' values and the pixels' residuals
   size_t seg_stride;   // age-binned dust: Y of attenuated block s at Y + s seg_stride
   const float* qneb;   // nebular age axis: [n][MAX_NEB_AGE] (k_prep's), or NULL
   int* win_reset;      // [2][win_mt] per-tile windows set back to empty by CTA 0 (the contraction,

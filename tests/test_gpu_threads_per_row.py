@@ -38,12 +38,13 @@ def _case(kind):
         return w, orc, lambda n: cases.lines_theta_pair(w, orc, n, seed=11)[0]
     w = {"tiny": synth.WORKLOADS["tiny_phot_16x4x512"], "phot": _small("phot_107x12x6000_b1024"),
          "calib": _small(SPEC, 257), "sgal": _small("specphot_afe_sgal_107x12x5x6000_b2048", 130),
-         "floor": _small("specphot_afe_floor_107x12x5x6000_b2048", 100)}[kind]
+         "floor": _small("specphot_afe_floor_107x12x5x6000_b2048", 100),
+         "dense": _small(SPEC, 2001)}[kind]   # more pixels than twice the row's nodes
     orc = cases.calib_case(w, [0.2] + [0.1] * 12) if kind == "calib" else cases.oracle_for(w)
     return w, orc, lambda n: cases.theta_pair(w, n, seed=11, orc=orc)[0]
 
 
-@pytest.mark.parametrize("kind", ["tiny", "phot", "calib", "sgal", "floor", "lines"])
+@pytest.mark.parametrize("kind", ["tiny", "phot", "calib", "sgal", "floor", "lines", "dense"])
 def test_rows_do_not_depend_on_the_threads_per_row(ctx, kind):
     w, orc, rows = _case(kind)
     model = cases.gpu_model_for(ctx, orc, w)
