@@ -15,7 +15,13 @@
 // every tile reads one A operand; the columns of a tile past the end of its
 // block are computed but not stored.
 //
-// One CTA computes a 128 (theta) x BN tile (of Y and of O, or of dW).  Warp roles:
+// One CTA computes a tile of 128 wavelengths (columns of Y and O, or of dW) by up
+// to 128 rows (theta): the SSP is the MMA's M operand, the rows its N operand, so
+// that an accumulator's lanes are consecutive columns of the output and each
+// store of a warp writes 128 consecutive bytes of one row.  (With the rows as M a
+// warp's store touched 32 rows: without the stores the 4096-row BF16 contraction
+// took 37 us instead of 55.)  The row operand is loaded in boxes of 32 rows, so a
+// small launch or a piece of a tile loads and multiplies only its own.  Warp roles:
 //   warp 0 lane 0 : TMA producer (128B-swizzled K tiles into a STAGES-deep ring)
 //   warp 1 lane 0 : MMA issuer (tcgen05.mma into a ping-pong pair of tensor-memory
 //                   accumulators; a commit frees a smem stage / hands over a buffer)
@@ -69,6 +75,22 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     if (mbar_try(bar, parity)) return true;
     if ((it & 255u) == 0 && gtimer() - t0 > 2000000000ull) return false;
   }
+}
+// One lane of the (converged) warp, the same one each time.  The TMA and MMA
+// instructions take their operands from uniform registers: issued under this
+// predicate, with the warp's control flow uniform around it, they are issued
+// back to back; under a test of the lane index every operand is made uniform
+// at run time, and an MMA took over 100 cycles to issue whatever its size.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t.reg .b32 l;\n\t"
+      "elect.sync l|q, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}\n"
+      : "=r"(p)
+      :
+      : "memory");
+  return p != 0;
 }
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1) {
   asm volatile(
@@ -188,16 +210,17 @@ __device__ __forceinline__ int knext(const uint32_t* km, int kt, int end) {
   return end;
 }
 
-constexpr int BM = 128;
+constexpr int BM = 128;    // columns of a tile (MMA M)
+constexpr int BOX = 32;    // rows of one load of the row operand
+constexpr int MAX_STAGES = 8;
 constexpr int ROWB = 128;  // bytes of one operand row in a K tile
 
 template <int PREC, int BN, int STAGES, int G, bool GRAD = false>
 struct Cfg {
-  static constexpr int A_BYTES = BM * ROWB;
-  static constexpr int B_BYTES = BN * ROWB;
+  static constexpr int S_BYTES = BM * ROWB;                   // the SSP part of a stage
   static constexpr int NOPS = PREC == SED_PREC_FP32 ? 2 : 1;  // hi/lo parts
-  static constexpr int STAGE_BYTES = NOPS * (A_BYTES + B_BYTES);
-  static constexpr int SMEM = STAGES * STAGE_BYTES + 1024;    // + alignment slack
+  static constexpr int RING = STAGES * NOPS * (S_BYTES + BN * ROWB);   // operand ring: STAGES stages of BN rows,
+  static constexpr int SMEM = RING + 1024;                             // more of fewer; + alignment slack
   // the two accumulator buffers; the 3xTF32 forward adds BN columns where an unsplit unit keeps the
   // old part's first half (see unit_range)
   static constexpr int COLS_USED = 2 * BN + (PREC == SED_PREC_FP32 && !GRAD ? BN : 0);
@@ -232,7 +255,8 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 // step 0.0927 against 0.0948 ms split, 4096 rows 0.2960 against 0.3125 ms, the
 // 2048-row [a/Fe] spectro-photometric forward 0.3648 against 0.3865 ms), but
 // with a few tiles more than SMs its leftover tiles leave a few CTAs a second
-// unit (154 tiles on 152 SMs: 0.109 against 0.099 ms split).
+// unit (154 tiles on 152 SMs: 0.109 against 0.099 ms split); and 51 tiles of
+// K = 6528 (301 rows) take 135 us as units against 70 us split.
 //  - Grid schedule (p.tile_win NULL): one unit per CTA from blockIdx; the CTA
 //    exits at once when the tile lies outside the union of its rows' windows.
 //  - Persistent schedule (forward, p.tile_win set): one CTA per SM; every CTA
@@ -240,16 +264,16 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 //    preparation kernel and takes every gridDim.x-th one.  The tiles (M tile,
 //    then the wavelength tiles of its window) are cut into full waves -- the
 //    largest multiple of gridDim.x, run as whole units -- and a remainder whose
-//    tiles are split along the wavelength axis into up to four pieces of
-//    BN/npc columns (an MMA of N = BN/npc), so the last partial wave costs a
-//    fraction of a unit.  Tensor memory, barriers and the smem ring are set up
+//    tiles are split along the rows into up to four pieces of BN/npc rows (an
+//    MMA of N = BN/npc), so the last partial wave costs a fraction of a unit.  Tensor memory, barriers and the smem ring are set up
 //    once, and one unit's drain overlaps the next unit's MMAs.
 constexpr int MAX_MT = 64;   // M tiles of a persistent launch (8192 rows)
 
 struct Unit {
   const uint32_t* km;        // K-tile mask row of the unit's M tile (NULL: every K tile)
-  int m0, n0, nr;
-  int ncol;                  // columns of the tile that are stored (a multiple of 4)
+  int m0, n0, nr;            // first row, first column, K ranges
+  int rows;                  // rows of the unit (a multiple of BOX; the MMA's N)
+  int ncol;                  // columns of the tile that are stored (the adjoint's may end within it)
   int kind;                  // 0, 1: the old part's halves (3-way split); 2: the young blocks, then the
                              // old part unless split; the adjoint has one range
   int K0, KY, KT;
@@ -289,26 +313,26 @@ __device__ __forceinline__ void unit_ranges(const Params& p, int z, int nz, int 
   u.nr = u.kind < 2 ? 1 : p.n_seg + (nz == 3 ? 0 : (PREC == SED_PREC_FP32 ? 2 : 1));
 }
 
-// Pieces of a leftover tile (1, 2 or 4 along the wavelength axis: BN/npc stays
-// a multiple of 16) when nz units per tile leave nrem tiles past the full waves.
-template <int BN>
-__device__ __forceinline__ int pieces_for(int P, int nz, int nrem) {
+// Pieces of a leftover tile (1, 2 or 4 along the rows, each whole boxes) when nz
+// units per tile leave nrem tiles past the full waves; a launch of fewer than
+// BN rows (rt, in whole boxes) splits those.
+__device__ __forceinline__ int pieces_for(int P, int nz, int nrem, int rt) {
   const int fit = nrem > 0 ? P / (nz * nrem) : 1;
-  return (fit >= 4 && BN / 4 >= 16) ? 4 : (fit >= 2 && BN / 2 >= 16 ? 2 : 1);
+  return (fit >= 4 && rt % (4 * BOX) == 0) ? 4 : (fit >= 2 && rt % (2 * BOX) == 0 ? 2 : 1);
 }
 // The longest CTA's work, in K tiles, of a persistent launch over `tiles`
 // tiles on P CTAs with nz units per tile of kmax K tiles at most (kt in all):
 // the full waves, then the leftover tiles' pieces spread over the CTAs, a
-// piece costing about 0.6 (two) or 0.4 (four pieces) of its unit (the A tile
-// and the MMA issue do not shrink with N).
-template <int BN>
-__device__ __forceinline__ float sched_longest(int tiles, int P, int nz, int kt, int kmax) {
+// piece costing about 0.9 (two) or 0.85 (four pieces) of its unit: an MMA of
+// M = 128 takes about 60 cycles for any N up to 128 (measured with the ring's
+// loads and waits left out), so a piece saves loads and stores alone.
+__device__ __forceinline__ float sched_longest(int tiles, int P, int nz, int kt, int kmax, int rt) {
   const int nfull = (tiles / P) * P, nrem = tiles - nfull;
   float w = (float)(nfull / P) * (float)kt;
   if (nrem > 0) {
-    const int npc = pieces_for<BN>(P, nz, nrem);
+    const int npc = pieces_for(P, nz, nrem, rt);
     const int per_cta = (nz * nrem * npc + P - 1) / P;
-    w += (float)per_cta * (float)kmax * (npc == 1 ? 1.f : (npc == 2 ? 0.6f : 0.4f));
+    w += (float)per_cta * (float)kmax * (npc == 1 ? 1.f : (npc == 2 ? 0.9f : 0.85f));
   }
   return w;
 }
@@ -319,11 +343,10 @@ __device__ __forceinline__ float sched_longest(int tiles, int P, int nz, int kt,
 // 16 us longer epilogue for no shorter contraction; at 1024 rows, 154 tiles,
 // the split step took 0.099 against 0.109 ms unsplit).
 constexpr float SPLIT_EPI_KT_PER_TILE = 0.04f;
-template <int BN>
-__device__ __forceinline__ bool split_pays(int tiles, int P, int ky, int kt) {
+__device__ __forceinline__ bool split_pays(int tiles, int P, int ky, int kt, int rt) {
   const int ko = kt - ky, kh = (ko + 1) / 2;
-  const float one = sched_longest<BN>(tiles, P, 1, kt, kt);
-  const float three = sched_longest<BN>(tiles, P, 3, kt, max(kh, ky)) + SPLIT_EPI_KT_PER_TILE * (float)tiles;
+  const float one = sched_longest(tiles, P, 1, kt, kt, rt);
+  const float three = sched_longest(tiles, P, 3, kt, max(kh, ky), rt) + SPLIT_EPI_KT_PER_TILE * (float)tiles;
   return three < 0.95f * one;
 }
 
@@ -331,10 +354,9 @@ __device__ __forceinline__ bool split_pays(int tiles, int P, int ky, int kt) {
 // unmasked loops carry no mask test)
 template <int PREC, int BN, int STAGES, int G, bool GRAD, bool KSKIP = false>
 __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ Params p) {
-  pdl_enter();
   using C = Cfg<PREC, BN, STAGES, G, GRAD>;
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t bars[2 * STAGES + 4];
+  __shared__ __align__(8) uint64_t bars[2 * MAX_STAGES + 4];
   __shared__ uint32_t tmem_base_s;
   __shared__ int s_klo, s_khi;
   __shared__ int s_nlo[MAX_MT], s_pref[MAX_MT + 1];
@@ -347,12 +369,16 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
   int nfull = 0, nrem = 0, npc = 1;   // persistent: tiles in full waves, leftover tiles, pieces per leftover tile
 
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[STAGES]);
-  const uint32_t tfull0 = smem_u32(&bars[2 * STAGES]), tempty0 = smem_u32(&bars[2 * STAGES + 2]);
+  const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[MAX_STAGES]);
+  const uint32_t tfull0 = smem_u32(&bars[2 * MAX_STAGES]), tempty0 = smem_u32(&bars[2 * MAX_STAGES + 2]);
+  // rows of the launch's tiles (whole boxes); a stage holds {SSP, rows} of each part
+  const int rt = min(BN, (p.n + BOX - 1) / BOX * BOX);
+  const int r_bytes = rt * ROWB, stage_bytes = C::NOPS * (C::S_BYTES + r_bytes);
+  const int stages = min(MAX_STAGES, C::RING / stage_bytes);
   // barriers and tensor memory (made visible by the barrier before the roles)
   auto setup = [&]() {
     if (threadIdx.x == 0) {
-      for (int s = 0; s < STAGES; ++s) {
+      for (int s = 0; s < stages; ++s) {
         mbar_init(full0 + 8 * s, 1);
         mbar_init(empty0 + 8 * s, 1);
       }
@@ -371,12 +397,19 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
     }
   };
 
+  if (threadIdx.x == 32) {
+    for (const CUtensorMap* m : {&p.a_hi, &p.b_hi}) asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
+    if constexpr (C::NOPS == 2)
+      for (const CUtensorMap* m : {&p.a_lo, &p.b_lo}) asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
+  }
+  // the persistent CTA always works (or frees its tensor memory below): barriers
+  // and tensor memory are set up in the shadow of the kernel before
+  if (persistent) setup();
+  pdl_enter();
+
   // a launch that cannot split records that it did not
   if (!GRAD && !persistent && p.split_out && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *p.split_out = 0;
   if (persistent) {
-    // the persistent CTA always works (or frees its tensor memory below):
-    // set up first, so that the allocation overlaps the reads of the windows
-    setup();
     // computed wavelength tiles of each M tile, and their prefix counts.  The
     // tiles of an M tile start at its window's first node rounded down to 16
     // columns (not to a whole tile), shifted down where the last one would pass
@@ -389,8 +422,8 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
       int a = 0, c = 0;
       if (hi >= 0) {
         a = lo & ~15;
-        c = (min(hi, p.ldn - 1) - a) / BN + 1;
-        a = min(a, p.ldn - c * BN);
+        c = (min(hi, p.ldn - 1) - a) / BM + 1;
+        a = min(a, p.ldn - c * BM);
       }
       s_nlo[threadIdx.x] = a;   // first column
       s_pref[threadIdx.x + 1] = c;
@@ -406,16 +439,14 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
     // (every CTA takes the same decision; CTA 0 records it for the epilogues).
     // Per kind, the largest multiple of gridDim.x tiles runs as whole units
     // (every CTA then takes the same number of units of each kind); the
-    // leftover tiles are cut along the wavelength axis into npc pieces of BN/npc
-    // columns so that the last partial wave spreads over the CTAs.  npc is 1, 2
-    // or 4 (BN/npc stays a multiple of 16: a valid MMA N and 16-byte aligned
-    // output columns)
+    // leftover tiles are cut along the rows into npc pieces of rt/npc rows so that
+    // the last partial wave spreads over the CTAs
     const int nctas = (int)gridDim.x;
-    nz = p.O2 && split_pays<BN>(upz, nctas, KY, KT) ? 3 : 1;
+    nz = p.O2 && split_pays(upz, nctas, KY, KT, rt) ? 3 : 1;
     if (blockIdx.x == 0 && threadIdx.x == 0 && p.split_out) *p.split_out = nz == 3 ? 1 : 0;
     nfull = (upz / nctas) * nctas;
     nrem = upz - nfull;
-    npc = pieces_for<BN>(nctas, nz, nrem);
+    npc = pieces_for(nctas, nz, nrem, rt);
     const int total = nz * nfull + nz * nrem * npc;
     n_units = total > (int)blockIdx.x ? (total - 1 - (int)blockIdx.x) / nctas + 1 : 0;
     if (n_units == 0) {   // no unit for this CTA: free the tensor memory and leave
@@ -433,10 +464,10 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
     // (invalid rows have none).  Forward: a wavelength tile outside it is never
     // read, so the CTA exits.  Adjoint: dlnL/dY and dlnL/dO vanish outside each
     // row's window, so the reduction over wavelength runs over the union only.
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+    const int m0 = blockIdx.y * BN, n0 = blockIdx.x * BM;
     if (threadIdx.x == 0) { s_klo = 0x7fffffff; s_khi = -1; }
     __syncthreads();
-    if (threadIdx.x < BM && m0 + (int)threadIdx.x < p.n) {
+    if (threadIdx.x < BN && m0 + (int)threadIdx.x < p.n) {
       const RowScal& q = p.rs[m0 + threadIdx.x];
       if (q.status == 0) { atomicMin(&s_klo, q.k_lo); atomicMax(&s_khi, q.k_hi); }
     }
@@ -444,7 +475,7 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
     const int klo = s_klo, khi = s_khi;
     if (khi < 0) return;
     if constexpr (!GRAD) {
-      if (n0 > khi || n0 + BN - 1 < klo) return;
+      if (n0 > khi || n0 + BM - 1 < klo) return;
     } else {
       // the reduction over lambda covers the union of the tile's row windows
       // (dlnL/dY and dlnL/dO are zero outside each row's own); its start is
@@ -456,8 +487,8 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
       KY = KT;
       if (p.kmask) {   // dW columns of this tile: none touched by the tile's rows -> not needed
         const int t = (int)blockIdx.x;
-        const int c0 = t < p.ny_tiles ? t * BN : p.n_split + (t - p.ny_tiles) * BN;
-        const int c1 = min(c0 + BN, t < p.ny_tiles ? p.n_split : p.ld_out);
+        const int c0 = t < p.ny_tiles ? t * BM : p.n_split + (t - p.ny_tiles) * BM;
+        const int c1 = min(c0 + BM, t < p.ny_tiles ? p.n_split : p.ld_out);
         if (knext(p.kmask + (size_t)blockIdx.y * p.kmask_w, c0 / 32, (c1 + 31) / 32) >= (c1 + 31) / 32) return;
       }
     }
@@ -472,7 +503,8 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
   // unit j of this CTA
   auto get_unit = [&](int j, Unit& u) {
     int z = 0;
-    u.ncol = BN;
+    u.ncol = BM;
+    u.rows = rt;
     if (persistent) {
       const int idx = (int)blockIdx.x + j * (int)gridDim.x;
       int t, pc = 0;
@@ -485,23 +517,28 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
         z = rest / nrem;
         t = nfull + rest - z * nrem;
       }
-      int m = 0;
-      while (s_pref[m + 1] <= t) ++m;
-      u.m0 = m * BM;
-      u.km = KSKIP ? p.kmask + m * p.kmask_w : nullptr;   // read through L1 (a few words per M tile)
-      if (t >= nfull) u.ncol = BN / npc;   // a piece of a leftover tile
-      u.n0 = s_nlo[m] + (t - s_pref[m]) * BN + pc * u.ncol;
+      int m = 0, m1 = p.m_tiles - 1;   // the row tile: s_pref[m] <= t < s_pref[m + 1]
+      while (m < m1) {
+        const int mid = (m + m1) >> 1;
+        if (s_pref[mid + 1] <= t) m = mid + 1; else m1 = mid;
+      }
+      u.km = KSKIP ? p.kmask + m * p.kmask_w : nullptr;   // read through L1 (a few words per row tile)
+      if (t >= nfull) u.rows = rt / npc;   // a piece of a leftover tile
+      u.m0 = m * BN + pc * u.rows;
+      u.n0 = s_nlo[m] + (t - s_pref[m]) * BM;
     } else {
-      u.m0 = blockIdx.y * BM;
-      u.n0 = blockIdx.x * BN;
+      u.m0 = blockIdx.y * BN;
+      u.n0 = blockIdx.x * BM;
       u.km = KSKIP ? p.kmask + (size_t)blockIdx.y * p.kmask_w : nullptr;
     }
     if constexpr (GRAD) u.km = nullptr;   // the adjoint reduces over lambda
     if constexpr (GRAD) {
       const int t = (int)blockIdx.x;
-      u.n0 = t < p.ny_tiles ? t * BN : p.n_split + (t - p.ny_tiles) * BN;
-      u.ncol = min(BN, (t < p.ny_tiles ? p.n_split : p.ld_out) - u.n0);
+      u.n0 = t < p.ny_tiles ? t * BM : p.n_split + (t - p.ny_tiles) * BM;
+      u.ncol = min(BM, (t < p.ny_tiles ? p.n_split : p.ld_out) - u.n0);
     }
+    // the last row tile's rows end with the launch's
+    u.rows = max(BOX, min(u.rows, (p.n - u.m0 + BOX - 1) / BOX * BOX));
     unit_ranges<PREC, GRAD>(p, z, nz, K0, KY, KT, u);
   };
 
@@ -512,96 +549,110 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
   const uint32_t tmem = tmem_base_s;
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ---------------- TMA producer
-      int it = 0;
-      bool ok = true;
-      for (int j = 0; j < n_units && ok; ++j) {
-        Unit u;
-        get_unit(j, u);
-        const CUtensorMap* amap_hi = &p.a_hi;
-        const CUtensorMap* amap_lo = &p.a_lo;
-        int arow = u.m0;   // adjoint: block s of the young columns reads rows s seg_rows + m of its A map
-        if (GRAD && u.n0 >= p.n_split) { amap_hi = &p.a2_hi; amap_lo = &p.a2_lo; }
-        else if (GRAD)
-          for (int sg = 1; sg < p.n_seg; ++sg)
-            if (u.n0 >= p.seg_col[sg]) arow = u.m0 + sg * p.seg_rows;
-        for (int r = 0; r < u.nr && ok; ++r) {
-          int rb, re;
-          float* ro_;
-          int mode_;
-          unit_range<PREC, GRAD>(p, u, r, rb, re, ro_, mode_);
-          for (int kt = kn(u.km, rb, re); kt < re; kt = kn(u.km, kt + 1, re), ++it) {
-            const int s = it % STAGES;
-            const uint32_t ph = (uint32_t)(it / STAGES) & 1u;
-            if (!mbar_wait(empty0 + 8 * s, ph ^ 1u)) { atomicOr(p.err, 1); ok = false; break; }
-            const uint32_t fb = full0 + 8 * s;
-            mbar_expect_tx(fb, C::STAGE_BYTES);
-            const uint32_t st = sbase + s * C::STAGE_BYTES;
+    // ---------------- TMA producer (the whole warp walks the loop, one lane issues)
+    int st_i = 0;          // stage and its phase
+    uint32_t st_ph = 0;
+    bool ok = true;
+    for (int j = 0; j < n_units && ok; ++j) {
+      Unit u;
+      get_unit(j, u);
+      const CUtensorMap* amap_hi = &p.a_hi;
+      const CUtensorMap* amap_lo = &p.a_lo;
+      int arow = u.m0;   // adjoint: block s of the young columns reads rows s seg_rows + m of its A map
+      if (GRAD && u.n0 >= p.n_split) { amap_hi = &p.a2_hi; amap_lo = &p.a2_lo; }
+      else if (GRAD)
+        for (int sg = 1; sg < p.n_seg; ++sg)
+          if (u.n0 >= p.seg_col[sg]) arow = u.m0 + sg * p.seg_rows;
+      for (int r = 0; r < u.nr && ok; ++r) {
+        int rb, re;
+        float* ro_;
+        int mode_;
+        unit_range<PREC, GRAD>(p, u, r, rb, re, ro_, mode_);
+        for (int kt = kn(u.km, rb, re); kt < re; kt = kn(u.km, kt + 1, re)) {
+          if (!__all_sync(0xffffffffu, mbar_wait(empty0 + 8 * st_i, st_ph ^ 1u))) {
+            if (lane == 0) atomicOr(p.err, 1);
+            ok = false;
+            break;
+          }
+          if (elect_one()) {
+            const uint32_t fb = full0 + 8 * st_i;
+            mbar_expect_tx(fb, C::NOPS * (C::S_BYTES + u.rows * ROWB));
+            const uint32_t st = sbase + st_i * stage_bytes;
             const int kc = kt * (ROWB / (PREC == SED_PREC_FP32 ? 4 : (PREC == SED_PREC_FP8 ? 1 : 2)));  // element coordinate along K
-            tma_load_2d(st, amap_hi, fb, kc, arow);
-            tma_load_2d(st + C::A_BYTES, &p.b_hi, fb, kc, u.n0);
+            tma_load_2d(st, &p.b_hi, fb, kc, u.n0);
+            for (int q = 0; q < u.rows; q += BOX) tma_load_2d(st + C::S_BYTES + q * ROWB, amap_hi, fb, kc, arow + q);
             if constexpr (C::NOPS == 2) {
-              tma_load_2d(st + C::A_BYTES + C::B_BYTES, amap_lo, fb, kc, arow);
-              tma_load_2d(st + 2 * C::A_BYTES + C::B_BYTES, &p.b_lo, fb, kc, u.n0);
+              const uint32_t lo = st + C::S_BYTES + r_bytes;
+              tma_load_2d(lo, &p.b_lo, fb, kc, u.n0);
+              for (int q = 0; q < u.rows; q += BOX) tma_load_2d(lo + C::S_BYTES + q * ROWB, amap_lo, fb, kc, arow + q);
             }
           }
+          __syncwarp();
+          if (++st_i == stages) { st_i = 0; st_ph ^= 1u; }
         }
       }
     }
-    __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer
-      constexpr uint32_t FMT = PREC == SED_PREC_FP32 ? 2u : (PREC == SED_PREC_FP8 ? 0u : 1u);
-      int g = 0, it = 0;
-      bool ok = true;
-      for (int j = 0; j < n_units && ok; ++j) {
-        Unit u;
-        get_unit(j, u);
-        const uint32_t ID = idesc(FMT, BM, (uint32_t)u.ncol);   // N = the unit's columns
-        for (int r = 0; r < u.nr && ok; ++r) {
-          int kb, ke;
-          float* ro_;
-          int mode_;
-          unit_range<PREC, GRAD>(p, u, r, kb, ke, ro_, mode_);
-          for (int gs = kb; gs < ke && ok; gs += G) {
-            const int ge = gs + G < ke ? gs + G : ke;
-            const int k_first = kn(u.km, gs, ge);
-            if (KSKIP && k_first >= ge) continue;   // no touched K tile in this group
-            const int b = g & 1;
-            if (!mbar_wait(tempty0 + 8 * b, (((uint32_t)g >> 1) & 1u) ^ 1u)) { atomicOr(p.err, 8); ok = false; break; }
+    // ---------------- MMA issuer (as above)
+    constexpr uint32_t FMT = PREC == SED_PREC_FP32 ? 2u : (PREC == SED_PREC_FP8 ? 0u : 1u);
+    const uint64_t d_ring = sdesc(sbase);   // descriptors differ in their address field alone, in units of 16 bytes
+    int g = 0, st_i = 0;
+    uint32_t st_ph = 0;
+    bool ok = true;
+    for (int j = 0; j < n_units && ok; ++j) {
+      Unit u;
+      get_unit(j, u);
+      const uint32_t ID = idesc(FMT, BM, (uint32_t)u.rows);
+      for (int r = 0; r < u.nr && ok; ++r) {
+        int kb, ke;
+        float* ro_;
+        int mode_;
+        unit_range<PREC, GRAD>(p, u, r, kb, ke, ro_, mode_);
+        for (int gs = kb; gs < ke && ok; gs += G) {
+          const int ge = gs + G < ke ? gs + G : ke;
+          const int k_first = kn(u.km, gs, ge);
+          if (KSKIP && k_first >= ge) continue;   // no touched K tile in this group
+          const int b = g & 1;
+          if (!__all_sync(0xffffffffu, mbar_wait(tempty0 + 8 * b, (((uint32_t)g >> 1) & 1u) ^ 1u))) {
+            if (lane == 0) atomicOr(p.err, 8);
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t d = tmem + (uint32_t)(b * BN);
+          uint32_t acc = 0;
+          for (int kt = k_first; kt < ge; kt = kn(u.km, kt + 1, ge)) {
+            if (!__all_sync(0xffffffffu, mbar_wait(full0 + 8 * st_i, st_ph))) {
+              if (lane == 0) atomicOr(p.err, 2);
+              ok = false;
+              break;
+            }
             tc_fence_after();
-            const uint32_t d = tmem + (uint32_t)(b * BN);
-            for (int kt = k_first; kt < ge; kt = kn(u.km, kt + 1, ge), ++it) {
-              const int s = it % STAGES;
-              const uint32_t ph = (uint32_t)(it / STAGES) & 1u;
-              if (!mbar_wait(full0 + 8 * s, ph)) { atomicOr(p.err, 2); ok = false; break; }
-              tc_fence_after();
-              const uint32_t st = sbase + s * C::STAGE_BYTES;
-              const uint32_t a_hi = st, b_hi = st + C::A_BYTES;
+            if (elect_one()) {
+              const uint64_t s_hi = d_ring + (uint32_t)(st_i * stage_bytes >> 4), r_hi = s_hi + (C::S_BYTES >> 4);
+              const uint64_t s_lo = r_hi + (uint32_t)(r_bytes >> 4), r_lo = s_lo + (C::S_BYTES >> 4);
 #pragma unroll
               for (int kk = 0; kk < 4; ++kk) {   // 4 MMAs of 32 bytes of K each
-                const uint32_t acc = (kt == k_first && kk == 0) ? 0u : 1u;
-                const uint64_t da = sdesc(a_hi + kk * 32), db = sdesc(b_hi + kk * 32);
                 if constexpr (C::NOPS == 2) {
-                  const uint32_t a_lo = st + C::A_BYTES + C::B_BYTES, b_lo = a_lo + C::A_BYTES;
-                  mma<PREC>(d, sdesc(a_lo + kk * 32), db, ID, acc);
-                  mma<PREC>(d, da, sdesc(b_lo + kk * 32), ID, 1u);
-                  mma<PREC>(d, da, db, ID, 1u);
+                  mma<PREC>(d, s_hi + 2 * kk, r_lo + 2 * kk, ID, kk ? 1u : acc);
+                  mma<PREC>(d, s_lo + 2 * kk, r_hi + 2 * kk, ID, 1u);
+                  mma<PREC>(d, s_hi + 2 * kk, r_hi + 2 * kk, ID, 1u);
                 } else {
-                  mma<PREC>(d, da, db, ID, acc);
+                  mma<PREC>(d, s_hi + 2 * kk, r_hi + 2 * kk, ID, kk ? 1u : acc);
                 }
               }
-              mma_commit(empty0 + 8 * s);
+              mma_commit(empty0 + 8 * st_i);
             }
-            if (ok) mma_commit(tfull0 + 8 * b);
-            ++g;
+            __syncwarp();
+            acc = 1u;
+            if (++st_i == stages) { st_i = 0; st_ph ^= 1u; }
           }
+          if (ok && elect_one()) mma_commit(tfull0 + 8 * b);
+          __syncwarp();
+          ++g;
         }
       }
     }
-    __syncwarp();
   } else {
     // ---------------- drain: warps 2..5 cover TMEM lane quadrants 2,3,0,1
     const int q = warp & 3;
@@ -611,7 +662,8 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
     for (int j = 0; j < n_units; ++j) {
       Unit u;
       get_unit(j, u);
-      const int row = u.m0 + q * 32 + lane;
+      const int col = q * 32 + lane;                 // this thread's column of the tile
+      const int vrow = min(u.rows, p.n - u.m0);      // rows to store
       for (int r = 0; r < u.nr; ++r) {
         int kb, ke;
         float* out;
@@ -628,7 +680,7 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
           if (ok) {
 #pragma unroll
             for (int c = 0; c < BN / 32; ++c) {
-              if (c * 32 >= u.ncol) break;
+              if (c * 32 >= u.rows) break;
               uint32_t rr[32];
               tmem_ld32(tmem + lane_off + (uint32_t)(b * BN + c * 32), rr);
               tmem_wait_ld();
@@ -647,7 +699,7 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
           const uint32_t scr = tmem + lane_off + (uint32_t)(2 * BN);
 #pragma unroll
           for (int c = 0; c < BN / 32; ++c) {
-            if (c * 32 >= u.ncol) break;
+            if (c * 32 >= u.rows) break;
             if (mode == 1) {
               tmem_st32(scr + (uint32_t)(c * 32), &run[c * 32]);
             } else {
@@ -663,11 +715,17 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
             continue;
           }
         }
-        if (row < p.n) {
-          float4* dst = reinterpret_cast<float4*>(out + (size_t)row * p.ld_out + u.n0);
+        if (col < u.ncol) {   // a warp stores 32 consecutive columns of one row at a time
+          float* dst = out + (size_t)u.m0 * p.ld_out + u.n0 + col;
 #pragma unroll
-          for (int c = 0; c < BN / 4; ++c)
-            if (4 * c < u.ncol) dst[c] = make_float4(run[4 * c], run[4 * c + 1], run[4 * c + 2], run[4 * c + 3]);
+          for (int c = 0; c < BN / 32; ++c) {
+            if (c * 32 >= vrow) break;
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+              if (c * 32 + i < vrow) *dst = run[c * 32 + i];
+              dst += p.ld_out;
+            }
+          }
         }
       }
     }
@@ -688,7 +746,7 @@ cudaError_t launch_cfg(const Params& p, int n_cols, cudaStream_t s) {
   static DynSmemCache attr;   // the raised shared-memory limit, set once per device
   if (cudaError_t e = ensure_dyn_smem(k, (size_t)C::SMEM, &attr)) return e;
   if (!GRAD && p.tile_win) return launch_pdl(k, dim3(n_sm, 1, 1), dim3(C::THREADS), C::SMEM, s, p);   // persistent: one CTA per SM
-  return launch_pdl(k, dim3(n_cols / BN, (p.n + BM - 1) / BM, 1), dim3(C::THREADS), C::SMEM, s, p);
+  return launch_pdl(k, dim3(n_cols / BM, (p.n + BN - 1) / BN, 1), dim3(C::THREADS), C::SMEM, s, p);
 }
 
 }  // namespace tc
@@ -729,11 +787,11 @@ int tc_encode_maps(void* fn, TcMaps* out, int prec, const void* a_hi, const void
   const CUtensorMapDataType dt = f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                                      : (f8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
   const int es = f32 ? 4 : (f8 ? 1 : 2);
-  if (encode_kmajor(fn, &out->a_hi, const_cast<void*>(a_hi), dt, es, kpad, n, tc::BM) != CUDA_SUCCESS) return 1;
+  if (encode_kmajor(fn, &out->a_hi, const_cast<void*>(a_hi), dt, es, kpad, n, tc::BOX) != CUDA_SUCCESS) return 1;
   const int bn = tc_bn_for(prec, kpad);
   if (encode_kmajor(fn, &out->b_hi, const_cast<void*>(b_hi), dt, es, kpad, n_lam, bn) != CUDA_SUCCESS) return 2;
   if (f32) {
-    if (encode_kmajor(fn, &out->a_lo, const_cast<void*>(a_lo), dt, es, kpad, n, tc::BM) != CUDA_SUCCESS) return 3;
+    if (encode_kmajor(fn, &out->a_lo, const_cast<void*>(a_lo), dt, es, kpad, n, tc::BOX) != CUDA_SUCCESS) return 3;
     if (encode_kmajor(fn, &out->b_lo, const_cast<void*>(b_lo), dt, es, kpad, n_lam, bn) != CUDA_SUCCESS) return 4;
   } else {
     out->a_lo = out->a_hi;
@@ -750,7 +808,7 @@ cudaError_t launch_contract_tc(const TcArgs& a, cudaStream_t s) {
   p.n = a.n; p.n_lam = a.n_lam; p.ldn = a.ldn; p.ld_out = a.ldn;
   p.Y = a.Y; p.O = a.O; p.err = a.err;
   p.split_out = a.split_out;
-  p.m_tiles = (a.n + tc::BM - 1) / tc::BM;
+  p.m_tiles = (a.n + 127) / 128;
   p.tile_win = (a.tile_win && p.m_tiles <= tc::MAX_MT) ? a.tile_win : nullptr;
   // the 3-way split is a choice of the persistent 3xTF32 launch
   p.O2 = a.prec == SED_PREC_FP32 && p.tile_win ? a.O2 : nullptr;
@@ -786,10 +844,10 @@ int tc_encode_dw_maps(void* fn, DwMaps* out, const float* gy_hi, const float* gy
                       const float* go_lo, const float* sk_hi, const float* sk_lo, int n, int n_gy, int ldg, int ldk,
                       int kpad) {
   const CUtensorMapDataType dt = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
-  if (encode_kmajor(fn, &out->gy_hi, (void*)gy_hi, dt, 4, ldg, n_gy, tc::BM) != CUDA_SUCCESS) return 1;
-  if (encode_kmajor(fn, &out->gy_lo, (void*)gy_lo, dt, 4, ldg, n_gy, tc::BM) != CUDA_SUCCESS) return 2;
-  if (encode_kmajor(fn, &out->go_hi, (void*)go_hi, dt, 4, ldg, n, tc::BM) != CUDA_SUCCESS) return 3;
-  if (encode_kmajor(fn, &out->go_lo, (void*)go_lo, dt, 4, ldg, n, tc::BM) != CUDA_SUCCESS) return 4;
+  if (encode_kmajor(fn, &out->gy_hi, (void*)gy_hi, dt, 4, ldg, n_gy, tc::BOX) != CUDA_SUCCESS) return 1;
+  if (encode_kmajor(fn, &out->gy_lo, (void*)gy_lo, dt, 4, ldg, n_gy, tc::BOX) != CUDA_SUCCESS) return 2;
+  if (encode_kmajor(fn, &out->go_hi, (void*)go_hi, dt, 4, ldg, n, tc::BOX) != CUDA_SUCCESS) return 3;
+  if (encode_kmajor(fn, &out->go_lo, (void*)go_lo, dt, 4, ldg, n, tc::BOX) != CUDA_SUCCESS) return 4;
   if (encode_kmajor(fn, &out->s_hi, (void*)sk_hi, dt, 4, ldk, kpad, DW_BN) != CUDA_SUCCESS) return 5;
   if (encode_kmajor(fn, &out->s_lo, (void*)sk_lo, dt, 4, ldk, kpad, DW_BN) != CUDA_SUCCESS) return 6;
   return 0;
