@@ -153,6 +153,8 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
   if constexpr (!MULTI) pdl_enter();
 
   if (a.win_reset && r == 0) empty_windows(a.win_reset, a.win_mt);
+  if (a.mask_reset && r == 0)
+    for (int i = tid; i < a.mask_words; i += NT) a.mask_reset[i] = 0u;
   RowScal rs = a.rs[r];
   if (a.err && *a.err) rs.status |= SED_ROW_DEVICE_TIMEOUT;
   const int ro = rs.orig;   // the caller's row index

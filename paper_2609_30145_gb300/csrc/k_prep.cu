@@ -361,6 +361,26 @@ constexpr int ORDER_CHUNK = 4096;
 constexpr int ORDER_THREADS = 1024;
 constexpr int ORDER_BINS = 1024;
 
+// The bracket pair of a row with one [Fe/H] (and [a/Fe]): its four blocks of W.
+__device__ __forceinline__ int row_pair(const ModelDev& md, const float* row) {
+  int j0, j1, n0 = 0, n1;
+  float w0, w1;
+  bracket_f(md.feh, md.n_feh, theta_col(md, row, md.offs[SED_KEY_LOGZSOL]), j0, w0, j1, w1);
+  if (md.use_afe && md.n_afe > 1) bracket_f(md.afe, md.n_afe, theta_col(md, row, md.offs[SED_KEY_AFE]), n0, w0, n1, w1);
+  return n0 * max(md.n_feh - 1, 1) + j0;
+}
+// Redshift ranges the bracket pairs are ordered within: two halves of the
+// launch's range, which keeps a tile's node window narrow, unless half the range
+// moves a row's window by less than a quarter of its width; one range then puts
+// half as many pairs into a tile (301 rows with z in [0.9, 1.3] on the [a/Fe]
+// grid: the call 117 -> 113 us).
+__device__ __forceinline__ int order_halves(const ModelDev& md, float zlo, float zhi) {
+  float width = 0.f;
+  if (md.n_filt > 0) width = logf(md.samp_lam_max / md.samp_lam_min);
+  if (md.n_pix > 0) width = fmaxf(width, (float)(md.pix_ln_max - md.pix_ln_min));
+  return 0.5f * logf((1.f + zhi) / (1.f + zlo)) < 0.25f * width ? 1 : 2;
+}
+
 struct OrderArgs {
   const float* theta;
   int n, ld;
@@ -424,10 +444,11 @@ __global__ void __launch_bounds__(ORDER_THREADS) k_order(const __grid_constant__
     if (lane == 0) { atomicMin(&s_zlo, lo); atomicMax(&s_zhi, hi); }
   }
   __syncthreads();
-  // bins over the chunk's own redshift range: by_pair, two halves of it, the
-  // bracket pair, then fine redshift bins; else fine redshift bins only
+  // bins over the chunk's own redshift range: by_pair, its halves (or all of it),
+  // the bracket pair, then fine redshift bins; else fine redshift bins only
   const float zlo = __int_as_float(s_zlo), zr = fmaxf(__int_as_float(s_zhi) - zlo, 1e-6f);
-  const int nf = oa.by_pair ? ORDER_BINS / (2 * oa.n_pairs) : ORDER_BINS;
+  const int halves = oa.by_pair ? order_halves(md, zlo, zlo + zr) : 1;
+  const int nf = oa.by_pair ? ORDER_BINS / (halves * oa.n_pairs) : ORDER_BINS;
   const float fscale = (float)nf / zr;
 #pragma unroll
   for (int u = 0; u < PER; ++u) {
@@ -438,13 +459,8 @@ __global__ void __launch_bounds__(ORDER_THREADS) k_order(const __grid_constant__
       if (z >= 0.f) {
         int b = min(nf - 1, (int)((z - zlo) * fscale));
         if (oa.by_pair) {
-          const float* row = oa.theta + (size_t)(base + i) * oa.ld;
-          int j0, j1, n0 = 0, n1;
-          float w0, w1;
-          bracket_f(md.feh, md.n_feh, theta_col(md, row, md.offs[SED_KEY_LOGZSOL]), j0, w0, j1, w1);
-          if (md.use_afe && md.n_afe > 1) bracket_f(md.afe, md.n_afe, theta_col(md, row, md.offs[SED_KEY_AFE]), n0, w0, n1, w1);
-          const int half = (z - zlo) * 2.f >= zr ? 1 : 0;
-          b += (half * oa.n_pairs + n0 * max(md.n_feh - 1, 1) + j0) * nf;
+          const int half = halves == 2 && (z - zlo) * 2.f >= zr ? 1 : 0;
+          b += (half * oa.n_pairs + row_pair(md, oa.theta + (size_t)(base + i) * oa.ld)) * nf;
         }
         bin[u] = b;
       } else {
@@ -492,6 +508,9 @@ constexpr int PREP_KWARPS = PREP_THREADS / 32 - 1;   // warps writing W; the las
 // Largest launch that orders itself (PrepArgs::self_order): each CTA reads
 // every row's redshift, so the cost grows with n^2
 constexpr int SELF_ORDER_MAX = 1024;
+// ... and one with K-tile masks, whose keys hold two brackets per row (301 rows
+// on the [a/Fe] grid: the call 134 us ordering itself, 113 us with k_order)
+constexpr int SELF_PAIR_MAX = 128;
 static_assert(SELF_ORDER_MAX <= 2 * MAX_SFH + 1, "the redshifts are staged in the edge and rate arrays");
 
 // Row p of the launch processes the caller's row r = perm[p] and records r in
@@ -501,7 +520,7 @@ static_assert(SELF_ORDER_MAX <= 2 * MAX_SFH + 1, "the redshifts are staged in th
 // counting the rows whose (redshift bin, index) key is below its own (stable
 // counting sort over the same bins; every CTA forms the same keys).
 template <bool MULTI>
-__global__ void __launch_bounds__(PREP_THREADS) k_prep(const __grid_constant__ PrepKernelArgs ka) {
+__global__ void __launch_bounds__(PREP_THREADS, 8) k_prep(const __grid_constant__ PrepKernelArgs ka) {
   const PrepArgs& a = ka.p;
   pdl_enter();
   const int b = blockIdx.x;
@@ -525,6 +544,7 @@ __global__ void __launch_bounds__(PREP_THREADS) k_prep(const __grid_constant__ P
   float* T = s_trate;
   float* rate = s_trate + MAX_SFH + 1;
   __shared__ int s_pos;
+  __shared__ uint8_t s_pair[SELF_PAIR_MAX];   // self-ordered launch with K-tile masks: the rows' bracket pairs
   __shared__ int zb[MAX_SFH];
   __shared__ float zt[MAX_SFH];
   __shared__ float s_red[PREP_THREADS / 32];
@@ -560,30 +580,41 @@ __global__ void __launch_bounds__(PREP_THREADS) k_prep(const __grid_constant__ P
     const TmaxRow t = row_tmax(md, theta_col(md, th, md.offs[SED_KEY_ZRED]), theta_col(md, th, md.offs[SED_KEY_LOGMASS]));
     if (lane == 0) { s_tmax = t.tmax; s_lrat = t.lrat; s_zst = t.status; }
   } else if (rank_warp) {
-    // the row's place in the redshift order: the valid redshifts (z in
-    // [0, z_f), others -1) and their range, then the keys of k_order's bins
-    // over that range (invalid rows in the last bin) and the count of rows
-    // whose (key, index) is below this row's
+    // the row's place in the launch's order: the valid redshifts (z in [0, z_f),
+    // others -1) and their range, then the keys of k_order's bins over that range
+    // (invalid rows in the last bin) and the count of rows whose (key, index) is
+    // below this row's
     float* zs = s_trate;
     const int zoff = md.offs[SED_KEY_ZRED];
     int lo = 0x7f7fffff, hi = 0;
 #pragma unroll 8
     for (int j = lane; j < a.n; j += 32) {
-      const float z = a.theta[(size_t)j * a.ld + zoff];
+      const float z = theta_col(md, a.theta + (size_t)j * a.ld, zoff);
       const float zv = z >= 0.f && z < (float)md.zf ? z : -1.f;
       zs[j] = zv;
       if (zv >= 0.f) { lo = min(lo, __float_as_int(zv)); hi = max(hi, __float_as_int(zv)); }
     }
+    if (a.by_pair)
+#pragma unroll 4
+      for (int j = lane; j < a.n; j += 32) s_pair[j] = (uint8_t)row_pair(md, a.theta + (size_t)j * a.ld);
     lo = __reduce_min_sync(0xffffffffu, lo);
     hi = __reduce_max_sync(0xffffffffu, hi);
     __syncwarp();
     const float zlo = __int_as_float(lo), zr = fmaxf(__int_as_float(hi) - zlo, 1e-6f);
-    const float fscale = (float)ORDER_BINS / zr;
-    auto key = [&](float z) { return z >= 0.f ? min(ORDER_BINS - 1, (int)((z - zlo) * fscale)) : ORDER_BINS; };
-    const int kb = key(zs[b]);
+    const int halves = a.by_pair ? order_halves(md, zlo, zlo + zr) : 1;
+    const int nf = a.by_pair ? ORDER_BINS / (halves * a.n_pairs) : ORDER_BINS;
+    const float fscale = (float)nf / zr;
+    auto key = [&](int j) {
+      const float z = zs[j];
+      if (!(z >= 0.f)) return ORDER_BINS;
+      int k = min(nf - 1, (int)((z - zlo) * fscale));
+      if (a.by_pair) k += ((halves == 2 && (z - zlo) * 2.f >= zr ? a.n_pairs : 0) + s_pair[j]) * nf;
+      return k;
+    };
+    const int kb = key(b);
     int below = 0;
     for (int j = lane; j < a.n; j += 32) {
-      const int kj = key(zs[j]);
+      const int kj = key(j);
       below += kj < kb || (kj == kb && j < b);
     }
     below = __reduce_add_sync(0xffffffffu, below);
@@ -1007,6 +1038,8 @@ constexpr int PREP_BWD_THREADS = 128;
 template <bool LINEAR>
 __global__ void __launch_bounds__(PREP_BWD_THREADS) k_prep_bwd(const __grid_constant__ PrepBwdArgs a) {
   pdl_enter();
+  if (a.mask_reset && blockIdx.x == 0)   // their last reader, the adjoint contraction, has finished
+    for (int i = threadIdx.x; i < a.mask_words; i += PREP_BWD_THREADS) a.mask_reset[i] = 0u;
   const ModelDev& md = a.md;
   const GridDev& g = a.g;
   const LayoutDev& L = a.L;
@@ -1240,15 +1273,21 @@ cudaError_t launch_prep_bwd(const PrepBwdArgs& p, cudaStream_t s) {
 
 cudaError_t launch_prep(const PrepArgs& p, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
-  // a fixed redshift (no column) needs no redshift order: the caller's order is kept
+  // a fixed redshift (no column) needs no redshift order, but rows of K-tile masks
+  // are ordered by their bracket pair all the same; else the caller's order is kept
   const bool z_col = p.md.offs[SED_KEY_ZRED] < p.md.n_param;
   const int mt = (p.n + 127) / 128;
-  // a small single-fit launch without K-tile masks orders itself; its windows
-  // start empty because the last kernel of every call that filled them (the
-  // epilogue) empties them again, and the workspace starts them empty
-  const bool self = p.self_order && z_col && !p.row_model && !p.kmask && p.n <= SELF_ORDER_MAX;
-  const bool order = !self && p.perm && (p.row_model || z_col);
-  if (!order && !self) {   // no ordering kernel to start the windows and masks empty
+  // bracket pair major when the contraction skips K tiles (the host gives
+  // masks only to models with one [Fe/H], and [a/Fe], per row)
+  const int pairs = std::max(p.md.n_feh - 1, 1) * (p.md.use_afe ? std::max(p.md.n_afe - 1, 1) : 1);
+  const bool by_pair = !p.row_model && p.kmask && pairs > 1 && pairs <= ORDER_BINS / 4;
+  const bool ordered = p.row_model || z_col || by_pair;
+  // a small single-fit launch orders itself; its windows and masks start empty
+  // because the last kernel of every call that filled them empties them again,
+  // and the workspace starts them empty
+  const bool self = ordered && p.self_order && !p.row_model && p.n <= (by_pair ? SELF_PAIR_MAX : SELF_ORDER_MAX);
+  const bool order = ordered && !self && p.perm;
+  if (!order && !p.self_order) {   // nothing before this kernel to start the windows and masks empty
     if (p.tile_win) {
       e = cudaMemsetAsync(p.tile_win, 0x7f, mt * sizeof(int), s);
       if (e == cudaSuccess) e = cudaMemsetAsync(p.tile_win + mt, 0xff, mt * sizeof(int), s);
@@ -1260,10 +1299,7 @@ cudaError_t launch_prep(const PrepArgs& p, cudaStream_t s) {
     OrderArgs oa;
     oa.theta = p.theta; oa.n = p.n; oa.ld = p.ld; oa.perm = p.perm; oa.md = p.md;
     oa.mtab = p.mtab; oa.row_model = p.row_model;
-    // bracket pair major when the contraction skips K tiles (the host gives
-    // masks only to models with one [Fe/H], and [a/Fe], per row)
-    const int pairs = std::max(p.md.n_feh - 1, 1) * (p.md.use_afe ? std::max(p.md.n_afe - 1, 1) : 1);
-    oa.by_pair = !p.row_model && p.kmask && pairs > 1 && pairs <= ORDER_BINS / 4;
+    oa.by_pair = by_pair;
     oa.n_pairs = pairs;
     oa.tile_win = p.tile_win;
     oa.kmask = p.kmask;
@@ -1275,7 +1311,9 @@ cudaError_t launch_prep(const PrepArgs& p, cudaStream_t s) {
   PrepKernelArgs ka;
   ka.p = p;
   ka.p.self_order = self ? 1 : 0;
-  if (self || (!p.row_model && !z_col)) ka.p.perm = nullptr;
+  ka.p.by_pair = by_pair ? 1 : 0;
+  ka.p.n_pairs = pairs;
+  if (!order) ka.p.perm = nullptr;
   // Ws [n_age][n_feh], the FP8 row scratch, the row's parameters (n_param <= ld
   // and n_param <= 2 MAX_SFH + SED_NKEYS + 2 MAX_DUST_BIN for every model)
   // (+ the fixed keys' values past the caller's columns)

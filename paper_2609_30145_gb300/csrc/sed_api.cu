@@ -1370,11 +1370,12 @@ sed::Workspace* get_ws(sed_ctx* ctx, void* stream, int rows, int kpad, int ldn, 
     AL(dW, R * K * 4); AL(rgrad, R * RGRAD * 8);
   }
 #undef AL
-  if (!s) {   // the error words cleared, the per-tile windows empty (k_prep's self-ordered launches expect it)
+  if (!s) {   // the error words cleared, the per-tile windows and masks empty (k_prep expects it)
     cudaError_t e = cudaMemset(w->err, 0, 64);
     const size_t mt = (R + 127) / 128;
     if (e == cudaSuccess) e = cudaMemset(w->tile_win, 0x7f, mt * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(w->tile_win + mt, 0xff, mt * sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(w->kmask, 0, mt * KMASK_WORDS * sizeof(uint32_t));
     if (e != cudaSuccess) s = fail(ctx, SED_ECUDA, "cudaMemset: %s", cudaGetErrorString(e));
   }
   *st = s;
@@ -1510,6 +1511,16 @@ sed_status run_forward_core(sed_ctx* ctx, Model* M, Workspace* w, const float* t
   return prof_mark(ctx, w, 2, s);
 }
 
+// The per-tile windows and K-tile masks, read by the contraction, are emptied
+// by the epilogue for the next call.
+void reset_after(EpiArgs& ea, Workspace* w, int n) {
+  const int mt = (n + 127) / 128;
+  ea.win_reset = w->tile_win;
+  ea.win_mt = mt;
+  ea.mask_reset = w->kmask_w_call > 0 ? w->kmask : nullptr;
+  ea.mask_words = mt * w->kmask_w_call;
+}
+
 int ldn_for(const Grid* g) { return (g->n_lam + 255) / 256 * 256; }
 
 }  // namespace
@@ -1535,7 +1546,7 @@ sed_status sed_forward(sed_ctx* ctx, sed_model_id id, const float* theta, int n,
   ea.md = M->dv; ea.g = grid_view(M->g);
   ea.seg_stride = (size_t)w->cap_rows * w->ldn;
   ea.qneb = M->dv.use_neb && M->g->neb_na > 0 ? w->qneb : nullptr;
-  ea.win_reset = w->tile_win; ea.win_mt = (n + 127) / 128;   // read by the contraction, emptied for the next call
+  reset_after(ea, w, n);
   ea.lam8 = precision == SED_PREC_FP8 ? M->L->lam8 : nullptr;
   ea.phot_out = M->dv.n_filt ? phot_out : nullptr;
   ea.spec_out = M->dv.n_pix ? spec_out : nullptr;
@@ -1565,7 +1576,7 @@ sed_status sed_line_fluxes(sed_ctx* ctx, sed_model_id id, const float* theta, in
   ea.md = M->dv; ea.g = grid_view(M->g);
   ea.seg_stride = (size_t)w->cap_rows * w->ldn;
   ea.qneb = M->dv.use_neb && M->g->neb_na > 0 ? w->qneb : nullptr;
-  ea.win_reset = w->tile_win; ea.win_mt = (n + 127) / 128;   // read by the contraction, emptied for the next call
+  reset_after(ea, w, n);
   ea.lam8 = precision == SED_PREC_FP8 ? M->L->lam8 : nullptr;
   ea.lines_out = flux_out;
   ea.err = w->err;
@@ -1594,7 +1605,7 @@ static sed_status loglike_impl(sed_ctx* ctx, sed_model_id id, const float* theta
   ea.md = M->dv; ea.g = grid_view(M->g);
   ea.seg_stride = (size_t)w->cap_rows * w->ldn;
   ea.qneb = M->dv.use_neb && M->g->neb_na > 0 ? w->qneb : nullptr;
-  ea.win_reset = w->tile_win; ea.win_mt = (n + 127) / 128;   // read by the contraction, emptied for the next call
+  reset_after(ea, w, n);
   ea.lnl = lnl_out; ea.status = row_status; ea.err = w->err;
   ea.lam8 = precision == SED_PREC_FP8 ? M->L->lam8 : nullptr;
   CK(launch_epilogue(ea, s));
@@ -1757,6 +1768,8 @@ sed_status sed_loglike_grad(sed_ctx* ctx, sed_model_id id, const float* theta, i
   pb.theta = theta; pb.n = n; pb.ld = ld;
   pb.md = M->dv; pb.g = g->dv; pb.L = L->dv();
   pb.rs = w->rs; pb.dW = w->dW; pb.rgrad = w->rgrad; pb.grad = grad_out;
+  pb.mask_reset = w->kmask_w_call > 0 ? w->kmask : nullptr;
+  pb.mask_words = (n + 127) / 128 * w->kmask_w_call;
   CK(launch_prep_bwd(pb, s));
   return prof_mark(ctx, w, 3, s);
 }
@@ -1802,11 +1815,16 @@ sed_status sed_last_stats(sed_ctx* ctx, void* stream, sed_stage_stats* out) {
     // K columns each 128-row tile multiplies: its touched K tiles when the call skipped the others
     std::vector<double> kcols((rs.size() + 127) / 128, (double)w->last_kpad);
     if (w->last_kmask_w > 0 && !simt) {
-      std::vector<uint32_t> km(kcols.size() * w->last_kmask_w);
-      CK(cudaMemcpy(km.data(), w->kmask, km.size() * 4, cudaMemcpyDeviceToHost));
+      // the tile masks themselves are emptied after the call: the union of the rows' own
+      std::vector<uint32_t> km(rs.size() * KMASK_WORDS);
+      CK(cudaMemcpy(km.data(), w->wmask, km.size() * 4, cudaMemcpyDeviceToHost));
       for (size_t t = 0; t < kcols.size(); ++t) {
         int bits = 0;
-        for (int j = 0; j < w->last_kmask_w; ++j) bits += __builtin_popcount(km[t * w->last_kmask_w + j]);
+        for (int j = 0; j < w->last_kmask_w; ++j) {
+          uint32_t m = 0;
+          for (size_t r = t * 128; r < std::min(rs.size(), t * 128 + 128); ++r) m |= km[r * KMASK_WORDS + j];
+          bits += __builtin_popcount(m);
+        }
         kcols[t] = (double)bits * (1 << w->last_kt_shift);
       }
     }

@@ -477,10 +477,10 @@ struct PrepArgs {
                        // non-zeros from before (read) and that hold them now (written); the row's
                        // other tiles are zeros and are not written.  NULL: every column written
   float* qneb;         // nebular age axis: [n][MAX_NEB_AGE] Q-weighted weight of each nebular SSP age, or NULL
-  int self_order;      // 1: the prep kernel finds each row's place in the redshift order itself (no
-                       // k_order launch) where launch_prep allows it: one fit, no K-tile masks, a
-                       // redshift column, n <= SELF_ORDER_MAX, theta in device memory (each CTA
-                       // reads every row's redshift), and tile_win already empty
+  int self_order;      // 1: tile_win and kmask are already empty, and the prep kernel may find each
+                       // row's place in the order itself (no k_order launch): theta in device memory
+                       // (each CTA reads every row's keys); done for one fit of n <= SELF_ORDER_MAX
+  int by_pair, n_pairs;   // set by launch_prep: rows ordered by bracket pair, and the pairs there are
 };
 // Per-tile windows (lo, hi) of the contraction back to empty (lo 0x7f7f7f7f,
 // hi -1) once their reader has finished, by one CTA, so that the next call's
@@ -661,6 +661,8 @@ struct EpiArgs {
   const float* qneb;   // nebular age axis: [n][MAX_NEB_AGE] (k_prep's), or NULL
   int* win_reset;      // [2][win_mt] per-tile windows set back to empty by CTA 0 (the contraction,
   int win_mt;          // their reader, has finished), or NULL
+  uint32_t* mask_reset;   // the K-tile masks likewise, mask_words of them
+  int mask_words;
 };
 cudaError_t launch_epilogue(const EpiArgs& a, cudaStream_t s);
 
@@ -703,6 +705,8 @@ struct PrepBwdArgs {
   const RowScal* rs;
   const float* dW; const double* rgrad;
   float* grad;          // [n][ld]
+  uint32_t* mask_reset; // K-tile masks (mask_words of them) set back to empty, or NULL
+  int mask_words;
 };
 cudaError_t launch_prep_bwd(const PrepBwdArgs& a, cudaStream_t s);
 
