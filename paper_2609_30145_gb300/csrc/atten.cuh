@@ -25,6 +25,13 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
+// e^(-u^2/2) (2^x by the hardware; used for u^2 <= 25, far from the subnormals)
+__device__ __forceinline__ float gauss_w(float u2) {
+  float w;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(w) : "f"(u2 * (-0.5f * 1.4426950408889634f)));
+  return w;
+}
+
 __device__ __forceinline__ float dust_shape(const ModelDev& md, const float4& c, float eb, float pw) {
   return md.dust_law == SED_DUST_POWER_LAW ? pw : (c.y + eb * c.z) * pw;
 }

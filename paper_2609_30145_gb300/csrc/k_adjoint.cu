@@ -31,6 +31,8 @@
 // it, and accumulates dlnL/dF in shared memory.  Every sum runs in a fixed
 // order (node-owned gathers, no atomics), so the gradient is bitwise
 // reproducible.
+#include <type_traits>
+
 #include "atten.cuh"
 #include "calib.cuh"
 #include "floor.cuh"
@@ -72,11 +74,16 @@ __device__ __forceinline__ void put_g(const EpiBwdArgs& a, float* hi, float* lo,
 constexpr size_t EB_CAL_BYTES = (size_t)EB_WARPS * CAL_NV * sizeof(float) +
                                 (size_t)(SED_MAX_CALIB * SED_MAX_CALIB + 2 * SED_MAX_CALIB) * sizeof(float);
 
+// bytes of the pixels' arrays: 4 floats + node range; with a sampled stellar
+// dispersion also dmu/ds; with a calibration polynomial mu/sigma, dmu/dx, dmu/ds, 1/sum w
+__host__ __device__ __forceinline__ size_t epi_bwd_pix(const ModelDev& md) {
+  return (size_t)md.n_pix * (md.calib_n ? 36 : md.sample_sgal ? 24 : 20);
+}
+
 size_t epi_bwd_lines_off(const EpiBwdArgs& a) {   // bytes, 8-aligned
   const size_t W = (size_t)a.md.win_max;
   const size_t samp = (size_t)a.md.n_samp * 8;    // node index + interpolation weight
-  // 4 floats + node range; with a calibration polynomial also mu/sigma, dmu/dx, dmu/ds, 1/sum w
-  const size_t pix = (size_t)a.md.n_pix * (a.md.calib_n ? 36 : 20);
+  const size_t pix = epi_bwd_pix(a.md);
   const size_t u = ((samp > pix ? samp : pix) + 7) & ~(size_t)7;
   return ((((2 * W + 3) & ~(size_t)3) * sizeof(float) + u + (a.md.calib_n ? EB_CAL_BYTES : 0)) + 7) & ~(size_t)7;
 }
@@ -144,11 +151,11 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
   // 1/sum w, then the per-warp moments, the Cholesky factor and c*
   float* mu_s = reinterpret_cast<float*>(prg + md.n_pix);
   float* dv_s = mu_s + md.n_pix;
-  float* dvs_s = dv_s + md.n_pix;
-  float* cw_s = dvs_s + md.n_pix;
+  float* dvs_s = md.calib_n ? dv_s + md.n_pix : mu_s;
+  float* cw_s = dv_s + 2 * md.n_pix;
   float *cal_part = nullptr, *cal_Lf = nullptr, *cal_Df = nullptr, *cal_cf = nullptr;
   if (md.calib_n) {
-    const size_t samp = (size_t)md.n_samp * 8, pix = (size_t)md.n_pix * 36;
+    const size_t samp = (size_t)md.n_samp * 8, pix = epi_bwd_pix(md);
     const size_t u = ((samp > pix ? samp : pix) + 7) & ~(size_t)7;
     cal_part = reinterpret_cast<float*>(reinterpret_cast<char*>(U) + u);
     cal_Lf = reinterpret_cast<float*>(cal_part + EB_WARPS * CAL_NV);
@@ -348,7 +355,10 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
   for (int k = kr0; k < kr1; ++k) phi[k] *= g.inv_lam2[k];
   __syncthreads();
 
-  // ---- spectrum forward (thread per pixel): m_i, u_i, each pixel's node range.
+  // ---- spectrum forward: m_i, its derivatives in x and s and each pixel's node
+  //      range.  Two neighbouring pixels per thread share each node's loads, as
+  //      in the forward epilogue (the loop is bound by instruction issue).  What the
+  //      pixel's terms need waits in its place of px4 for the thread that sums them.
   //      A Gaussian row's range comes from the index table alone (a superset of
   //      the nodes within 5 sigma, clamped to the window): the |u| <= 5 test
   //      decides which nodes enter the sums.
@@ -357,78 +367,108 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
   double l_spec = 0.0, um_spec = 0.0;
   float chi = 0.f, um_f = 0.f, gz_spec = 0.f, g_sgal = 0.f;
   float gfs[4] = {0.f, 0.f, 0.f, 0.f};   // d lnL / d log10 of the spectral noise-floor terms
-  const float ll0 = g.lnl_hi[0], llN = g.lnl_hi[N - 1];
-  for (int i = tid; i < md.n_pix; i += EB_THREADS) {
-    float xh, xl;
-    ln_rest(md.pix_ln2[i], rs.ln1pz_hi, rs.ln1pz_lo, xh, xl);
-    // total dispersion: fixed, or sigma_fix composed with the row's sigma_gal (Eq. one_kernel)
-    const float s = md.sample_sgal ? sqrtf(md.pix_fix2[i] + rs.sg_ln * rs.sg_ln) : md.pix_s[i];
-    float v = 0.f, dv = 0.f, dvs = 0.f, cw = 0.f, tl = 0.f;
-    // node range of the pixel; outside the grid a one-node range at the
-    // window's edge keeps the ranges in pixel order (the pixel has c = 0)
-    int jlo = xh < ll0 ? k_lo : k_hi, jhi = jlo;
-    bool valid = false;
-    if (xh >= ll0 && xh <= llN) {
-      const int k = locate_ln(g, xh, g.lnl_hi);
-      const float dln = (g.lnl_hi[k + 1] - g.lnl_hi[k]) + (g.lnl_lo[k + 1] - g.lnl_lo[k]);
-      if (s < 0.5f * dln) {
-        const float t = ((xh - g.lnl_hi[k]) + (xl - g.lnl_lo[k])) / dln;
-        v = Fs[k] + t * (Fs[k + 1] - Fs[k]);
-        dv = (Fs[k + 1] - Fs[k]) / dln;
-        valid = true;
-        jlo = k; jhi = k + 1; tl = t; cw = 1.f;
-      } else {
-        const float inv_s = 1.f / s;
-        int qa = (int)((fmaxf(xh - 5.f * s, ll0) - g.lut_x0) * g.lut_inv_h);
-        int qb = (int)((fminf(xh + 5.f * s, llN) - g.lut_x0) * g.lut_inv_h);
-        qa = min(max(qa, 0), g.lut_n - 1);
-        qb = min(max(qb, 0), g.lut_n - 1);
-        jlo = max(g.lut[qa] - 1, k_lo);
-        jhi = min(g.lut[qb] + 3, k_hi);
-        // a node past 5 dispersions weighs exactly 0 (its terms add zeros), so
-        // the loop carries no branch and its loads pipeline
-        float sw = 0.f, sf = 0.f, swd = 0.f, sfd = 0.f, sws = 0.f, sfs = 0.f;
-        if (md.sample_sgal) {
-#pragma unroll 4
-          for (int j = jlo; j <= jhi; ++j) {
-            const float d = (g.lnl_hi[j] - xh) + (g.lnl_lo[j] - xl);
-            const float u = d * inv_s;
-            const float w = fabsf(u) <= 5.f ? __expf(-0.5f * u * u) : 0.f;
-            const float wd = w * u * inv_s;   // dw/dx
-            const float ws = wd * u;          // dw/ds = w u^2 / s
-            const float f = Fs[j];
-            sw += w;
-            sf = fmaf(w, f, sf);
-            swd += wd;
-            sfd = fmaf(wd, f, sfd);
-            sws += ws;
-            sfs = fmaf(ws, f, sfs);
+  if (md.n_pix > 0) {
+    const float ll0 = g.lnl_hi[0], llN = g.lnl_hi[N - 1];
+    const int last = md.n_pix - 1;
+    for (int ib = 2 * 32 * warp; ib < md.n_pix; ib += 2 * EB_THREADS) {
+      float2 pl[2];
+      float xh[2], xl[2], inv_s[2], v[2], dv[2], dvs[2], cw[2], tl[2];
+      float sw[2], sf[2], swu[2], sfu[2], swq[2], sfq[2];
+      int jlo[2], jhi[2];
+      int jl = k_hi, jh = k_lo - 1;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int i = min(ib + 2 * lane + q, last);
+        pl[q] = md.pix_ln2[i];
+        ln_rest(pl[q], rs.ln1pz_hi, rs.ln1pz_lo, xh[q], xl[q]);
+        v[q] = dv[q] = dvs[q] = cw[q] = tl[q] = inv_s[q] = 0.f;
+        sw[q] = sf[q] = swu[q] = sfu[q] = swq[q] = sfq[q] = 0.f;
+        // node range of the pixel; outside the grid a one-node range at the
+        // window's edge keeps the ranges in pixel order (the pixel has c = 0)
+        jlo[q] = jhi[q] = xh[q] < ll0 ? k_lo : k_hi;
+        if (xh[q] >= ll0 && xh[q] <= llN) {
+          // total dispersion: fixed, or sigma_fix composed with the row's sigma_gal (Eq. one_kernel)
+          const float s = md.sample_sgal ? sqrtf(md.pix_fix2[i] + rs.sg_ln * rs.sg_ln) : md.pix_s[i];
+          const int k = locate_ln(g, xh[q], g.lnl_hi);
+          const float2 n0 = __ldg(g.lnl2 + k), n1 = __ldg(g.lnl2 + k + 1);
+          const float dln = (n1.x - n0.x) + (n1.y - n0.y);
+          if (s < 0.5f * dln) {
+            const float t = ((xh[q] - n0.x) + (xl[q] - n0.y)) / dln;
+            v[q] = Fs[k] + t * (Fs[k + 1] - Fs[k]);
+            dv[q] = (Fs[k + 1] - Fs[k]) / dln;
+            jlo[q] = k;
+            jhi[q] = k + 1;
+            tl[q] = t;
+            cw[q] = 1.f;
+          } else {
+            inv_s[q] = 1.f / s;
+            int qa = (int)((fmaxf(xh[q] - 5.f * s, ll0) - g.lut_x0) * g.lut_inv_h);
+            int qb = (int)((fminf(xh[q] + 5.f * s, llN) - g.lut_x0) * g.lut_inv_h);
+            qa = min(max(qa, 0), g.lut_n - 1);
+            qb = min(max(qb, 0), g.lut_n - 1);
+            jlo[q] = max(g.lut[qa] - 1, k_lo);
+            jhi[q] = min(g.lut[qb] + 3, k_hi);
+            jl = min(jl, jlo[q]);
+            jh = max(jh, jhi[q]);
+            tl[q] = -1.f - inv_s[q];
           }
-        } else {
-#pragma unroll 4
-          for (int j = jlo; j <= jhi; ++j) {
-            const float d = (g.lnl_hi[j] - xh) + (g.lnl_lo[j] - xl);
-            const float u = d * inv_s;
-            const float w = fabsf(u) <= 5.f ? __expf(-0.5f * u * u) : 0.f;
-            const float wd = w * u * inv_s;   // dw/dx
-            const float f = Fs[j];
-            sw += w;
-            sf = fmaf(w, f, sf);
-            swd += wd;
-            sfd = fmaf(wd, f, sfd);
-          }
-        }
-        tl = -1.f - inv_s;
-        if (sw > 0.f) {
-          v = sf / sw;
-          dv = (sfd * sw - sf * swd) / (sw * sw);
-          dvs = (sfs * sw - sf * sws) / (sw * sw);
-          valid = true;
-          cw = 1.f / sw;
         }
       }
+      // sums of w, w F, w u, w u F and, with a sampled dispersion, w u^2, w u^2 F
+      // (dw/dx = w u / s, dw/ds = w u^2 / s); a node past 5 dispersions is left out
+      // by predication, so the loop carries no branch (its loads pipeline)
+      auto add_nodes = [&](auto sgal) {
+#pragma unroll 4
+        for (int j = jl; j <= jh; ++j) {
+          const float2 n = __ldg(g.lnl2 + j);
+          const float f = Fs[j];
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            const float u = ((n.x - xh[q]) + (n.y - xl[q])) * inv_s[q];
+            const float w = gauss_w(u * u), wu = w * u;
+            if (fabsf(u) <= 5.f) {
+              sw[q] += w;
+              sf[q] = fmaf(w, f, sf[q]);
+              swu[q] += wu;
+              sfu[q] = fmaf(wu, f, sfu[q]);
+              if (sgal) {
+                const float wq = wu * u;
+                swq[q] += wq;
+                sfq[q] = fmaf(wq, f, sfq[q]);
+              }
+            }
+          }
+        }
+      };
+      if (md.sample_sgal) add_nodes(std::true_type{}); else add_nodes(std::false_type{});
+      float la[2] = {0.f, 0.f};
+      if (LINES && NLn)
+        lines_at_pixels(NLn, ln_A, ln_is, ln_x, pl[0], pl[1], __shfl_sync(0xffffffffu, pl[0].x, 0),
+                        __shfl_sync(0xffffffffu, pl[1].x, 31), lane, la[0], la[1]);
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int i = ib + 2 * lane + q;
+        if (i > last) break;
+        if (tl[q] < -0.5f && sw[q] > 0.f) {
+          const float n = inv_s[q] / (sw[q] * sw[q]);
+          v[q] = sf[q] / sw[q];
+          dv[q] = (sfu[q] * sw[q] - sf[q] * swu[q]) * n;
+          dvs[q] = (sfq[q] * sw[q] - sf[q] * swq[q]) * n;
+          cw[q] = 1.f / sw[q];
+        }
+        px4[i] = make_float4(v[q], dv[q], cw[q], tl[q]);
+        if (md.sample_sgal) dvs_s[i] = dvs[q];
+        if (LINES && NLn) upx[i] = la[q] * md.pix_lamc[i];
+        prg[i] = (jlo[q] & 0xffff) | (jhi[q] << 16);
+      }
     }
-    const float mline = LINES && NLn ? lines_at_pixel(md, i, NLn, ln_A, ln_is, ln_x) : 0.f;
+    __syncthreads();
+  }
+  for (int i = tid; i < md.n_pix; i += EB_THREADS) {
+    const float4 pv = px4[i];   // {v, dv/dx, 1/sum w (0: no node reached), t or -1 - 1/sigma}
+    const float v = pv.x, dv = pv.y, cw = pv.z, tl = pv.w, dvs = md.sample_sgal ? dvs_s[i] : 0.f;
+    const bool valid = cw != 0.f;
+    const float mline = LINES && NLn ? upx[i] : 0.f;
     const float mi = LINES && NLn ? fmaf(rs.s_spec, v, mline) : rs.s_spec * v;
     float ci = 0.f;
     const float isf = md.spec_isf[i];
@@ -464,11 +504,15 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
       const float us = wsn * (isf * rs.s_spec);
       gz_spec += us * dv * (-rs.inv1pz);
       // s = sqrt(sigma_fix^2 + sigma_gal^2) / c: ds/dsigma_gal = (sigma_gal / c) / (s c)
-      if (md.sample_sgal && s > 0.f) g_sgal += us * dvs * (rs.sg_ln / (s * (float)C_KMS));
+      if (md.sample_sgal) {
+        const float s = sqrtf(md.pix_fix2[i] + rs.sg_ln * rs.sg_ln);
+        if (s > 0.f) g_sgal += us * dvs * (rs.sg_ln / (s * (float)C_KMS));
+      }
       ci = us * cw;
     }
     if (NLn && !md.calib_n) upx[i] = inc ? wsn : 0.f;   // sigma_i d lnL / d mu_i
-    prg[i] = (jlo & 0xffff) | (jhi << 16);
+    float xh, xl;
+    ln_rest(md.pix_ln2[i], rs.ln1pz_hi, rs.ln1pz_lo, xh, xl);
     px4[i] = make_float4(xh, xl, ci, tl);   // x_hi ascending in i: the pixels' wavelengths are strictly increasing
   }
   if (md.calib_n) {
@@ -547,67 +591,85 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
   //      pixel whose node range holds k.  When the ranges' ends ascend with the
   //      pixel (the usual case: wavelengths ascend and the dispersion varies
   //      slowly), those pixels are exactly [first p with hi_p >= k, last p with
-  //      lo_p <= k], two binary searches.  Otherwise they lie within R of
+  //      lo_p <= k], two binary searches.  A thread then takes two neighbouring nodes,
+  //      which share the searches, the pixels' loads and 1/sigma.  Otherwise they lie within R of
   //      ln(lam_k) in ln(lambda) (R = 5 sigma_max for Gaussian rows, one node
   //      spacing for linear ones), a run of the ascending pixel positions that is
   //      tested pixel by pixel.  Neighbouring threads take neighbouring nodes, so
   //      the searches and scans of a warp read nearby pixels.
   if (md.n_pix > 0) {
     const int P = md.n_pix;
-    int mono = 1;
+    int mono = 1, linear = 0;
+    for (int i = tid; i < P; i += EB_THREADS) linear |= px4[i].w > -0.5f && px4[i].z != 0.f;
     for (int i = tid + 1; i < P; i += EB_THREADS) {
       const int r0 = prg[i - 1], r1 = prg[i];
       if ((r1 & 0xffff) < (r0 & 0xffff) || (r1 >> 16) < (r0 >> 16)) mono = 0;
     }
     mono = __syncthreads_and(mono);
+    linear = __syncthreads_or(linear);
     const float R = 5.f * md.pix_s_max * 1.0001f + g.dln_max * 1.0001f + 1e-6f;
-    for (int k = k_lo + tid; k <= k_hi; k += EB_THREADS) {
-      const float lh = g.lnl_hi[k], ll = g.lnl_lo[k];
-      float acc = 0.f;
-      if (mono) {
-        int pa = 0, pe = P;
-        while (pa < pe) {
-          const int mid = (pa + pe) >> 1;
-          if ((prg[mid] >> 16) < k) pa = mid + 1; else pe = mid;
-        }
-        int pb = pa;
-        pe = P;
-        while (pb < pe) {
-          const int mid = (pb + pe) >> 1;
-          if ((prg[mid] & 0xffff) <= k) pb = mid + 1; else pe = mid;
-        }
-        // lo_p <= k <= hi_p for every p here; a pixel with c = 0 (excluded)
-        // adds an exact zero, so the loop carries no branch
+    for (int k0 = mono ? k_lo + 2 * tid : k_hi + 1; k0 <= k_hi; k0 += 2 * EB_THREADS) {
+      const int k1 = min(k0 + 1, k_hi);
+      const float2 n0 = __ldg(g.lnl2 + k0), n1 = __ldg(g.lnl2 + k1);
+      int pa = 0, pe = P;
+      while (pa < pe) {   // first pixel whose range ends at k0 or later
+        const int mid = (pa + pe) >> 1;
+        if ((prg[mid] >> 16) < k0) pa = mid + 1; else pe = mid;
+      }
+      int pb = pa;
+      pe = P;
+      while (pb < pe) {   // first pixel whose range begins past k1
+        const int mid = (pb + pe) >> 1;
+        if ((prg[mid] & 0xffff) <= k1) pb = mid + 1; else pe = mid;
+      }
+      // a pixel of [pa, pb) whose range holds only one of the two nodes lies past
+      // 5 dispersions of the other, and one with c = 0 (excluded) adds an exact
+      // zero, so the loop carries no branch
+      float acc0 = 0.f, acc1 = 0.f;
+      auto add_pixels = [&](auto any_linear) {
 #pragma unroll 4
         for (int p = pa; p < pb; ++p) {
           const float4 q = px4[p];
-          const float d = (lh - q.x) + (ll - q.y);
-          const float u = d * (-1.f - q.w);   // Gaussian row: 1/sigma = -1 - q.w
-          const float wg = fabsf(u) <= 5.f ? __expf(-0.5f * u * u) : 0.f;
-          const float wl = k == (prg[p] & 0xffff) ? 1.f - q.w : q.w;   // linear row: q.w = t in [0, 1]
-          acc = fmaf(q.z, q.w > -0.5f ? wl : wg, acc);
-        }
-      } else {
-        int p = 0, p1 = P;
-        while (p < p1) {
-          const int mid = (p + p1) >> 1;
-          if (px4[mid].x < lh - R) p = mid + 1; else p1 = mid;
-        }
-        for (; p < P; ++p) {
-          const float4 q = px4[p];
-          if (q.x >= lh + R) break;
-          const int rg = prg[p], lo = rg & 0xffff, hi = rg >> 16;
-          if (q.z == 0.f || k < lo || k > hi) continue;
-          float w;
-          if (q.w > -0.5f) {   // linear row
-            w = k == lo ? 1.f - q.w : q.w;
-          } else {              // Gaussian row, 1/sigma = -1 - q.w
-            const float d = (lh - q.x) + (ll - q.y);
-            const float u = d * (-1.f - q.w);
-            w = fabsf(u) <= 5.f ? __expf(-0.5f * u * u) : 0.f;
+          const float is = -1.f - q.w;   // Gaussian row: 1/sigma
+          const float u0 = ((n0.x - q.x) + (n0.y - q.y)) * is, u1 = ((n1.x - q.x) + (n1.y - q.y)) * is;
+          const float w0 = gauss_w(u0 * u0), w1 = gauss_w(u1 * u1);
+          if (any_linear && q.w > -0.5f) {   // linear row: q.w = t in [0, 1]
+            const int lo = prg[p] & 0xffff;
+            const float a1 = 1.f - q.w, a2 = q.w;
+            if (k0 == lo || k0 == lo + 1) acc0 = fmaf(q.z, k0 == lo ? a1 : a2, acc0);
+            if (k1 == lo || k1 == lo + 1) acc1 = fmaf(q.z, k1 == lo ? a1 : a2, acc1);
+          } else {
+            if (fabsf(u0) <= 5.f) acc0 = fmaf(q.z, w0, acc0);
+            if (fabsf(u1) <= 5.f) acc1 = fmaf(q.z, w1, acc1);
           }
-          acc = fmaf(q.z, w, acc);
         }
+      };
+      if (linear) add_pixels(std::true_type{}); else add_pixels(std::false_type{});
+      phi[k0] += acc0;
+      if (k1 > k0) phi[k1] += acc1;
+    }
+    for (int k = mono ? k_hi + 1 : k_lo + tid; k <= k_hi; k += EB_THREADS) {
+      const float lh = g.lnl_hi[k], ll = g.lnl_lo[k];
+      float acc = 0.f;
+      int p = 0, p1 = P;
+      while (p < p1) {
+        const int mid = (p + p1) >> 1;
+        if (px4[mid].x < lh - R) p = mid + 1; else p1 = mid;
+      }
+      for (; p < P; ++p) {
+        const float4 q = px4[p];
+        if (q.x >= lh + R) break;
+        const int rg = prg[p], lo = rg & 0xffff, hi = rg >> 16;
+        if (q.z == 0.f || k < lo || k > hi) continue;
+        float w;
+        if (q.w > -0.5f) {   // linear row
+          w = k == lo ? 1.f - q.w : q.w;
+        } else {              // Gaussian row, 1/sigma = -1 - q.w
+          const float d = (lh - q.x) + (ll - q.y);
+          const float u = d * (-1.f - q.w);
+          w = fabsf(u) <= 5.f ? __expf(-0.5f * u * u) : 0.f;
+        }
+        acc = fmaf(q.z, w, acc);
       }
       phi[k] += acc;
     }

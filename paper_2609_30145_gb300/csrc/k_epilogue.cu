@@ -106,12 +106,6 @@ __device__ __forceinline__ float lg2_approx(float x) {
   asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// e^(-u^2/2) (2^x by the hardware; used for u^2 <= 25, far from the subnormals)
-__device__ __forceinline__ float gauss_w(float u2) {
-  float w;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(w) : "f"(u2 * (-0.5f * 1.4426950408889634f)));
-  return w;
-}
 // four bytes of global memory to shared memory without a register (the thread
 // itself reads them after cp_async_wait_all)
 __device__ __forceinline__ void cp_async4(float* dst, const float* src) {
