@@ -87,20 +87,70 @@ __device__ __forceinline__ uint4 philox(uint4 c, uint32_t k0, uint32_t k1) {
 // uniform in (0, 1) from the top 24 bits
 __device__ __forceinline__ float u01(uint32_t x) { return ((float)(x >> 8) + 0.5f) * (1.0f / 16777216.0f); }
 
-__device__ __forceinline__ double lae(double a, double b) {   // ln(e^a + e^b)
-  if (a == -INFINITY) return b;
-  if (b == -INFINITY) return a;
-  const double m = fmax(a, b);
-  return m + log1p(exp(-fabs(a - b)));
+// Sum (or maximum) of v over the block's first RED_THREADS threads in a fixed
+// order, the result in every thread; red holds one value per warp.  (An FP64
+// instruction of a warp takes 16 cycles of the SM's pipe on this GPU, so that
+// all 32 warps of a block would wait for one another.)
+constexpr int RED_THREADS = 256;
+template <bool MAX>
+__device__ double block_reduce(double v, double* red) {
+  auto tree = [](double x, int o0) {
+    for (int o = o0; o; o >>= 1) {
+      const double w = __shfl_xor_sync(0xffffffffu, x, o);
+      x = MAX ? fmax(x, w) : x + w;
+    }
+    return x;
+  };
+  if (threadIdx.x < RED_THREADS) {
+    v = tree(v, 16);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    v = tree(red[threadIdx.x & (RED_THREADS / 32 - 1)], RED_THREADS / 64);
+    __syncwarp();
+    if (threadIdx.x == 0) red[0] = v;
+  }
+  __syncthreads();
+  v = red[0];
+  __syncthreads();
+  return v;
 }
+// the points of thread j's share of a reduction: j, j + RED_THREADS, ...
+__device__ __forceinline__ int red_start(int cnt) { return threadIdx.x < RED_THREADS ? (int)threadIdx.x : cnt; }
 
-// Skilling's update of ln Z and H for one removed point of weight ln w.
-__device__ __forceinline__ void add_point(NssState* st, double lnl, double lnw) {
-  if (lnl == -INFINITY) return;
-  const double lz = lae(st->lnZ, lnw + lnl);
-  const double h = exp(lnw + lnl - lz) * lnl + (st->lnZ == -INFINITY ? 0.0 : exp(st->lnZ - lz) * (st->H + st->lnZ)) - lz;
-  st->H = h;
-  st->lnZ = lz;
+// Skilling's update of ln Z and H for the removed points j < cnt of likelihood
+// lnl(j) and ln weight lnw(j), by the whole block at once.  Point by point it
+// is Z' = Z + w L and H' + ln Z' = (w L ln L + Z (H + ln Z)) / Z'; after all of
+// them, with every term scaled by the largest one, Z' = Z + sum w L and
+// H' + ln Z' = (Z (H + ln Z) + sum w L ln L) / Z'.  (One thread going through
+// the points waited on four FP64 exponentials or logarithms a point.)
+template <class Lnl, class Lnw>
+__device__ void add_points(NssState* st, int cnt, Lnl lnl, Lnw lnw, double* red) {
+  const double lz0 = st->lnZ, h0 = st->H;
+  double m = threadIdx.x == 0 ? lz0 : -INFINITY;
+  for (int j = red_start(cnt); j < cnt; j += RED_THREADS) m = fmax(m, lnw(j) + lnl(j));
+  m = block_reduce<true>(m, red);
+  if (m == -INFINITY) return;   // no point with a likelihood yet
+  double z = 0.0, u = 0.0;
+  if (threadIdx.x == 0 && lz0 > -INFINITY) {
+    z = exp(lz0 - m);
+    u = z * (h0 + lz0);
+  }
+  for (int j = red_start(cnt); j < cnt; j += RED_THREADS) {
+    const double l = lnl(j);
+    if (l == -INFINITY) continue;
+    const double e = exp(lnw(j) + l - m);
+    z += e;
+    u += e * l;
+  }
+  z = block_reduce<false>(z, red);
+  u = block_reduce<false>(u, red);
+  if (threadIdx.x == 0) {
+    const double lz = m + log(z);
+    st->lnZ = lz;
+    st->H = u / z - lz;
+  }
 }
 
 __global__ void k_nss_init(int n, int d, const double* lo, const double* hi, Live lv, NssState* st, uint32_t k0,
@@ -120,17 +170,35 @@ __global__ void k_nss_init(int n, int d, const double* lo, const double* hi, Liv
   lv.TH[i] = (float)(lo[j] + (double)u * (hi[j] - lo[j]));
 }
 
-// Ranks of lnL (ascending, ties broken by index) into ord[], one CTA.
-__device__ void rank_live(int n, const double* lnl_s, int* ord) {
+// A double's place among the doubles as a whole number (equal for -0 and 0): the
+// comparisons below take two integer instructions instead of the FP64 pipe,
+// which takes 16 cycles an instruction and warp on this GPU.
+__device__ __forceinline__ long long order_key(double x) {
+  const long long b = __double_as_longlong(x + 0.0);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+
+// Ranks of lnL (ascending, ties broken by index) into ord[], one CTA; key: n
+// words of scratch.
+__device__ void rank_live(int n, const double* lnl_s, long long* key, int* ord) {
+  for (int i = threadIdx.x; i < n; i += blockDim.x) key[i] = order_key(lnl_s[i]);
+  __syncthreads();
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const double a = lnl_s[i];
+    const long long a = key[i];
     int r = 0;
-    for (int j = 0; j < n; ++j) {
-      const double b = lnl_s[j];
-      r += (b < a) || (b == a && j < i);
-    }
+#pragma unroll 4
+    for (int j = 0; j < n; ++j) r += key[j] < a + (j < i);   // b < a, or b == a and j < i
     ord[r] = i;
   }
+  __syncthreads();
+}
+
+constexpr int SEL_STAGE = 32768;   // bytes: the ranks' keys (8 NSS_MAX_LIVE), then the survivors' coordinates
+
+// Shared memory of k_nss_select in bytes: lnL, step and ln weight of the
+// removed points, the stage, ranks, means, and the covariance
+size_t sel_smem_bytes(int n, int k, int d, bool full) {
+  return 8ull * n + 16ull * k + SEL_STAGE + 4ull * n + 4ull * d + (full ? 4ull * d * d : 0);
 }
 
 // One CTA: remove the k lowest live points (evidence, dead records), start the
@@ -139,10 +207,15 @@ __global__ void __launch_bounds__(1024) k_nss_select(int n, int k, int d, int it
                                                      float* chol, NssState* st, uint32_t k0, uint32_t k1) {
   extern __shared__ __align__(16) uint8_t smem[];
   double* lnl_s = reinterpret_cast<double*>(smem);
-  int* ord = reinterpret_cast<int*>(lnl_s + n);
+  double* step_s = lnl_s + n;                 // [k] ln X lost with each removed point
+  double* lnw_s = step_s + k;                 // [k] its ln weight
+  long long* key = reinterpret_cast<long long*>(lnw_s + k);
+  float* stage = reinterpret_cast<float*>(key);
+  int* ord = reinterpret_cast<int*>(stage + SEL_STAGE / 4);
   float* mu = reinterpret_cast<float*>(ord + n);
   float* A = mu + d;                          // [d][d] covariance, then its Cholesky factor (full mode)
   __shared__ int s_above, s_nd0;
+  __shared__ double red[RED_THREADS / 32];
   const bool full = d <= NSS_FULL_COV;
   const int tid = threadIdx.x;
   for (int i = tid; i < n; i += blockDim.x) lnl_s[i] = lv.lnl[i];
@@ -151,9 +224,13 @@ __global__ void __launch_bounds__(1024) k_nss_select(int n, int k, int d, int it
     s_nd0 = st->n_dead;
     st->active[0] = st->active[1] = 0;
   }
+  // the removed points' shares of the prior volume
+  for (int j = tid; j < k; j += blockDim.x) {
+    step_s[j] = 1.0 / (double)(n - j);
+    lnw_s[j] = log(-expm1(-step_s[j]));
+  }
   __syncthreads();
-  rank_live(n, lnl_s, ord);
-  __syncthreads();
+  rank_live(n, lnl_s, key, ord);
   const double lstar = lnl_s[ord[k - 1]];
   int cnt = 0;
   for (int i = tid; i < n; i += blockDim.x) cnt += lnl_s[i] > lstar;
@@ -171,15 +248,9 @@ __global__ void __launch_bounds__(1024) k_nss_select(int n, int k, int d, int it
   if (tid == 0) {
     double lnX = st->lnX;
     for (int j = 0; j < k; ++j) {
-      const double step = 1.0 / (double)(n - j);
-      const double lnw = lnX + log(-expm1(-step));
+      const double step = step_s[j];
+      step_s[j] = lnX;
       lnX -= step;
-      const double l = lnl_s[ord[j]];
-      add_point(st, l, lnw);
-      if (nd0 + j < dd.cap) {
-        dd.lnl[nd0 + j] = l;
-        dd.lnw[nd0 + j] = lnw;
-      }
     }
     st->lnX = lnX;
     st->lstar = lstar;
@@ -187,6 +258,17 @@ __global__ void __launch_bounds__(1024) k_nss_select(int n, int k, int d, int it
     st->n_dead = nd0 + k;
     if (n_above == 0) st->stop = 2;   // every survivor sits on the contour: nothing left to climb
   }
+  __syncthreads();
+  for (int j = tid; j < k; j += blockDim.x) {
+    const double lnw = step_s[j] + lnw_s[j];
+    lnw_s[j] = lnw;
+    if (nd0 + j < dd.cap) {
+      dd.lnl[nd0 + j] = lnl_s[ord[j]];
+      dd.lnw[nd0 + j] = lnw;
+    }
+  }
+  __syncthreads();
+  add_points(st, k, [&](int j) { return lnl_s[ord[j]]; }, [&](int j) { return lnw_s[j]; }, red);
   // chains: start at a random survivor strictly above the contour
   for (int c = tid; c < k; c += blockDim.x) {
     const uint4 r = philox(make_uint4((uint32_t)iter, (uint32_t)c, 0u, TAG_START), k0, k1);
@@ -204,36 +286,53 @@ __global__ void __launch_bounds__(1024) k_nss_select(int n, int k, int d, int it
     if (n_above > 0) src = ord[n - n_above + min((int)(u01(r.x) * n_above), n_above - 1)];
     ch.x0[q] = lv.U[(size_t)src * d + j];
   }
-  // covariance of the survivors (all live points but the k removed), unit-cube coordinates
-  const int m = n - k;
-  for (int j = tid; j < d; j += blockDim.x) {
-    float s = 0.f;
-    for (int q = 0; q < m; ++q) s += lv.U[(size_t)ord[k + q] * d + j];
-    mu[j] = s / (float)m;
-  }
-  __syncthreads();
+  // covariance of the survivors (all live points but the k removed), unit-cube
+  // coordinates.  The survivors pass through shared memory in chunks, loaded by
+  // all threads at once; every sum runs over them in order.  (Threads that read
+  // the survivors one after the other waited on L2 for each: with that, the
+  // evidence and the ranks above in FP64, this kernel took 425 us at 300 points.)
+  const int m = n - k, chunk = max(SEL_STAGE / 4 / d, 1);
   const float inv = 1.f / (float)max(m - 1, 1);
-  if (!full) {
-    for (int j = tid; j < d; j += blockDim.x) {
-      float s = 0.f;
-      for (int q = 0; q < m; ++q) {
-        const float x = lv.U[(size_t)ord[k + q] * d + j] - mu[j];
-        s = fmaf(x, x, s);
-      }
-      chol[j] = sqrtf(s * inv + 1e-14f);
-    }
-    return;
-  }
-  for (int e = tid; e < d * d; e += blockDim.x) {
-    const int i = e / d, j = e - i * d;
-    if (j > i) continue;
+  for (int e = tid; e < (full ? d * d : 0); e += blockDim.x) A[e] = 0.f;
+  for (int pass = 0; pass < 2; ++pass) {   // means, then covariances or variances
     float s = 0.f;
-    for (int q = 0; q < m; ++q) {
-      const float* u = lv.U + (size_t)ord[k + q] * d;
-      s = fmaf(u[i] - mu[i], u[j] - mu[j], s);
+    for (int q0 = 0; q0 < m; q0 += chunk) {
+      const int nq = min(chunk, m - q0);
+      if (pass == 0 || m > chunk) {
+        __syncthreads();
+        for (int e = tid; e < nq * d; e += blockDim.x) {
+          const int q = e / d;
+          stage[e] = lv.U[(size_t)ord[k + q0 + q] * d + (e - q * d)];
+        }
+        __syncthreads();
+      }
+      if (pass == 0) {
+        if (tid < d)
+          for (int q = 0; q < nq; ++q) s += stage[q * d + tid];
+      } else if (!full) {
+        if (tid < d)
+          for (int q = 0; q < nq; ++q) {
+            const float x = stage[q * d + tid] - mu[tid];
+            s = fmaf(x, x, s);
+          }
+      } else {
+        for (int e = tid; e < d * d; e += blockDim.x) {
+          const int i = e / d, j = e - i * d;
+          if (j > i) continue;
+          float c = A[e];
+          const float mi = mu[i], mj = mu[j];
+#pragma unroll 4
+          for (int q = 0; q < nq; ++q) c = fmaf(stage[q * d + i] - mi, stage[q * d + j] - mj, c);
+          A[e] = c;
+        }
+      }
     }
-    A[i * d + j] = s * inv;
+    if (tid < d && pass == 0) mu[tid] = s / (float)m;
+    if (tid < d && pass == 1 && !full) chol[tid] = sqrtf(s * inv + 1e-14f);
+    __syncthreads();
   }
+  if (!full) return;
+  for (int e = tid; e < d * d; e += blockDim.x) A[e] *= inv;
   __syncthreads();
   for (int j = tid; j < d; j += blockDim.x) mu[j] = A[j * d + j];   // the variances, for the pivot floor
   __syncthreads();
@@ -401,14 +500,20 @@ __global__ void __launch_bounds__(CHAINS_PER_BLOCK * 32) k_nss_round(RoundArgs a
 __global__ void __launch_bounds__(1024) k_nss_replace(int n, int k, int d, int iter, const double* lo,
                                                       const double* hi, Live lv, Dead dd, Chains ch, NssState* st,
                                                       double stop_dlnz, int last) {
-  __shared__ double red[32];
+  __shared__ double red[RED_THREADS / 32];
+  __shared__ long long key[NSS_MAX_LIVE];   // the survivors' lnL in order
   const int tid = threadIdx.x;
   const int nd0 = st->n_dead - k;   // first dead record of this iteration
+  for (int q = k + tid; q < n; q += blockDim.x) key[q] = order_key(lv.lnl[lv.order[q]]);
+  __syncthreads();
   for (int c = tid; c < k; c += blockDim.x) {
-    const double l = ch.lnl0[c];
-    int r = 0;
-    for (int q = k; q < n; ++q) r += lv.lnl[lv.order[q]] < l;
-    if (nd0 + c < dd.cap && dd.rank) dd.rank[nd0 + c] = r;
+    const long long l = order_key(ch.lnl0[c]);
+    int q = k, q1 = n;   // they ascend: the first one not below l
+    while (q < q1) {
+      const int mid = (q + q1) >> 1;
+      if (key[mid] < l) q = mid + 1; else q1 = mid;
+    }
+    if (nd0 + c < dd.cap && dd.rank) dd.rank[nd0 + c] = q - k;
   }
   __syncthreads();
   for (int q = tid; q < k * d; q += blockDim.x) {
@@ -422,31 +527,14 @@ __global__ void __launch_bounds__(1024) k_nss_replace(int n, int k, int d, int i
   __syncthreads();
   // ln Z_live = ln X + ln(mean L_live)
   double mx = -INFINITY;
-  for (int i = tid; i < n; i += blockDim.x) mx = fmax(mx, lv.lnl[i]);
-#pragma unroll
-  for (int o = 16; o; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if ((tid & 31) == 0) red[tid >> 5] = mx;
-  __syncthreads();
-  if (tid < 32) {
-    double v = tid < (int)(blockDim.x >> 5) ? red[tid] : -INFINITY;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if (tid == 0) red[0] = v;
-  }
-  __syncthreads();
-  mx = red[0];
-  __syncthreads();
+  for (int i = red_start(n); i < n; i += RED_THREADS) mx = fmax(mx, lv.lnl[i]);
+  mx = block_reduce<true>(mx, red);
   double sm = 0.0;
   if (mx > -INFINITY)
-    for (int i = tid; i < n; i += blockDim.x) sm += exp(lv.lnl[i] - mx);
-#pragma unroll
-  for (int o = 16; o; o >>= 1) sm += __shfl_xor_sync(0xffffffffu, sm, o);
-  if ((tid & 31) == 0) red[tid >> 5] = sm;
-  __syncthreads();
+    for (int i = red_start(n); i < n; i += RED_THREADS) sm += exp(lv.lnl[i] - mx);
+  sm = block_reduce<false>(sm, red);
   if (tid == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    const double lz_live = mx == -INFINITY ? -INFINITY : st->lnX + mx + log(t) - log((double)n);
+    const double lz_live = mx == -INFINITY ? -INFINITY : st->lnX + mx + log(sm) - log((double)n);
     if (st->lnZ > -INFINITY && lz_live - st->lnZ < stop_dlnz) st->stop = 1;
     if (last && !st->stop) st->stop = 3;
   }
@@ -457,31 +545,31 @@ __global__ void __launch_bounds__(1024) k_nss_replace(int n, int k, int d, int i
 __global__ void __launch_bounds__(1024) k_nss_final(int n, int d, Live lv, Dead dd, NssState* st) {
   extern __shared__ __align__(16) uint8_t smem[];
   double* lnl_s = reinterpret_cast<double*>(smem);
-  int* ord = reinterpret_cast<int*>(lnl_s + n);
+  long long* key = reinterpret_cast<long long*>(lnl_s + n);
+  int* ord = reinterpret_cast<int*>(key + n);
   __shared__ int s_nd0;
+  __shared__ double s_lnw;
+  __shared__ double red[RED_THREADS / 32];
   const int tid = threadIdx.x;
   for (int i = tid; i < n; i += blockDim.x) lnl_s[i] = lv.lnl[i];
   if (tid == 0) s_nd0 = st->n_dead;
   __syncthreads();
-  rank_live(n, lnl_s, ord);
-  __syncthreads();
+  rank_live(n, lnl_s, key, ord);
   const int nd0 = s_nd0;
   for (int q = tid; q < n * d; q += blockDim.x) {
     const int j = q / d, c = q - j * d;
     if (nd0 + j < dd.cap) dd.TH[(size_t)(nd0 + j) * d + c] = lv.TH[(size_t)ord[j] * d + c];
   }
-  if (tid == 0) {
-    const double lnw = st->lnX - log((double)n);
-    for (int j = 0; j < n; ++j) {
-      const double l = lnl_s[ord[j]];
-      add_point(st, l, lnw);
-      if (nd0 + j < dd.cap) {
-        dd.lnl[nd0 + j] = l;
-        dd.lnw[nd0 + j] = lnw;
-      }
+  if (tid == 0) s_lnw = st->lnX - log((double)n);
+  __syncthreads();
+  const double lnw = s_lnw;
+  for (int j = tid; j < n; j += blockDim.x)
+    if (nd0 + j < dd.cap) {
+      dd.lnl[nd0 + j] = lnl_s[ord[j]];
+      dd.lnw[nd0 + j] = lnw;
     }
-    st->n_dead = nd0 + n;
-  }
+  add_points(st, n, [&](int j) { return lnl_s[ord[j]]; }, [&](int) { return lnw; }, red);
+  if (tid == 0) st->n_dead = nd0 + n;
   __syncthreads();
   const double lz = st->lnZ;
   const int nrec = min(st->n_dead, dd.cap);
@@ -558,8 +646,8 @@ sed_status sed_nss_run(sed_ctx* ctx, sed_model_id model, const sed_nss_desc* des
   Dead dd{(float*)F(o_dth), (double*)F(o_dl), (double*)F(o_dw), (int*)F(o_dr), cap};
   const uint32_t k0 = (uint32_t)desc->seed, k1 = (uint32_t)(desc->seed >> 32);
   const float w = desc->slice_width > 0.0 ? (float)desc->slice_width : sqrtf((float)d + 2.f);
-  const size_t sel_smem = 12ull * n + 4ull * d + (full ? 4ull * d * d : 0);
-  const size_t fin_smem = 12ull * n;
+  const size_t sel_smem = sel_smem_bytes(n, k, d, full);
+  const size_t fin_smem = 20ull * n;
   const size_t round_smem = 4ull * CHAINS_PER_BLOCK * 2 * d;
   static DynSmemCache a_sel, a_fin, a_round;
   const long long max_rounds = (long long)desc->n_slice_steps * (2 * MAXOUT + MAXSHRINK) + 4;
