@@ -162,6 +162,22 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const float* v) {
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+// four floats at shared-memory address addr of the cluster's CTA `rank`
+__device__ __forceinline__ float4 ld_cluster(uint32_t addr, uint32_t rank) {
+  uint32_t ra;
+  float4 v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(addr), "r"(rank));
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(ra)
+               : "memory");
+  return v;
+}
+
 struct Params {
   const RowScal* rs;         // per-row rest-frame node windows (NULL: no window)
   CUtensorMap a_hi, a_lo, b_hi, b_lo;
@@ -189,6 +205,7 @@ struct Params {
   int seg_col[MAX_SEG + 1];
   int seg_rows;
   size_t seg_stride;
+  int cz;                    // adjoint: CTAs of a cluster that share a tile's accumulation groups (1: no cluster)
 };
 
 // K tiles of a unit's range.  A K tile that no row of the M tile touches holds
@@ -267,7 +284,18 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 //    tiles are split along the rows into up to four pieces of BN/npc rows (an
 //    MMA of N = BN/npc), so the last partial wave costs a fraction of a unit.  Tensor memory, barriers and the smem ring are set up
 //    once, and one unit's drain overlaps the next unit's MMAs.
+//  - Clusters (adjoint, p.cz > 1): a launch with few tiles (200 rows of the
+//    paper-scale grid: 22 on 152 SMs) gives each to a cluster of cz CTAs along
+//    blockIdx.z, which share the groups of its reduction over wavelength: CTA 0
+//    takes the first ones and sums them as above, each other CTA at most
+//    CL_SLOTS more, every group in tensor memory of its own.  The sums then go to
+//    the CTAs' shared memory (the ring's), and each CTA adds a share of the rows'
+//    from all of them, CTA 0's first and then group by group: every output is the
+//    same sum, rounded the same way, as without the cluster.  A tile's MMAs run at
+//    the tensor core's rate (an MMA of 128 x 128 x 8 in TF32 takes about 60
+//    cycles), so only more SMs help.
 constexpr int MAX_MT = 64;   // M tiles of a persistent launch (8192 rows)
+constexpr int CL_SLOTS = 3;  // groups of a CTA past the cluster's first: 64 KB of the ring and BN columns of tensor memory each
 
 struct Unit {
   const uint32_t* km;        // K-tile mask row of the unit's M tile (NULL: every K tile)
@@ -366,6 +394,9 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
   int nz = 1;   // units per tile (3: the persistent launch splits its tiles)
   int K0 = 0, KY = p.ky_tiles, KT = p.k_tiles;
   int n_units = 1, upz = 0;
+  const int cz = GRAD ? p.cz : 1, crank = GRAD && p.cz > 1 ? (int)blockIdx.z : 0;
+  int c_gpc = 1, c_terms = 1, c_own = 0;   // cluster: groups per further CTA, sums of an output, this CTA's groups
+  const uint32_t tm_cols = GRAD && cz > 1 ? 512u : C::TMEM_COLS;
   int nfull = 0, nrem = 0, npc = 1;   // persistent: tiles in full waves, leftover tiles, pieces per leftover tile
 
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -391,7 +422,7 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
     }
     if (warp == 2) {
       asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)),
-                   "r"(C::TMEM_COLS)
+                   "r"(tm_cols)
                    : "memory");
       asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -490,6 +521,17 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
         const int c0 = t < p.ny_tiles ? t * BM : p.n_split + (t - p.ny_tiles) * BM;
         const int c1 = min(c0 + BM, t < p.ny_tiles ? p.n_split : p.ld_out);
         if (knext(p.kmask + (size_t)blockIdx.y * p.kmask_w, c0 / 32, (c1 + 31) / 32) >= (c1 + 31) / 32) return;
+      }
+      if (cz > 1) {   // this CTA's groups (all of the cluster's CTAs are here: the returns above are the tile's)
+        const int ng = (KT - K0 + G - 1) / G;
+        c_gpc = min((ng + cz - 1) / cz, CL_SLOTS);
+        const int first = max(c_gpc, ng - c_gpc * (cz - 1));   // CTA 0's
+        c_terms = 1 + max(ng - first, 0);
+        const int g0 = min(crank == 0 ? 0 : first + (crank - 1) * c_gpc, ng);
+        c_own = min(crank == 0 ? first : c_gpc, ng - g0);
+        KT = min(KT, K0 + (g0 + c_own) * G);
+        K0 = K0 + g0 * G;
+        KY = KT;
       }
     }
   }
@@ -612,8 +654,8 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
           const int ge = gs + G < ke ? gs + G : ke;
           const int k_first = kn(u.km, gs, ge);
           if (KSKIP && k_first >= ge) continue;   // no touched K tile in this group
-          const int b = g & 1;
-          if (!__all_sync(0xffffffffu, mbar_wait(tempty0 + 8 * b, (((uint32_t)g >> 1) & 1u) ^ 1u))) {
+          const int b = crank > 0 ? g : g & 1;   // a cluster's further CTAs keep each group in columns of its own
+          if (crank == 0 && !__all_sync(0xffffffffu, mbar_wait(tempty0 + 8 * b, (((uint32_t)g >> 1) & 1u) ^ 1u))) {
             if (lane == 0) atomicOr(p.err, 8);
             ok = false;
             break;
@@ -647,7 +689,11 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
             acc = 1u;
             if (++st_i == stages) { st_i = 0; st_ph ^= 1u; }
           }
-          if (ok && elect_one()) mma_commit(tfull0 + 8 * b);
+          if (crank > 0) {   // one hand-over, after the last group
+            if (ok && ge == ke && elect_one()) mma_commit(tfull0);
+          } else if (ok && elect_one()) {
+            mma_commit(tfull0 + 8 * b);
+          }
           __syncwarp();
           ++g;
         }
@@ -669,6 +715,25 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
         float* out;
         int mode;
         unit_range<PREC, GRAD>(p, u, r, kb, ke, out, mode);
+        float* slot = nullptr;   // cluster: the sums go to shared memory, [row][column]
+        if constexpr (GRAD)
+          if (cz > 1) slot = reinterpret_cast<float*>(smem_raw + (sbase - smem_u32(smem_raw))) + col;
+        if (GRAD && crank > 0) {
+          if (c_own > 0 && !mbar_wait(tfull0, 0u)) { atomicOr(p.err, 4); ok = false; }
+          tc_fence_after();
+          for (int i = 0; ok && i < c_own; ++i) {
+#pragma unroll
+            for (int c = 0; c < BN / 32; ++c) {
+              if (c * 32 >= u.rows) break;
+              uint32_t rr[32];
+              tmem_ld32(tmem + lane_off + (uint32_t)(i * BN + c * 32), rr);
+              tmem_wait_ld();
+#pragma unroll
+              for (int q2 = 0; q2 < 32; ++q2) slot[(i * rt + c * 32 + q2) * BM] = __uint_as_float(rr[q2]);
+            }
+          }
+          continue;
+        }
         float run[BN];
 #pragma unroll
         for (int c = 0; c < BN; ++c) run[c] = 0.f;
@@ -715,7 +780,11 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
             continue;
           }
         }
-        if (col < u.ncol) {   // a warp stores 32 consecutive columns of one row at a time
+        if (GRAD && cz > 1) {
+#pragma unroll
+          for (int c = 0; c < BN; ++c)
+            if (c < u.rows) slot[c * BM] = run[c];
+        } else if (col < u.ncol) {   // a warp stores 32 consecutive columns of one row at a time
           float* dst = out + (size_t)u.m0 * p.ld_out + u.n0 + col;
 #pragma unroll
           for (int c = 0; c < BN / 32; ++c) {
@@ -730,11 +799,31 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
       }
     }
   }
+  if constexpr (GRAD) {
+    if (cz > 1) {   // one row at a time per warp, four columns per lane
+      Unit u;
+      get_unit(0, u);
+      cluster_sync();
+      const int vrow = min(u.rows, p.n - u.m0), c4 = 4 * lane;
+      for (int row = crank + cz * warp; row < vrow; row += cz * (C::THREADS / 32)) {
+        const uint32_t at = sbase + (uint32_t)(row * BM + c4) * 4u;
+        float4 v = ld_cluster(at, 0u);
+#pragma unroll 4
+        for (int t = 1; t < c_terms; ++t) {
+          const int rk = (t - 1) / c_gpc, i = t - 1 - rk * c_gpc;
+          const float4 w = ld_cluster(at + (uint32_t)(i * rt * BM) * 4u, (uint32_t)(rk + 1));
+          v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+        }
+        if (c4 < u.ncol) *reinterpret_cast<float4*>(p.Y + (size_t)(u.m0 + row) * p.ld_out + u.n0 + c4) = v;
+      }
+      cluster_sync();   // the others' shared memory is read until here
+    }
+  }
   tc_fence_before();
   __syncthreads();
   if (warp == 2) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::TMEM_COLS) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tm_cols) : "memory");
   }
 }
 
@@ -746,7 +835,9 @@ cudaError_t launch_cfg(const Params& p, int n_cols, cudaStream_t s) {
   static DynSmemCache attr;   // the raised shared-memory limit, set once per device
   if (cudaError_t e = ensure_dyn_smem(k, (size_t)C::SMEM, &attr)) return e;
   if (!GRAD && p.tile_win) return launch_pdl(k, dim3(n_sm, 1, 1), dim3(C::THREADS), C::SMEM, s, p);   // persistent: one CTA per SM
-  return launch_pdl(k, dim3(n_cols / BM, (p.n + BN - 1) / BN, 1), dim3(C::THREADS), C::SMEM, s, p);
+  const dim3 grid(n_cols / BM, (p.n + BN - 1) / BN, GRAD ? p.cz : 1);
+  if (GRAD && p.cz > 1) return launch_pdl_cluster(k, grid, dim3(C::THREADS), C::SMEM, s, dim3(1, 1, p.cz), p);
+  return launch_pdl(k, grid, dim3(C::THREADS), C::SMEM, s, p);
 }
 
 }  // namespace tc
@@ -873,6 +964,13 @@ cudaError_t launch_dw_tc(const DwArgs& a, cudaStream_t s) {
   p.n_seg = a.n_seg > 0 ? a.n_seg : 1;
   p.seg_rows = a.seg_rows;
   for (int sg = 0; sg <= MAX_SEG; ++sg) p.seg_col[sg] = sg < p.n_seg ? a.seg_k0[sg] : a.Ky_pad;
+  // As many CTAs per tile (1, 2, 4 or 8) as the tiles leave SMs for -- a cluster
+  // lies within one GPC, of about 18 SMs -- and the reduction has groups for.  200
+  // rows of the paper-scale grid (22 tiles): 43.6 us with one CTA each, 25.6 with
+  // four, the gradient call 163.6 -> 149.4 us.
+  const int tiles = (p.ny_tiles + no_tiles) * ((a.n + DW_BN - 1) / DW_BN), n_sm = device_sm_count();
+  p.cz = tiles * 8 <= n_sm - n_sm / 8 ? 8 : tiles * 4 <= n_sm ? 4 : tiles * 2 <= n_sm ? 2 : 1;
+  while (p.cz > 1 && (p.cz - 1) * 8 >= p.k_tiles) p.cz /= 2;
   return tc::launch_cfg<SED_PREC_FP32, DW_BN, 3, 8, true>(p, (p.ny_tiles + no_tiles) * DW_BN, s);
 }
 
