@@ -32,6 +32,18 @@ __device__ __forceinline__ float gauss_w(float u2) {
   return w;
 }
 
+__device__ __forceinline__ float lg2_approx(float x) {
+  float y;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// four bytes of global memory to shared memory without a register (the thread
+// itself reads them after cp_async_wait_all)
+__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 __device__ __forceinline__ float dust_shape(const ModelDev& md, const float4& c, float eb, float pw) {
   return md.dust_law == SED_DUST_POWER_LAW ? pw : (c.y + eb * c.z) * pw;
 }

@@ -171,11 +171,7 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
   float* ln_is = ln_A + NLn;
   float* upx = ln_is + NLn;
   float* ulc = upx + (NLn ? md.n_pix : 0);
-  // each thread owns a contiguous run of CH window nodes (CH odd: the runs of a
-  // warp fall in distinct shared-memory banks) for the node-owned gathers
   const int nw = k_hi - k_lo + 1;
-  const int CH = ((nw + EB_THREADS - 1) / EB_THREADS) | 1;
-  const int kr0 = k_lo + tid * CH, kr1 = min(kr0 + CH, k_hi + 1);   // this thread's nodes [kr0, kr1)
   const float* Yr = a.Y + ro;
   const float* Or = a.O + ro;
   const float* O2r = a.O2 && a.o2_split && *a.o2_split ? a.O2 + ro : nullptr;
@@ -194,23 +190,54 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
   // ---- forward: attenuated spectrum in the window (the forward epilogue's
   //      arithmetic); phi holds the window's wavelengths until the photometric
   //      gather starts
+  if constexpr (VAR != 1)   // Y and O of all the thread's nodes into the nodes' own places at once
+    for (int k = k_lo + tid; k <= k_hi; k += EB_THREADS) {
+      cp_async4(Fs + k, Yr + k);
+      cp_async4(phi + k, Or + k);
+    }
+  // what a node needs besides, loaded one node ahead (the loops over a thread's
+  // nodes wait on L2 for every node otherwise)
+  struct Node { float4 c, nt; float v; };
+  auto load_node = [&](int k, const float* vr, Node& n) {
+    if (k > k_hi) return;
+    n.c = __ldg(g.att4 + k);
+    if (VAR == 0 && md.use_neb) n.nt = neb_corners(rs, g, k);
+    if (vr) n.v = vr[k];
+  };
+  Node nx{};
+  load_node(k_lo + tid, O2r, nx);
+  // dlnL/dY and dlnL/dO are zero outside the window, four nodes at a time (the
+  // rows and the window's ends within four are the dust pass's)
+  for (int q = 4 * tid; q < a.ldn; q += 4 * EB_THREADS) {
+    if (q + 3 >= k_lo && q <= k_hi) continue;
+    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int sg = 0; sg < (VAR == 1 ? md.n_seg : 1); ++sg) {
+      *reinterpret_cast<float4*>(a.gy_hi + sg * a.seg_stride + ro + q) = z;
+      if (a.split) *reinterpret_cast<float4*>(a.gy_lo + sg * a.seg_stride + ro + q) = z;
+    }
+    *reinterpret_cast<float4*>(a.go_hi + ro + q) = z;
+    if (a.split) *reinterpret_cast<float4*>(a.go_lo + ro + q) = z;
+  }
+  cp_async_wait_all();
 #pragma unroll 1
   for (int k = k_lo + tid; k <= k_hi; k += EB_THREADS) {
+    const Node n = nx;
+    load_node(k + EB_THREADS, O2r, nx);
     if constexpr (VAR == 1) {
       float yv[MAX_SEG];
 #pragma unroll
       for (int sg = 0; sg < MAX_SEG; ++sg) yv[sg] = sg < md.n_seg ? Yr[sg * a.seg_stride + k] : 0.f;
-      Fs[k] = attenuated_bins(md, rs, g.att4[k], eb_kc, yv, O2r ? Or[k] + O2r[k] : Or[k], g, k);
+      Fs[k] = attenuated_bins(md, rs, n.c, eb_kc, yv, O2r ? Or[k] + n.v : Or[k], g, k);
     } else {
-      const float nb = !md.use_neb ? 0.f : VAR == 2 ? neb_emission(rs, g, qa, k) : neb_emission(rs, neb_corners(rs, g, k));
-      Fs[k] = attenuated(md, rs, g.att4[k], eb_kc, Yr[k], O2r ? Or[k] + O2r[k] : Or[k], nb, k);
+      const float nb = !md.use_neb ? 0.f : VAR == 2 ? neb_emission(rs, g, qa, k) : neb_emission(rs, n.nt);
+      Fs[k] = attenuated(md, rs, n.c, eb_kc, Fs[k], O2r ? phi[k] + n.v : phi[k], nb, k);
     }
-    if (md.use_igm && g.lam_f[k] < IGM_LYA) {   // the IGM transmission (the forward epilogue's)
+    if (md.use_igm && n.c.w < IGM_LYA) {   // the IGM transmission (the forward epilogue's)
       float tau, dtau;
-      igm_madau(g.att4[k].w, opz, tau, dtau);
+      igm_madau(n.c.w, opz, tau, dtau);
       Fs[k] *= __expf(-rs.igm_f * tau);
     }
-    phi[k] = g.lam_f[k];
+    phi[k] = n.c.w;
   }
   for (int l = tid; l < NLn; l += EB_THREADS) line_setup(md, g, rs, eb_kc, l, ln_F, ln_A, ln_is, ln_x);
   __syncthreads();
@@ -227,58 +254,76 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
     ulc[k] = (float)u;
   }
 
-  // ---- photometry forward (warp per band, four samples in flight per lane),
+  // ---- photometry forward (warp per band, eight samples in flight per lane),
   //      the sample brackets, u_b and the gather part of dlnL/dz (the sample
-  //      positions lam_j/(1+z) move with z).  Brackets start from the index
-  //      table over ln(lambda) (fast logarithm: the walk within the window
-  //      ends on the same node from any start).
+  //      positions lam_j/(1+z) move with z).  A sample's bracket is the index
+  //      table's node or the next one where the forward epilogue picks it so (its
+  //      comment has the bounds), else it is found by a walk from there: the same
+  //      bracket either way.
   const float lam0 = g.lam_f[0], lamN = g.lam_f[N - 1];
   const int kmin = k_lo, kmax = k_hi - 1;
   const float* lam_s = phi;
   float gz_gather = 0.f;
+  const float slack = 8e-6f * g.lut_inv_h;
+  const bool pick = slack <= 0.25f && k_hi - k_lo >= 2 && md.samp_lam_min * rs.inv1pz >= lam0 &&
+                    md.samp_lam_max * rs.inv1pz <= lamN;
+  const float q_mul = 0.6931471805599453f * g.lut_inv_h, q_add = fmaf(-g.lut_x0, g.lut_inv_h, -slack);
   for (int b = warp; b < md.n_filt; b += EB_WARPS) {
     const int js = md.band_start[b], je = md.band_start[b + 1];
     float acc = 0.f, gzb = 0.f;
     int bmin = 0x7fffffff, bmax = -1;
-    for (int j0 = js + lane; j0 < je; j0 += 128) {
-      float2 sp[4];   // {lambda_obs, weight}
-      int kg[4];
+    // one sample between the nodes k (at la) and k + 1 (at lb)
+    auto sample = [&](int j, float x, float w, int k, float la, float lb) {
+      const float t = (x - la) / (lb - la);
+      const float G0 = __fdividef(Fs[k], la * la), G1 = __fdividef(Fs[k + 1], lb * lb);
+      gzb = fmaf(w, __fdividef(G1 - G0, lb - la) * (-x * rs.inv1pz), gzb);
+      bmin = min(bmin, k);
+      bmax = max(bmax, k);
+      sk[j] = k;
+      st[j] = t;
+      acc = fmaf(w, G0 + t * (G1 - G0), acc);
+    };
+    for (int j0 = js + lane; j0 < je; j0 += 256) {
+      if (pick) {
+        float2 sp[8];   // {lambda_obs, weight}
+        int kg[8];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) sp[u] = j0 + 32 * u < je ? md.samp2[j0 + 32 * u] : make_float2(0.f, 0.f);
+        for (int u = 0; u < 8; ++u)
+          if (j0 + 32 * u < je) sp[u] = __ldg(md.samp2 + j0 + 32 * u);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        int q = (int)((__logf(fmaxf(sp[u].x * rs.inv1pz, lam0)) - g.lut_x0) * g.lut_inv_h);
-        q = q < 0 ? 0 : (q >= g.lut_n ? g.lut_n - 1 : q);
-        kg[u] = g.lut[q];
-      }
+        for (int u = 0; u < 8; ++u)
+          if (j0 + 32 * u < je) {
+            sp[u].x *= rs.inv1pz;
+            kg[u] = __ldg(g.lut + (int)fmaf(lg2_approx(sp[u].x), q_mul, q_add));
+          }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int j = j0 + 32 * u;
-        if (j >= je) continue;
-        const float x = sp[u].x * rs.inv1pz;
-        float v = 0.f, t = 0.f;
-        int k;
-        if (x < lam0) {
-          k = -2;
-        } else if (x > lamN) {
-          k = N;
-        } else {
-          k = min(max(kg[u], kmin), kmax);
+        for (int u = 0; u < 8; ++u)
+          if (j0 + 32 * u < je) {
+            const float x = sp[u].x;
+            const int k = min(kg[u], kmax - 1);
+            const float l1 = lam_s[k + 1];
+            const bool up = l1 <= x;
+            const float lx = lam_s[up ? k + 2 : k];
+            sample(j0 + 32 * u, x, sp[u].y, up ? k + 1 : k, up ? l1 : lx, up ? lx : l1);
+          }
+      } else {
+#pragma unroll 1
+        for (int j = j0; j < min(j0 + 256, je); j += 32) {
+          const float2 s2 = __ldg(md.samp2 + j);
+          const float x = s2.x * rs.inv1pz;
+          if (!(x >= lam0 && x <= lamN)) {   // outside the grid: weight zero, past every bracket
+            sk[j] = x < lam0 ? -2 : N;
+            st[j] = 0.f;
+            continue;
+          }
+          int k = g.lut[min(max((int)fmaf(lg2_approx(x), q_mul, q_add), 0), g.lut_n - 1)];
+          k = min(max(k, kmin), kmax);
 #pragma unroll 1
           while (k < kmax && lam_s[k + 1] <= x) ++k;
 #pragma unroll 1
           while (k > kmin && lam_s[k] > x) --k;
-          const float la = lam_s[k], lb = lam_s[k + 1];
-          t = (x - la) / (lb - la);
-          const float G0 = __fdividef(Fs[k], la * la), G1 = __fdividef(Fs[k + 1], lb * lb);
-          v = G0 + t * (G1 - G0);
-          gzb += sp[u].y * ((G1 - G0) / (lb - la)) * (-x * rs.inv1pz);
-          bmin = min(bmin, k);
-          bmax = max(bmax, k);
+          sample(j, x, s2.y, k, lam_s[k], lam_s[k + 1]);
         }
-        sk[j] = k;
-        st[j] = t;
-        acc = fmaf(sp[u].y, v, acc);
       }
     }
 #pragma unroll
@@ -317,42 +362,68 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
   __syncthreads();
 
   // ---- dlnL/dF from the photometry: node k gathers the samples bracketed by
-  //      [k-1, k] (weight t) and [k, k+1] (weight 1-t), band by band in order
-  //      and in sample order within a band.  Each thread owns a run of nodes and
-  //      walks the samples that reach it once per band, from one binary search
-  //      over the band's (ascending) brackets, with four sample weights in flight.
-  for (int k = kr0; k < kr1; ++k) phi[k] = 0.f;
-  for (int b = 0; b < md.n_filt; ++b) {
-    const float cb = ubp[b];
-    const int lo = max(bk0[b], kr0), hi = min(bk1[b] + 1, kr1 - 1);
-    if (cb == 0.f || lo > hi) continue;
-    const int je = md.band_start[b + 1];
-    int j = md.band_start[b], j1 = je;
-    while (j < j1) {
-      const int mid = (j + j1) >> 1;
-      if (sk[mid] < lo - 1) j = mid + 1; else j1 = mid;
-    }
-    for (; j < je && sk[j] <= hi; j += 4) {
-      int kk[4];
-      float ww[4], tt[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const bool ok = j + u < je;
-        kk[u] = ok ? sk[j + u] : 0x7fffffff;
-        ww[u] = ok ? md.samp2[j + u].y : 0.f;
-        tt[u] = ok ? st[j + u] : 0.f;
+  //      [k-1, k] (weight t) and [k, k+1] (weight 1-t).  A warp owns a run of
+  //      nodes and takes the bands that reach it in order, 32 samples at a time:
+  //      the lanes of one bracket (they ascend) sum their parts by shuffles, and
+  //      the last of them adds the sums to the bracket's two nodes.  (With a thread
+  //      per run of 9 nodes that went through its samples one by one, this phase
+  //      took 36,000 of a row's 190,000 cycles, and as many of the 135,000 of a row
+  //      alone on its SM.  With the photometry above and the loads ahead: 2048 rows
+  //      with a spectrum 353 -> 300 us, 200 photometric rows 62 -> 46 us.)
+  {
+    const int run = (nw + EB_WARPS - 1) / EB_WARPS;
+    const int n0 = k_lo + warp * run, n1 = min(n0 + run, k_hi + 1);   // this warp's nodes [n0, n1)
+    for (int k = n0 + lane; k < n1; k += 32) phi[k] = 0.f;
+    __syncwarp();
+    for (int b = 0; b < md.n_filt; ++b) {
+      const float cb = ubp[b];
+      const int lo = max(bk0[b], n0 - 1), hi = min(bk1[b], n1 - 1);   // brackets that touch the run
+      if (cb == 0.f || lo > hi) continue;
+      const int je = md.band_start[b + 1];
+      int j = md.band_start[b];
+      for (int c = je - j; c > 0;) {   // first sample whose bracket is lo or later, in [j, j + c]
+        const int step = (c + 31) >> 5;
+        const int below = __popc(__ballot_sync(0xffffffffu, lane * step < c && sk[j + lane * step] < lo));
+        if (below == 0) break;
+        const int end = min(below * step, c);
+        j += (below - 1) * step + 1;
+        c = end - (below - 1) * step - 1;
       }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int k = kk[u];
-        if (k > hi) continue;   // brackets ascend: the later samples lie beyond the run too
-        const float c = cb * ww[u];
-        if (k >= lo) phi[k] += c * (1.f - tt[u]);
-        if (k + 1 >= lo && k + 1 <= hi) phi[k + 1] += c * tt[u];
+      int k = 0;
+      float w = 0.f, t = 0.f;
+      auto load = [&](int i) {
+        const bool ok = i < je;
+        k = ok ? sk[i] : 0x7fffffff;
+        w = ok ? __ldg(&md.samp2[i].y) : 0.f;
+        t = ok ? st[i] : 0.f;
+      };
+      load(j + lane);
+      while (true) {
+        const int kk = k;
+        const bool in = kk <= hi;
+        const float c = in ? cb * w : 0.f;
+        float a0 = c * (1.f - t), a1 = c * t;
+        const bool more = __shfl_sync(0xffffffffu, kk, 31) <= hi;
+        j += 32;
+        if (more) load(j + lane);
+        for (int o = 1; o < 32; o <<= 1) {
+          const int k_prev = __shfl_up_sync(0xffffffffu, kk, o);
+          const bool same = lane >= o && k_prev == kk;
+          if (!__any_sync(0xffffffffu, same)) break;
+          const float p0 = __shfl_up_sync(0xffffffffu, a0, o), p1 = __shfl_up_sync(0xffffffffu, a1, o);
+          if (same) { a0 += p0; a1 += p1; }
+        }
+        const int k_next = __shfl_down_sync(0xffffffffu, kk, 1);   // by every lane: not behind a && or ?:
+        const bool last = in && (lane == 31 || k_next != kk);
+        if (last && kk >= n0) phi[kk] += a0;
+        __syncwarp();
+        if (last && kk + 1 < n1) phi[kk + 1] += a1;
+        __syncwarp();
+        if (!more) break;
       }
     }
+    for (int k = n0 + lane; k < n1; k += 32) phi[k] *= g.inv_lam2[k];
   }
-  for (int k = kr0; k < kr1; ++k) phi[k] *= g.inv_lam2[k];
   __syncthreads();
 
   // ---- spectrum forward: m_i, its derivatives in x and s and each pixel's node
@@ -788,12 +859,14 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
     }
     gz_spec += gzl;
   }
+  // the window's nodes and, with zeros, the rest of its first and last four
+  const int d_lo = k_lo & ~3, d_hi = min(k_hi | 3, a.ldn - 1);
   // age-binned dust: d/d(tau_b, slope_b) of each bin, d/dQ of each block
   float g_bin[2 * MAX_DUST_BIN] = {}, g_qs[MAX_SEG + 1] = {};
   if constexpr (VAR == 1) {
     // F = e^{-tau_d} [ sum_s A_s (Y_s + Q_s neb) + O + Q_rest neb ], A_s = e^{-tau_s},
     // tau_s = sum_b M_sb tau_b shape_b (atten.cuh's attenuated_bins)
-    for (int k = tid; k < a.ldn; k += EB_THREADS) {
+    for (int k = d_lo + tid; k <= d_hi; k += EB_THREADS) {
       if (k < k_lo || k > k_hi) {
         for (int sg = 0; sg < md.n_seg; ++sg) put_g(a, a.gy_hi, a.gy_lo, sg * a.seg_stride + ro + k, 0.f);
         put_g(a, a.go_hi, a.go_lo, ro + k, 0.f);
@@ -878,14 +951,20 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
         g_lz += glg * sz;
       }
     }
-  } else
-  for (int k = tid; k < a.ldn; k += EB_THREADS) {
-    if (k < k_lo || k > k_hi) {
+  } else {
+  if (tid < 8) {
+    const int k = tid < 4 ? d_lo + tid : (k_hi & ~3) + tid - 4;
+    if (k <= d_hi && (k < k_lo || k > k_hi)) {
       put_g(a, a.gy_hi, a.gy_lo, ro + k, 0.f);
       put_g(a, a.go_hi, a.go_lo, ro + k, 0.f);
-      continue;
     }
-    const float4 c = g.att4[k];
+  }
+  load_node(k_lo + tid, Yr, nx);
+#pragma unroll 1
+  for (int k = k_lo + tid; k <= k_hi; k += EB_THREADS) {
+    const Node n = nx;
+    load_node(k + EB_THREADS, Yr, nx);
+    const float4 c = n.c;
     const float lnp = c.x;
     const float pa = __expf(rs.alpha_bc * lnp);
     const float tbc = rs.tau_bc * pa;
@@ -894,13 +973,13 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
     const float dshape = md.dust_law == SED_DUST_POWER_LAW ? pw * lnp : -1.9f * c.z * pw + shape * lnp;
     const float td = rs.tau_d * shape;
     const float ed = __expf(-td), eb = __expf(-tbc);
-    const float y = Yr[k];
+    const float y = n.v;
     float lg = 0.f, nb = 0.f;
     if (md.use_neb) {
       if (qa) {
         nb = neb_emission(rs, g, qa, k);
       } else {
-        lg = neb_log10(rs, neb_corners(rs, g, k));
+        lg = neb_log10(rs, n.nt);
         nb = ex2_approx(rs.log2_qy + 3.3219280948873623f * lg);
       }
     }
@@ -952,16 +1031,17 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
     } else if (md.use_neb) {
       g_qy += gnb * ex2_approx(3.3219280948873623f * lg);
       const float glg = gnb * nb * 2.302585092994046f;
+      const float tv[4] = {n.nt.x, n.nt.y, n.nt.z, n.nt.w};
       float su = 0.f, sz = 0.f;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        const float tv = g.neb_tab[rs.neb_off[c] + k];
-        su += rs.neb_dwu[c] * tv;
-        sz += rs.neb_dwz[c] * tv;
+        su += rs.neb_dwu[c] * tv[c];
+        sz += rs.neb_dwz[c] * tv[c];
       }
       g_lu += glg * su;
       g_lz += glg * sz;
     }
+  }
   }
   if (qa) {
     // nebular age axis: warp per nebular SSP age, lanes over the window's
