@@ -374,25 +374,53 @@ struct RoundArgs {
   uint32_t k0, k1;
 };
 
-__device__ __forceinline__ void write_row(const RoundArgs& a, int c, const float* x, int lane) {
-  for (int j = lane; j < a.d; j += 32)
-    a.th_b[(size_t)c * a.d + j] = (float)(a.lo[j] + (double)x[j] * (a.hi[j] - a.lo[j]));
+// Columns of the directions' factor kept in shared memory by k_nss_round
+constexpr int ROUND_CHOL = 64;
+// Shared memory of k_nss_round in bytes: per chain normals, proposal, direction
+// and current point, then the factor
+size_t round_smem_bytes(int d, bool full) {
+  return 4ull * (CHAINS_PER_BLOCK * 4 * d + (full && d <= ROUND_CHOL ? d * d : 0));
 }
 
 // One warp per chain: consume the chain's last likelihood, advance its slice
 // state machine to its next proposal (proposals outside the unit cube are
-// decided without an evaluation) and write it as a parameter row.
+// decided without an evaluation) and write it as a parameter row.  The kernel is
+// one chain of dependent steps, so what any of them may need (the point, the
+// direction, the factor, the prior's box) is loaded at once at its start, and
+// the direction is not read back from global memory.
 __global__ void __launch_bounds__(CHAINS_PER_BLOCK * 32) k_nss_round(RoundArgs a) {
-  extern __shared__ float zsh[];                       // [CHAINS_PER_BLOCK][d] normals, then x
+  sed::pdl_enter();
+  extern __shared__ float zsh[];                       // [CHAINS_PER_BLOCK][4][d], then the factor
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int c = blockIdx.x * CHAINS_PER_BLOCK + warp;
   if (blockIdx.x == 0 && threadIdx.x == 0) a.st->active[(a.round + 1) & 1] = 0;
-  if (c >= a.k) return;
-  float* z = zsh + (size_t)warp * 2 * a.d;
-  float* x = z + a.d;
   const int d = a.d;
-  float* x0 = a.ch.x0 + (size_t)c * d;
-  float* v = a.ch.v + (size_t)c * d;
+  float* z = zsh + (size_t)warp * 4 * d;
+  float* x = z + d;
+  float* v = x + d;
+  float* x0 = v + d;
+  const float* chol = a.chol;
+  if (a.full && d <= ROUND_CHOL) {
+    float* L = zsh + CHAINS_PER_BLOCK * 4 * d;
+    for (int j = threadIdx.x; j < d * d; j += CHAINS_PER_BLOCK * 32) L[j] = a.chol[j];
+    chol = L;
+  }
+  double box_lo = 0.0, box_hi = 0.0;   // the lane's first column
+  if (lane < d) { box_lo = a.lo[lane]; box_hi = a.hi[lane]; }
+  if (c < a.k)
+    for (int j = lane; j < d; j += 32) {
+      x0[j] = a.ch.x0[(size_t)c * d + j];
+      v[j] = a.ch.v[(size_t)c * d + j];
+    }
+  __syncthreads();
+  if (c >= a.k) return;
+  auto write_row = [&](const float* p) {
+    for (int j = lane; j < d; j += 32) {
+      const double lo = j == lane ? box_lo : a.lo[j], hi = j == lane ? box_hi : a.hi[j];
+      a.th_b[(size_t)c * d + j] = (float)(lo + (double)p[j] * (hi - lo));
+    }
+  };
+  bool moved = false, turned = false;   // the point, the direction to be written back
   int ph = a.ch.phase[c], s = a.ch.step[c], nl = a.ch.nl[c], nr = a.ch.nr[c], ns = a.ch.ns[c];
   float tL = a.ch.tL[c], tR = a.ch.tR[c], t = a.ch.t[c];
   uint32_t draw = a.ch.draw[c];
@@ -411,6 +439,7 @@ __global__ void __launch_bounds__(CHAINS_PER_BLOCK * 32) k_nss_round(RoundArgs a
       } else if (ph == PH_SHRINK) {
         if (inside) {
           for (int j = lane; j < d; j += 32) x0[j] = fmaf(t, v[j], x0[j]);
+          moved = true;
           if (lane == 0) a.ch.lnl0[c] = lc;
           ++s;
           ph = PH_NEW;
@@ -448,13 +477,14 @@ __global__ void __launch_bounds__(CHAINS_PER_BLOCK * 32) k_nss_round(RoundArgs a
       for (int i = lane; i < d; i += 32) {
         float acc = 0.f;
         if (a.full) {
-          const float* Li = a.chol + (size_t)i * d;
+          const float* Li = chol + (size_t)i * d;
           for (int j = 0; j <= i; ++j) acc = fmaf(Li[j], z[j], acc);
         } else {
-          acc = a.chol[i] * z[i];
+          acc = chol[i] * z[i];
         }
         v[i] = acc * rz;
       }
+      turned = true;
       const uint4 r = philox(make_uint4((uint32_t)a.iter, (uint32_t)c, draw++, TAG_SLICE), a.k0, a.k1);
       tL = -u01(r.x) * a.w;
       tR = tL + a.w;
@@ -481,11 +511,15 @@ __global__ void __launch_bounds__(CHAINS_PER_BLOCK * 32) k_nss_round(RoundArgs a
       inside = false;
       continue;
     }
-    write_row(a, c, x, lane);
+    write_row(x);
     wrote = true;
     break;
   }
-  if (!wrote) write_row(a, c, x0, lane);   // an idle row (done chain): evaluated, not used
+  for (int j = lane; j < d; j += 32) {
+    if (moved) a.ch.x0[(size_t)c * d + j] = x0[j];
+    if (turned) a.ch.v[(size_t)c * d + j] = v[j];
+  }
+  if (!wrote) write_row(x0);   // an idle row (done chain): evaluated, not used
   if (lane == 0) {
     a.ch.phase[c] = ph; a.ch.step[c] = s; a.ch.nl[c] = nl; a.ch.nr[c] = nr; a.ch.ns[c] = ns;
     a.ch.tL[c] = tL; a.ch.tR[c] = tR; a.ch.t[c] = t; a.ch.draw[c] = draw;
@@ -648,7 +682,7 @@ sed_status sed_nss_run(sed_ctx* ctx, sed_model_id model, const sed_nss_desc* des
   const float w = desc->slice_width > 0.0 ? (float)desc->slice_width : sqrtf((float)d + 2.f);
   const size_t sel_smem = sel_smem_bytes(n, k, d, full);
   const size_t fin_smem = 20ull * n;
-  const size_t round_smem = 4ull * CHAINS_PER_BLOCK * 2 * d;
+  const size_t round_smem = round_smem_bytes(d, full);
   static DynSmemCache a_sel, a_fin, a_round;
   const long long max_rounds = (long long)desc->n_slice_steps * (2 * MAXOUT + MAXSHRINK) + 4;
   long long n_rows = n;
@@ -683,8 +717,8 @@ sed_status sed_nss_run(sed_ctx* ctx, sed_model_id model, const sed_nss_desc* des
     while (!done && !ret) {
       for (int q = 0; q < ROUNDS && !ret; ++q, ++r) {
         ra.round = (int)(r & 1);
-        k_nss_round<<<(k + CHAINS_PER_BLOCK - 1) / CHAINS_PER_BLOCK, CHAINS_PER_BLOCK * 32, round_smem, s>>>(ra);
-        if (!CKE(cudaGetLastError())) break;
+        if (!CKE(sed::launch_pdl(k_nss_round, dim3((k + CHAINS_PER_BLOCK - 1) / CHAINS_PER_BLOCK),
+                                 dim3(CHAINS_PER_BLOCK * 32), round_smem, s, ra))) break;
         ret = sed_loglike(ctx, model, th_b, k, d, lnl_b, st_b, desc->precision, stream);
         n_rows += k;
       }
