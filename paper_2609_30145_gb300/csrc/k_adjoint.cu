@@ -74,10 +74,10 @@ __device__ __forceinline__ void put_g(const EpiBwdArgs& a, float* hi, float* lo,
 constexpr size_t EB_CAL_BYTES = (size_t)EB_WARPS * CAL_NV * sizeof(float) +
                                 (size_t)(SED_MAX_CALIB * SED_MAX_CALIB + 2 * SED_MAX_CALIB) * sizeof(float);
 
-// bytes of the pixels' arrays: 4 floats + node range; with a sampled stellar
-// dispersion also dmu/ds; with a calibration polynomial mu/sigma, dmu/dx, dmu/ds, 1/sum w
+// bytes of the pixels' arrays: 4 floats + node range; with a calibration
+// polynomial also mu/sigma, dmu/dx, dmu/ds, 1/sum w
 __host__ __device__ __forceinline__ size_t epi_bwd_pix(const ModelDev& md) {
-  return (size_t)md.n_pix * (md.calib_n ? 36 : md.sample_sgal ? 24 : 20);
+  return (size_t)md.n_pix * (md.calib_n ? 36 : 20);
 }
 
 size_t epi_bwd_lines_off(const EpiBwdArgs& a) {   // bytes, 8-aligned
@@ -151,8 +151,8 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
   // 1/sum w, then the per-warp moments, the Cholesky factor and c*
   float* mu_s = reinterpret_cast<float*>(prg + md.n_pix);
   float* dv_s = mu_s + md.n_pix;
-  float* dvs_s = md.calib_n ? dv_s + md.n_pix : mu_s;
-  float* cw_s = dv_s + 2 * md.n_pix;
+  float* dvs_s = dv_s + md.n_pix;
+  float* cw_s = dvs_s + md.n_pix;
   float *cal_part = nullptr, *cal_Lf = nullptr, *cal_Df = nullptr, *cal_cf = nullptr;
   if (md.calib_n) {
     const size_t samp = (size_t)md.n_samp * 8, pix = epi_bwd_pix(md);
@@ -526,9 +526,12 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
           dv[q] = (sfu[q] * sw[q] - sf[q] * swu[q]) * n;
           dvs[q] = (sfq[q] * sw[q] - sf[q] * swq[q]) * n;
           cw[q] = 1.f / sw[q];
+          if (md.sample_sgal) {
+            cw[q] = -cw[q];
+            tl[q] = dvs[q];
+          }
         }
         px4[i] = make_float4(v[q], dv[q], cw[q], tl[q]);
-        if (md.sample_sgal) dvs_s[i] = dvs[q];
         if (LINES && NLn) upx[i] = la[q] * md.pix_lamc[i];
         prg[i] = (jlo[q] & 0xffff) | (jhi[q] << 16);
       }
@@ -536,9 +539,13 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
     __syncthreads();
   }
   for (int i = tid; i < md.n_pix; i += EB_THREADS) {
-    const float4 pv = px4[i];   // {v, dv/dx, 1/sum w (0: no node reached), t or -1 - 1/sigma}
-    const float v = pv.x, dv = pv.y, cw = pv.z, tl = pv.w, dvs = md.sample_sgal ? dvs_s[i] : 0.f;
+    // {v, dv/dx, 1/sum w (0: no node reached), t or -1 - 1/sigma}; a Gaussian row of a
+    // sampled dispersion has -1/sum w and dv/ds (1/sigma follows from the row's)
+    const float4 pv = px4[i];
+    const float v = pv.x, dv = pv.y, cw = fabsf(pv.z), dvs = pv.z < 0.f ? pv.w : 0.f;
     const bool valid = cw != 0.f;
+    float tl = pv.w;
+    if (pv.z < 0.f) tl = -1.f - 1.f / sqrtf(md.pix_fix2[i] + rs.sg_ln * rs.sg_ln);
     const float mline = LINES && NLn ? upx[i] : 0.f;
     const float mi = LINES && NLn ? fmaf(rs.s_spec, v, mline) : rs.s_spec * v;
     float ci = 0.f;
