@@ -99,8 +99,9 @@ size_t epi_bwd_smem(const EpiBwdArgs& a) {
 // LINES: an instance with the emission lines (the one without keeps its code free of them);
 // VAR: 1 the age-binned attenuation (one Y and one dlnL/dY per attenuated
 // block), 2 the nebular age axis (per-age ionising weights); 0 neither
-template <bool LINES, int VAR = 0>
-__global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant__ EpiBwdArgs a) {
+// NT threads per row: 256, or 512 without pixels (below)
+template <bool LINES, int VAR = 0, int NT = EB_THREADS>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_epi_bwd(const __grid_constant__ EpiBwdArgs a) {
   pdl_enter();
   const ModelDev& md = a.md;
   const GridDev& g = a.g;
@@ -111,14 +112,14 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
   __shared__ float ubp[EB_MAX_BANDS], mbp[EB_MAX_BANDS];
   __shared__ int bk0[EB_MAX_BANDS], bk1[EB_MAX_BANDS];
   __shared__ float mlb[EB_MAX_BANDS], ubm[EB_MAX_BANDS];   // lines: each band's line part, dlnL/dm_b
-  __shared__ double red[EB_WARPS][EB_NRED + EB_NREDB];
+  __shared__ double red[(NT / 32)][EB_NRED + EB_NREDB];
 
   if (a.win_reset && r == 0) empty_windows(a.win_reset, a.win_mt);
   const size_t ro = (size_t)r * a.ldn;
   RowScal rs = a.rs[r];
   if (a.err && *a.err) rs.status |= SED_ROW_DEVICE_TIMEOUT;
   if (rs.status) {
-    for (int k = tid; k < a.ldn; k += EB_THREADS) {
+    for (int k = tid; k < a.ldn; k += NT) {
       for (int sg = 0; sg < (VAR == 1 ? md.n_seg : 1); ++sg) {
         a.gy_hi[sg * a.seg_stride + ro + k] = 0.f;
         if (a.split) a.gy_lo[sg * a.seg_stride + ro + k] = 0.f;
@@ -158,7 +159,7 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
     const size_t samp = (size_t)md.n_samp * 8, pix = epi_bwd_pix(md);
     const size_t u = ((samp > pix ? samp : pix) + 7) & ~(size_t)7;
     cal_part = reinterpret_cast<float*>(reinterpret_cast<char*>(U) + u);
-    cal_Lf = reinterpret_cast<float*>(cal_part + EB_WARPS * CAL_NV);
+    cal_Lf = reinterpret_cast<float*>(cal_part + (NT / 32) * CAL_NV);
     cal_Df = cal_Lf + SED_MAX_CALIB * SED_MAX_CALIB;   // after L
     cal_cf = cal_Df + SED_MAX_CALIB;
   }
@@ -182,7 +183,7 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
   __shared__ float qa_s[MAX_NEB_AGE], gqa_s[MAX_NEB_AGE];
   const float* qa = nullptr;
   if constexpr (VAR == 2) {
-    for (int i = tid; i < g.neb_na; i += EB_THREADS) qa_s[i] = a.qneb[(size_t)r * MAX_NEB_AGE + i];
+    for (int i = tid; i < g.neb_na; i += NT) qa_s[i] = a.qneb[(size_t)r * MAX_NEB_AGE + i];
     __syncthreads();
     qa = qa_s;
   }
@@ -191,7 +192,7 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
   //      arithmetic); phi holds the window's wavelengths until the photometric
   //      gather starts
   if constexpr (VAR != 1)   // Y and O of all the thread's nodes into the nodes' own places at once
-    for (int k = k_lo + tid; k <= k_hi; k += EB_THREADS) {
+    for (int k = k_lo + tid; k <= k_hi; k += NT) {
       cp_async4(Fs + k, Yr + k);
       cp_async4(phi + k, Or + k);
     }
@@ -208,7 +209,7 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
   load_node(k_lo + tid, O2r, nx);
   // dlnL/dY and dlnL/dO are zero outside the window, four nodes at a time (the
   // rows and the window's ends within four are the dust pass's)
-  for (int q = 4 * tid; q < a.ldn; q += 4 * EB_THREADS) {
+  for (int q = 4 * tid; q < a.ldn; q += 4 * NT) {
     if (q + 3 >= k_lo && q <= k_hi) continue;
     const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int sg = 0; sg < (VAR == 1 ? md.n_seg : 1); ++sg) {
@@ -220,9 +221,9 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
   }
   cp_async_wait_all();
 #pragma unroll 1
-  for (int k = k_lo + tid; k <= k_hi; k += EB_THREADS) {
+  for (int k = k_lo + tid; k <= k_hi; k += NT) {
     const Node n = nx;
-    load_node(k + EB_THREADS, O2r, nx);
+    load_node(k + NT, O2r, nx);
     if constexpr (VAR == 1) {
       float yv[MAX_SEG];
 #pragma unroll
@@ -239,12 +240,12 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
     }
     phi[k] = n.c.w;
   }
-  for (int l = tid; l < NLn; l += EB_THREADS) line_setup(md, g, rs, eb_kc, l, ln_F, ln_A, ln_is, ln_x);
+  for (int l = tid; l < NLn; l += NT) line_setup(md, g, rs, eb_kc, l, ln_F, ln_A, ln_is, ln_x);
   __syncthreads();
   // the catalogue entries' sigma dlnL/dm = (d - m)/sigma, 0 for a respected
   // upper limit or an entry outside the mask (Eq. app_line_chi2_det,
   // app_line_chi2_UL)
-  for (int k = tid; k < md.n_lcat; k += EB_THREADS) {
+  for (int k = tid; k < md.n_lcat; k += NT) {
     const double is = md.lcat_isig[k];
     float m = 0.f;
     for (int j = md.lcat_start[k]; j < md.lcat_start[k + 1]; ++j) m += ln_F[md.lcat_line[j]];
@@ -268,7 +269,7 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
   const bool pick = slack <= 0.25f && k_hi - k_lo >= 2 && md.samp_lam_min * rs.inv1pz >= lam0 &&
                     md.samp_lam_max * rs.inv1pz <= lamN;
   const float q_mul = 0.6931471805599453f * g.lut_inv_h, q_add = fmaf(-g.lut_x0, g.lut_inv_h, -slack);
-  for (int b = warp; b < md.n_filt; b += EB_WARPS) {
+  for (int b = warp; b < md.n_filt; b += (NT / 32)) {
     const int js = md.band_start[b], je = md.band_start[b + 1];
     float acc = 0.f, gzb = 0.f;
     int bmin = 0x7fffffff, bmax = -1;
@@ -371,7 +372,7 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
   //      alone on its SM.  With the photometry above and the loads ahead: 2048 rows
   //      with a spectrum 353 -> 300 us, 200 photometric rows 62 -> 46 us.)
   {
-    const int run = (nw + EB_WARPS - 1) / EB_WARPS;
+    const int run = (nw + (NT / 32) - 1) / (NT / 32);
     const int n0 = k_lo + warp * run, n1 = min(n0 + run, k_hi + 1);   // this warp's nodes [n0, n1)
     for (int k = n0 + lane; k < n1; k += 32) phi[k] = 0.f;
     __syncwarp();
@@ -441,7 +442,7 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
   if (md.n_pix > 0) {
     const float ll0 = g.lnl_hi[0], llN = g.lnl_hi[N - 1];
     const int last = md.n_pix - 1;
-    for (int ib = 2 * 32 * warp; ib < md.n_pix; ib += 2 * EB_THREADS) {
+    for (int ib = 2 * 32 * warp; ib < md.n_pix; ib += 2 * NT) {
       float2 pl[2];
       float xh[2], xl[2], inv_s[2], v[2], dv[2], dvs[2], cw[2], tl[2];
       float sw[2], sf[2], swu[2], sfu[2], swq[2], sfq[2];
@@ -538,7 +539,7 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
     }
     __syncthreads();
   }
-  for (int i = tid; i < md.n_pix; i += EB_THREADS) {
+  for (int i = tid; i < md.n_pix; i += NT) {
     // {v, dv/dx, 1/sum w (0: no node reached), t or -1 - 1/sigma}; a Gaussian row of a
     // sampled dispersion has -1/sum w and dv/ds (1/sigma follows from the row's)
     const float4 pv = px4[i];
@@ -600,26 +601,26 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
     //      d lnL / d mu_i = [(d_i - mu_i (1 + p_i)) (1 + p_i) - mu_i q_i] / sigma_i^2
     //      (all in FP32 on the normalised values),
     //      p = A c*, q_i = |L^-1 T(x_i)|^2 (M = L L^T)
-    calib_block<0, 0, EB_THREADS>(md, mu_s, cal_cf, tid, lane, warp, cal_part);
-    calib_block<SED_MAX_CALIB, 0, EB_THREADS>(md, mu_s, cal_cf, tid, lane, warp, cal_part);
-    calib_block<0, 1, EB_THREADS>(md, mu_s, cal_cf, tid, lane, warp, cal_part);
+    calib_block<0, 0, NT>(md, mu_s, cal_cf, tid, lane, warp, cal_part);
+    calib_block<SED_MAX_CALIB, 0, NT>(md, mu_s, cal_cf, tid, lane, warp, cal_part);
+    calib_block<0, 1, NT>(md, mu_s, cal_cf, tid, lane, warp, cal_part);
     __syncthreads();
     if (warp == 0) {
-      const double f = calib_first_solve(md, cal_part, EB_WARPS, cal_Lf, cal_Df, cal_cf, lane);
+      const double f = calib_first_solve(md, cal_part, (NT / 32), cal_Lf, cal_Df, cal_cf, lane);
       if (lane == 0) l_spec += f;
     }
     __syncthreads();
     // one refinement of c* from the pixels' calibrated residuals (the gradient
     // takes c* at first order)
-    calib_block<0, 2, EB_THREADS>(md, mu_s, cal_cf, tid, lane, warp, cal_part);
+    calib_block<0, 2, NT>(md, mu_s, cal_cf, tid, lane, warp, cal_part);
     __syncthreads();
     if (warp == 0) {
-      const double f = calib_refine(md, cal_part, EB_WARPS, cal_Lf, cal_Df, cal_cf, lane);
+      const double f = calib_refine(md, cal_part, (NT / 32), cal_Lf, cal_Df, cal_cf, lane);
       if (lane == 0) l_spec += f;
     }
     __syncthreads();
     const int n = md.calib_n;
-    for (int i = tid; i < md.n_pix; i += EB_THREADS) {
+    for (int i = tid; i < md.n_pix; i += NT) {
       const float m = mu_s[i];
       if (m == 0.f) {
         if (NLn) upx[i] = 0.f;
@@ -678,15 +679,15 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
   if (md.n_pix > 0) {
     const int P = md.n_pix;
     int mono = 1, linear = 0;
-    for (int i = tid; i < P; i += EB_THREADS) linear |= px4[i].w > -0.5f && px4[i].z != 0.f;
-    for (int i = tid + 1; i < P; i += EB_THREADS) {
+    for (int i = tid; i < P; i += NT) linear |= px4[i].w > -0.5f && px4[i].z != 0.f;
+    for (int i = tid + 1; i < P; i += NT) {
       const int r0 = prg[i - 1], r1 = prg[i];
       if ((r1 & 0xffff) < (r0 & 0xffff) || (r1 >> 16) < (r0 >> 16)) mono = 0;
     }
     mono = __syncthreads_and(mono);
     linear = __syncthreads_or(linear);
     const float R = 5.f * md.pix_s_max * 1.0001f + g.dln_max * 1.0001f + 1e-6f;
-    for (int k0 = mono ? k_lo + 2 * tid : k_hi + 1; k0 <= k_hi; k0 += 2 * EB_THREADS) {
+    for (int k0 = mono ? k_lo + 2 * tid : k_hi + 1; k0 <= k_hi; k0 += 2 * NT) {
       const int k1 = min(k0 + 1, k_hi);
       const float2 n0 = __ldg(g.lnl2 + k0), n1 = __ldg(g.lnl2 + k1);
       int pa = 0, pe = P;
@@ -726,7 +727,7 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
       phi[k0] += acc0;
       if (k1 > k0) phi[k1] += acc1;
     }
-    for (int k = mono ? k_hi + 1 : k_lo + tid; k <= k_hi; k += EB_THREADS) {
+    for (int k = mono ? k_hi + 1 : k_lo + tid; k <= k_hi; k += NT) {
       const float lh = g.lnl_hi[k], ll = g.lnl_lo[k];
       float acc = 0.f;
       int p = 0, p1 = P;
@@ -767,7 +768,7 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
   //      G = B dlnL/dF, Gx and Gs the centre's and width's (per unit of Q fac)
   //      from the pixels within 5 s_l (pixel order), every band (in order) and
   //      the catalogue entries naming the line; then to the parameters
-  for (int l = tid; l < NLn; l += EB_THREADS) {
+  for (int l = tid; l < NLn; l += NT) {
     const float is = ln_is[l];
     const float2 xlp = ln_x[l];
     const float4 c = g.line_att4[l];
@@ -873,7 +874,7 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
   if constexpr (VAR == 1) {
     // F = e^{-tau_d} [ sum_s A_s (Y_s + Q_s neb) + O + Q_rest neb ], A_s = e^{-tau_s},
     // tau_s = sum_b M_sb tau_b shape_b (atten.cuh's attenuated_bins)
-    for (int k = d_lo + tid; k <= d_hi; k += EB_THREADS) {
+    for (int k = d_lo + tid; k <= d_hi; k += NT) {
       if (k < k_lo || k > k_hi) {
         for (int sg = 0; sg < md.n_seg; ++sg) put_g(a, a.gy_hi, a.gy_lo, sg * a.seg_stride + ro + k, 0.f);
         put_g(a, a.go_hi, a.go_lo, ro + k, 0.f);
@@ -968,9 +969,9 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
   }
   load_node(k_lo + tid, Yr, nx);
 #pragma unroll 1
-  for (int k = k_lo + tid; k <= k_hi; k += EB_THREADS) {
+  for (int k = k_lo + tid; k <= k_hi; k += NT) {
     const Node n = nx;
-    load_node(k + EB_THREADS, Yr, nx);
+    load_node(k + NT, Yr, nx);
     const float4 c = n.c;
     const float lnp = c.x;
     const float pa = __expf(rs.alpha_bc * lnp);
@@ -1057,7 +1058,7 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
     // at node k (phi), e_a(k) = 10^(the cube at age a)
     __syncthreads();
     const size_t plane = (size_t)g.neb_nu * g.neb_nz * N;
-    for (int i = warp; i < g.neb_na; i += EB_WARPS) {
+    for (int i = warp; i < g.neb_na; i += (NT / 32)) {
       const float q = qa[i];
       const float* tb = g.neb_tab + i * plane;
       float sq = 0.f;
@@ -1124,7 +1125,7 @@ __global__ void __launch_bounds__(EB_THREADS, 4) k_epi_bwd(const __grid_constant
   if (warp == 0) {
     double col = 0.0;
     if (lane < (VAR == 1 ? EB_NRED + EB_NREDB : EB_NRED))
-      for (int w = 0; w < EB_WARPS; ++w) col += red[w][lane];
+      for (int w = 0; w < (NT / 32); ++w) col += red[w][lane];
     // the photometric lnL terms and d lnL/d ln(mass) pieces in FP64, one band per lane
     double bl = 0.0, bu = 0.0, gfp[4] = {0.0, 0.0, 0.0, 0.0};
     for (int b = lane; b < md.n_filt; b += 32) {
@@ -1199,7 +1200,18 @@ cudaError_t launch_epilogue_bwd(const EpiBwdArgs& a_in, size_t* smem_needed, cud
   a.lines_off = (int)epi_bwd_lines_off(a);
   const size_t smem = epi_bwd_smem(a);
   if (smem_needed) *smem_needed = smem;
-  static DynSmemCache set_for[4];
+  static DynSmemCache set_for[6];
+  // Without pixels a row is a chain of loads over its nodes and samples with
+  // hardly a sum, and 512 threads are as many warps per SM as 256 (2 CTAs
+  // instead of 4): the gradient of 200 rows 120 -> 105 us.  With pixels the 256 threads' order of the sums over
+  // them is part of lnL.
+  if (a.md.n_pix == 0 && a.md.n_bin == 0 && !a.qneb) {
+    const bool lines = a.md.use_lines != 0;
+    auto k = lines ? k_epi_bwd<true, 0, 2 * EB_THREADS> : k_epi_bwd<false, 0, 2 * EB_THREADS>;
+    cudaError_t e = ensure_dyn_smem(k, smem, &set_for[lines ? 5 : 4]);
+    if (e == cudaSuccess) return launch_pdl(k, dim3(a.n), dim3(2 * EB_THREADS), smem, s, a);
+    if (e != cudaErrorInvalidConfiguration) return e;   // its sums over more warps may be what does not fit
+  }
   const int m = a.md.n_bin > 0 ? 2 : a.qneb ? 3 : (a.md.use_lines ? 1 : 0);
   auto k = m == 3 ? k_epi_bwd<false, 2> : m == 2 ? k_epi_bwd<false, 1> : (m == 1 ? k_epi_bwd<true> : k_epi_bwd<false>);
   cudaError_t e = ensure_dyn_smem(k, smem, &set_for[m]);
