@@ -191,7 +191,7 @@ struct Params {
   float* O2;                 // forward, persistent schedule: second half of the old part when the
                              // launch splits its tiles three ways (NULL: never split)
   int* split_out;            // forward: the launch's choice (1 = split, O + O2 is the old part), or NULL
-  const int* tile_win;       // forward, persistent schedule: [2][m_tiles] window (lo, hi) of each M tile
+  const int* tile_win;       // forward, persistent schedule: [m_tiles][2] window of each M tile (WIN_EMPTY)
   int m_tiles;
   const uint32_t* kmask;     // [m_tiles][kmask_w] K tiles some row of the M tile touches (NULL: all);
   int kmask_w;               // adjoint: 32-column tiles of dW's columns
@@ -449,7 +449,8 @@ __global__ void __launch_bounds__(192, 1) k_contract_tc(const __grid_constant__ 
     // which tile or tile position computes it.
     const int MT = p.m_tiles;
     if (threadIdx.x < MT) {
-      const int lo = p.tile_win[threadIdx.x], hi = p.tile_win[MT + threadIdx.x];
+      const int2 tw = reinterpret_cast<const int2*>(p.tile_win)[threadIdx.x];
+      const int lo = tw.x, hi = ~tw.y;
       int a = 0, c = 0;
       if (hi >= 0) {
         a = lo & ~15;

@@ -390,7 +390,7 @@ struct OrderArgs {
   const int* row_model;   // NULL: every row uses md
   int by_pair;       // 1: two redshift halves, bracket pair, then redshift
   int n_pairs;       // bracket pairs (by_pair)
-  int* tile_win;     // set to empty windows by CTA 0 (lo = 0x7f7f7f7f, hi = -1), or NULL
+  int* tile_win;     // set to empty windows by CTA 0, or NULL
   uint32_t* kmask;   // cleared by CTA 0, or NULL
   int mt, kmask_w;   // 128-row tiles; mask words per tile
 };
@@ -400,10 +400,7 @@ __global__ void __launch_bounds__(ORDER_THREADS) k_order(const __grid_constant__
   // the per-tile windows and K-tile masks the preparation kernel accumulates
   // into start empty (done here rather than by separate memsets)
   if (blockIdx.x == 0) {
-    for (int i = threadIdx.x; i < oa.mt && oa.tile_win; i += ORDER_THREADS) {
-      oa.tile_win[i] = 0x7f7f7f7f;
-      oa.tile_win[oa.mt + i] = -1;
-    }
+    if (oa.tile_win) empty_windows(oa.tile_win, oa.mt);
     for (int i = threadIdx.x; i < oa.mt * oa.kmask_w && oa.kmask; i += ORDER_THREADS) oa.kmask[i] = 0u;
   }
   __shared__ int cnt[ORDER_BINS + 1];
@@ -929,11 +926,7 @@ __global__ void __launch_bounds__(PREP_THREADS, 8) k_prep(const __grid_constant_
           rs.bin_tau[b] = th[md.offs[SED_KEY_DUST_BINS] + 2 * b];
           rs.bin_slope[b] = th[md.offs[SED_KEY_DUST_BINS] + 2 * b + 1];
         }
-      if (a.tile_win) {   // union of the windows of this row's 128-row tile
-        const int mt = (a.n + 127) >> 7;
-        atomicMin(&a.tile_win[p >> 7], win_lo);
-        atomicMax(&a.tile_win[mt + (p >> 7)], win_hi);
-      }
+      if (a.tile_win) add_to_window(a.tile_win, p >> 7, win_lo, win_hi);   // the row's 128-row tile
     }
   }
   // the passes below read the weights with every warp
@@ -1327,10 +1320,7 @@ cudaError_t launch_prep(const PrepArgs& p, cudaStream_t s) {
   const bool self = ordered && p.self_order && !p.row_model && p.n <= (by_pair ? SELF_PAIR_MAX : SELF_ORDER_MAX);
   const bool order = ordered && !self && p.perm;
   if (!order && !p.self_order) {   // nothing before this kernel to start the windows and masks empty
-    if (p.tile_win) {
-      e = cudaMemsetAsync(p.tile_win, 0x7f, mt * sizeof(int), s);
-      if (e == cudaSuccess) e = cudaMemsetAsync(p.tile_win + mt, 0xff, mt * sizeof(int), s);
-    }
+    if (p.tile_win) e = cudaMemsetAsync(p.tile_win, WIN_EMPTY_BYTE, 2 * mt * sizeof(int), s);
     if (e == cudaSuccess && p.kmask) e = cudaMemsetAsync(p.kmask, 0, (size_t)mt * p.kmask_w * sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
   }

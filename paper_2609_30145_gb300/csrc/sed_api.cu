@@ -1373,8 +1373,7 @@ sed::Workspace* get_ws(sed_ctx* ctx, void* stream, int rows, int kpad, int ldn, 
   if (!s) {   // the error words cleared, the per-tile windows and masks empty (k_prep expects it)
     cudaError_t e = cudaMemset(w->err, 0, 64);
     const size_t mt = (R + 127) / 128;
-    if (e == cudaSuccess) e = cudaMemset(w->tile_win, 0x7f, mt * sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(w->tile_win + mt, 0xff, mt * sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(w->tile_win, WIN_EMPTY_BYTE, 2 * mt * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(w->kmask, 0, mt * KMASK_WORDS * sizeof(uint32_t));
     if (e != cudaSuccess) s = fail(ctx, SED_ECUDA, "cudaMemset: %s", cudaGetErrorString(e));
   }
@@ -1640,7 +1639,7 @@ sed_status sed_loglike_host(sed_ctx* ctx, sed_model_id id, const float* theta, i
   // all buffers in place, on a caller's stream (capture is not possible on the
   // legacy default stream), not profiling: the second identical call captures
   // its launches into a CUDA graph, later ones replay it (one launch instead of
-  // two memsets and four kernels)
+  // four kernels)
   if (th_d && lnl_d && (!row_status || st_d) && stream && !ctx->profiling) {
     Workspace::HostKey k;
     k.model = id; k.mp = M; k.th = th_d; k.lnl = lnl_d; k.st = st_d; k.n = n; k.ld = ld; k.prec = precision;

@@ -353,7 +353,7 @@ struct Workspace {
   float* W_hi = nullptr;         // [rows][Kpad]
   float* W_lo = nullptr;
   int* perm = nullptr;           // [rows] processing order
-  int* tile_win = nullptr;       // [2][ceil(rows/128)] per-tile node windows
+  int* tile_win = nullptr;       // [ceil(rows/128)][2] per-tile node windows (WIN_EMPTY)
   uint32_t* kmask = nullptr;     // [ceil(rows/128)][KMASK_WORDS] per-tile K-tile occupancy
   int kmask_w_call = 0;          // words per tile of the current call's masks (0: the call has none)
   // The K tiles of W_hi/W_lo row p that may hold non-zeros (bit set), for the
@@ -467,8 +467,8 @@ struct PrepArgs {
   RowScal* rs;
   int* err;            // device error word of the contraction, cleared by the prep kernel
   int* perm;           // [n] scratch: processing order (rows sorted by redshift), or NULL = caller's order
-  int* tile_win;       // [2][ceil(n/128)] union of the row windows of each 128-row tile (launch_prep
-                       // starts them empty: lo 0x7f7f7f7f, hi -1), or NULL
+  int* tile_win;       // [ceil(n/128)][2] union of the row windows of each 128-row tile (WIN_EMPTY;
+                       // launch_prep starts them empty), or NULL
   uint32_t* kmask;     // [ceil(n/128)][kmask_w] K tiles that some row of each 128-row tile touches
                        // (launch_prep clears them), or NULL
   int kmask_w;         // words per 128-row tile (<= KMASK_WORDS)
@@ -482,14 +482,22 @@ struct PrepArgs {
                        // (each CTA reads every row's keys); done for one fit of n <= SELF_ORDER_MAX
   int by_pair, n_pairs;   // set by launch_prep: rows ordered by bracket pair, and the pairs there are
 };
-// Per-tile windows (lo, hi) of the contraction back to empty (lo 0x7f7f7f7f,
-// hi -1) once their reader has finished, by one CTA, so that the next call's
-// prep kernel can fill them without an ordering kernel or memsets before it.
+// A 128-row tile's node window is two words side by side, its first node and the
+// complement of its last one, both taken as minima over the tile's rows and both
+// WIN_EMPTY without any (bytes of one value: a memset).  A word's place and its
+// empty value then do not depend on how many tiles a call has, so what one call
+// leaves empty is empty for the next call of any size, and a window left
+// filled (a call that failed on the way) only widens the next one's.
+constexpr int WIN_EMPTY_BYTE = 0x7f, WIN_EMPTY = 0x7f7f7f7f;
+__device__ __forceinline__ void add_to_window(int* win, int tile, int lo, int hi) {
+  atomicMin(&win[2 * tile], lo);
+  atomicMin(&win[2 * tile + 1], ~hi);
+}
+// The windows of mt tiles back to empty once their reader (the contraction) has
+// finished, by one CTA, so that the next call's prep kernel can fill them
+// without an ordering kernel or a memset before it.
 __device__ __forceinline__ void empty_windows(int* win, int mt) {
-  for (int i = threadIdx.x; i < mt; i += blockDim.x) {
-    win[i] = 0x7f7f7f7f;
-    win[mt + i] = -1;
-  }
+  for (int i = threadIdx.x; i < 2 * mt; i += blockDim.x) win[i] = WIN_EMPTY;
 }
 // A pixel's rest-frame ln(lambda) = ln(lambda_obs) - ln(1+z), both given as
 // FP32 pairs {hi, lo}, returned as an FP32 pair: the high parts' difference is
@@ -673,7 +681,7 @@ struct EpiArgs {
   int samp_off, res_off;   //   the samples' values and the pixels' residuals
   size_t seg_stride;   // age-binned dust: Y of attenuated block s at Y + s seg_stride
   const float* qneb;   // nebular age axis: [n][MAX_NEB_AGE] (k_prep's), or NULL
-  int* win_reset;      // [2][win_mt] per-tile windows set back to empty by CTA 0 (the contraction,
+  int* win_reset;      // [win_mt][2] per-tile windows set back to empty by CTA 0 (the contraction,
   int win_mt;          // their reader, has finished), or NULL
   uint32_t* mask_reset;   // the K-tile masks likewise, mask_words of them
   int mask_words;

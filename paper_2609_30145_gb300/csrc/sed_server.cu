@@ -65,7 +65,7 @@ struct SrvSlot {
   float* theta = nullptr;       // [max_rows][SRV_LD]
   int* rowm = nullptr;          // [max_rows]
   int* perm = nullptr;          // [max_rows] processing order (rows grouped by redshift)
-  int* tile_win = nullptr;      // [2][ceil(max_rows/128)] node windows of the 128-row tiles
+  int* tile_win = nullptr;      // [ceil(max_rows/128)][2] node windows of the 128-row tiles (WIN_EMPTY)
   double* lnl = nullptr;
   uint32_t* st = nullptr;
   float *W = nullptr, *W_hi = nullptr, *W_lo = nullptr, *Y = nullptr, *O = nullptr, *O2 = nullptr;
