@@ -1370,12 +1370,13 @@ sed::Workspace* get_ws(sed_ctx* ctx, void* stream, int rows, int kpad, int ldn, 
     AL(dW, R * K * 4); AL(rgrad, R * RGRAD * 8);
   }
 #undef AL
-  if (!s) {   // the error words cleared, the per-tile windows and masks empty (k_prep expects it)
-    cudaError_t e = cudaMemset(w->err, 0, 64);
+  if (!s) {   // the error words cleared, the per-tile windows and masks empty (k_prep expects it), in the stream's order
+    const cudaStream_t cs = (cudaStream_t)stream;
     const size_t mt = (R + 127) / 128;
-    if (e == cudaSuccess) e = cudaMemset(w->tile_win, WIN_EMPTY_BYTE, 2 * mt * sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(w->kmask, 0, mt * KMASK_WORDS * sizeof(uint32_t));
-    if (e != cudaSuccess) s = fail(ctx, SED_ECUDA, "cudaMemset: %s", cudaGetErrorString(e));
+    cudaError_t e = cudaMemsetAsync(w->err, 0, 64, cs);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w->tile_win, WIN_EMPTY_BYTE, 2 * mt * sizeof(int), cs);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w->kmask, 0, mt * KMASK_WORDS * sizeof(uint32_t), cs);
+    if (e != cudaSuccess) s = fail(ctx, SED_ECUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
   }
   *st = s;
   return s ? nullptr : w;
