@@ -81,6 +81,14 @@ void free_all(sed_ctx* ctx, std::vector<void*>& v, size_t& acct) {
   acct = 0;
 }
 
+void free_ws_buffers(const Workspace* w) {
+  for (void* p : {(void*)w->perm, (void*)w->tile_win, (void*)w->kmask, (void*)w->W, (void*)w->W_hi, (void*)w->W_lo,
+                  (void*)w->W_bf16, (void*)w->W_f8, (void*)w->Y, (void*)w->O, (void*)w->O2, (void*)w->rs, (void*)w->err,
+                  (void*)w->wmask, (void*)w->theta_h, (void*)w->lnl_h, (void*)w->st_h, (void*)w->G_hi, (void*)w->G_lo,
+                  (void*)w->GO_hi, (void*)w->GO_lo, (void*)w->dW, (void*)w->rgrad, (void*)w->qneb})
+    if (p) cudaFree(p);
+}
+
 bool strictly_increasing(const double* x, int n) {
   for (int i = 0; i < n; i++)
     if (!std::isfinite(x[i]) || (i && !(x[i] > x[i - 1]))) return false;
@@ -215,11 +223,7 @@ sed_status sed_destroy(sed_ctx* ctx) {
     }
     for (auto& kv : ctx->ws) {
       Workspace* w = kv.second;
-      std::vector<void*> v = {w->perm, w->tile_win, w->kmask, w->W, w->W_hi, w->W_lo, w->W_bf16, w->W_f8, w->Y, w->O, w->O2, w->rs, w->err,
-                              w->wmask, w->theta_h, w->lnl_h, w->st_h, w->G_hi, w->G_lo, w->GO_hi, w->GO_lo,
-                              w->dW, w->rgrad, w->qneb};
-      for (void* p : v)
-        if (p) cudaFree(p);
+      free_ws_buffers(w);
       for (cudaEvent_t e : w->ev)
         if (e) cudaEventDestroy(e);
       if (w->host_exec) cudaGraphExecDestroy(w->host_exec);
@@ -1342,11 +1346,7 @@ sed::Workspace* get_ws(sed_ctx* ctx, void* stream, int rows, int kpad, int ldn, 
   if (!need) return w;
   // grow: free and reallocate everything (the stream's previous work must finish first)
   cudaStreamSynchronize((cudaStream_t)stream);
-  std::vector<void*> old = {w->perm, w->tile_win, w->kmask, w->W, w->W_hi, w->W_lo, w->W_bf16, w->W_f8, w->Y, w->O, w->O2, w->rs, w->err,
-                            w->wmask, w->theta_h, w->lnl_h, w->st_h, w->G_hi, w->G_lo, w->GO_hi, w->GO_lo,
-                            w->dW, w->rgrad, w->qneb};
-  for (void* p : old)
-    if (p) cudaFree(p);
+  free_ws_buffers(w);
   budget_release(ctx, w->bytes);
   const bool had_grad = w->dW != nullptr;
   const int seg = std::max(nseg, w->cap_seg);
@@ -1379,7 +1379,12 @@ sed::Workspace* get_ws(sed_ctx* ctx, void* stream, int rows, int kpad, int ldn, 
     if (e != cudaSuccess) s = fail(ctx, SED_ECUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
   }
   *st = s;
-  return s ? nullptr : w;
+  if (!s) return w;
+  // no part of it is kept: a later, smaller call makes its own
+  free_ws_buffers(w);
+  budget_release(ctx, w->bytes);
+  *w = Workspace();
+  return nullptr;
 }
 
 sed_status check_hot_args(sed_ctx* ctx, Model* M, const float* theta, int n, int ld, int precision) {
