@@ -48,10 +48,10 @@ __device__ __forceinline__ float dust_shape(const ModelDev& md, const float4& c,
   return md.dust_law == SED_DUST_POWER_LAW ? pw : (c.y + eb * c.z) * pw;
 }
 
-// A node's four template corners: the cell's float4 where the grid keeps them
-// together, else one load per corner.
+// A node's four template corners: one float4 at the first corner's place where
+// the grid keeps them together, else one load per corner.
 __device__ __forceinline__ float4 neb_corners(const RowScal& rs, const GridDev& g, int k) {
-  if (g.neb4) return __ldg(g.neb4 + rs.neb_cell + k);
+  if (g.neb4) return __ldg(g.neb4 + rs.neb_off[0] + k);
   return make_float4(g.neb_tab[rs.neb_off[0] + k], g.neb_tab[rs.neb_off[1] + k], g.neb_tab[rs.neb_off[2] + k],
                      g.neb_tab[rs.neb_off[3] + k]);
 }

@@ -892,7 +892,6 @@ __global__ void __launch_bounds__(PREP_THREADS, 8) k_prep(const __grid_constant_
         bracket_f(md.neb_logu, md.neb_nu, th[md.offs[SED_KEY_GAS_LOGU]], u0, wu0, u1, wu1);
         bracket_f(md.neb_logz, md.neb_nz, th[md.offs[SED_KEY_GAS_LOGZ]], z0, wz0, z1, wz1);
         const int nl = g.n_lam;
-        rs.neb_cell = (u0 * max(md.neb_nz - 1, 1) + z0) * nl;
         rs.neb_w[0] = wu0 * wz0; rs.neb_off[0] = (u0 * md.neb_nz + z0) * nl;
         rs.neb_w[1] = wu0 * wz1; rs.neb_off[1] = (u0 * md.neb_nz + z1) * nl;
         rs.neb_w[2] = wu1 * wz0; rs.neb_off[2] = (u1 * md.neb_nz + z0) * nl;

@@ -123,10 +123,10 @@ sed_status ensure_f8_layout(sed_ctx* ctx, Grid* g, Layout* L);
 
 namespace sed {
 __global__ void k_neb4(const float* __restrict__ tab, int nu, int nz, int nl, float4* __restrict__ out) {
-  const int cz = max(nz - 1, 1), cell = blockIdx.y, u = cell / cz, z = cell - u * cz;
+  const int cell = blockIdx.y, u = cell / nz, z = cell - u * nz;
   const int u1 = min(u + 1, nu - 1), z1 = min(z + 1, nz - 1);
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nl; k += gridDim.x * blockDim.x)
-    out[(size_t)cell * nl + k] = make_float4(tab[(size_t)(u * nz + z) * nl + k], tab[(size_t)(u * nz + z1) * nl + k],
+    out[(size_t)cell * nl + k] = make_float4(tab[(size_t)cell * nl + k], tab[(size_t)(u * nz + z1) * nl + k],
                                              tab[(size_t)(u1 * nz + z) * nl + k], tab[(size_t)(u1 * nz + z1) * nl + k]);
 }
 void ensure_neb4(sed_ctx* ctx, Grid* g, cudaStream_t s) {
@@ -138,7 +138,7 @@ void ensure_neb4(sed_ctx* ctx, Grid* g, cudaStream_t s) {
   }
   std::lock_guard<std::mutex> lk(ctx->mu);
   if (g->neb4_tried.load(std::memory_order_relaxed)) return;
-  const int cells = std::max(g->neb_nu - 1, 1) * std::max(g->neb_nz - 1, 1);
+  const int cells = g->neb_nu * g->neb_nz;
   const size_t bytes = (size_t)cells * g->n_lam * sizeof(float4);
   if (bytes <= NEB4_MAX_BYTES && (!ctx->budget || ctx->used.load() + 8 * bytes <= ctx->budget)) {
     const std::string kept = ctx->last_error;

@@ -64,7 +64,6 @@ struct RowScal {
   float log2_qy;    // log2(Q_young, device units) (-inf when Q_young = 0)
   float neb_w[4];   // bilinear weights of the nebular template corners
   int neb_off[4];   // corner offsets (rows of the template)
-  int neb_cell;     // offset of the cell's row of corners (GridDev::neb4)
   float neb_dwu[4]; // d neb_w / d gas_logu (adjoint)
   float neb_dwz[4]; // d neb_w / d gas_logz (adjoint)
   float dlnp_dz;    // d ln(p_phot)/dz (adjoint)
@@ -121,8 +120,9 @@ struct GridDev {
   const float* neb_tab;    // [nu][nz][n_lam] log10 template + device-unit offset; with an age axis
                            // [neb_na][nu][nz][n_lam], plane i the cube at SSP age neb_a0 + i
   const float4* neb4;      // the template's four corners {(u,z), (u,z+1), (u+1,z), (u+1,z+1)} of each cell of its
-                           // axes, [cells in u][cells in z][n_lam]: a node's corners in one load.  NULL in a grid's
-                           // own view (grid_view() fills it in); where it is NULL neb_tab is read instead
+                           // axes (indices past an axis's end: its last), laid out as neb_tab's (u,z): a node's
+                           // corners in one load.  NULL in a grid's own view (grid_view() fills it in); where it is
+                           // NULL neb_tab is read instead
   int neb_nu, neb_nz;
   int neb_a0, neb_na;      // nebular age axis: the SSP ages [neb_a0, neb_a0 + neb_na) (neb_na = 0: none)
   // emission-line cube: per line {ln(lam/5500), k'/4.05, Drude/4.05, lam},
