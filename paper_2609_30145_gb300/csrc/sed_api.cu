@@ -122,38 +122,6 @@ sed_status ensure_f8_layout(sed_ctx* ctx, Grid* g, Layout* L);
 }  // namespace
 
 namespace sed {
-__global__ void k_neb4(const float* __restrict__ tab, int nu, int nz, int nl, float4* __restrict__ out) {
-  const int cell = blockIdx.y, u = cell / nz, z = cell - u * nz;
-  const int u1 = min(u + 1, nu - 1), z1 = min(z + 1, nz - 1);
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nl; k += gridDim.x * blockDim.x)
-    out[(size_t)cell * nl + k] = make_float4(tab[(size_t)cell * nl + k], tab[(size_t)(u * nz + z1) * nl + k],
-                                             tab[(size_t)(u1 * nz + z) * nl + k], tab[(size_t)(u1 * nz + z1) * nl + k]);
-}
-void ensure_neb4(sed_ctx* ctx, Grid* g, cudaStream_t s) {
-  if (g->neb4_tried.load(std::memory_order_acquire) || !g->dv.neb_tab || g->neb_na > 0) return;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-    cudaGetLastError();
-    return;
-  }
-  std::lock_guard<std::mutex> lk(ctx->mu);
-  if (g->neb4_tried.load(std::memory_order_relaxed)) return;
-  const int cells = g->neb_nu * g->neb_nz;
-  const size_t bytes = (size_t)cells * g->n_lam * sizeof(float4);
-  if (bytes <= NEB4_MAX_BYTES && (!ctx->budget || ctx->used.load() + 8 * bytes <= ctx->budget)) {
-    const std::string kept = ctx->last_error;
-    float4* p = nullptr;
-    if (dalloc(ctx, (void**)&p, bytes, &g->allocs, &g->bytes) == SED_OK) {
-      k_neb4<<<dim3((g->n_lam + 255) / 256, cells), 256, 0, s>>>(g->dv.neb_tab, g->neb_nu, g->neb_nz, g->n_lam, p);
-      // other streams may read it as soon as it is published
-      if (cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(s) == cudaSuccess)
-        g->neb4.store(p, std::memory_order_release);
-    } else {
-      ctx->last_error = kept;
-    }
-  }
-  g->neb4_tried.store(true, std::memory_order_release);
-}
 sed_status ensure_f8_layout_shared(sed_ctx* ctx, Grid* g, Layout* L) { return ensure_f8_layout(ctx, g, L); }
 }  // namespace sed
 
@@ -457,6 +425,28 @@ sed_status sed_load_grid(sed_ctx* ctx, const sed_grid_desc* d, sed_grid_id* out)
     st = upload(ctx, &p, tab.data(), tab.size(), &g->allocs, &g->bytes);
     dv.neb_tab = p;
     dv.neb_nu = g->neb_nu; dv.neb_nz = g->neb_nz;
+    // A node's four corners side by side (GridDev::neb4).  Made here, where a caller
+    // expects allocations and waits.  Not under a memory budget, whose room is the
+    // calls' own, nor for a caller who named the copies of the grid to keep: four
+    // times the template is half a BF16 copy of the paper-scale grid.
+    const size_t bytes4 = plane * sizeof(float4);
+    if (!st && neb_na == 0 && !ctx->budget && !d->precision_mask && bytes4 <= NEB4_MAX_BYTES) {
+      const int nu = g->neb_nu, nz = g->neb_nz;
+      std::vector<float4> t4(plane);
+      for (int u = 0; u < nu; u++)
+        for (int z = 0; z < nz; z++) {
+          const int u1 = std::min(u + 1, nu - 1), z1 = std::min(z + 1, nz - 1);
+          const float *c00 = &tab[(size_t)(u * nz + z) * nl], *c01 = &tab[(size_t)(u * nz + z1) * nl];
+          const float *c10 = &tab[(size_t)(u1 * nz + z) * nl], *c11 = &tab[(size_t)(u1 * nz + z1) * nl];
+          for (size_t k = 0; k < nl; k++) t4[(size_t)(u * nz + z) * nl + k] = make_float4(c00[k], c01[k], c10[k], c11[k]);
+        }
+      const std::string kept = ctx->last_error;
+      float4* p4 = nullptr;
+      const sed_status s4 = upload(ctx, &p4, t4.data(), t4.size(), &g->allocs, &g->bytes);
+      if (s4 == SED_OK) dv.neb4 = p4;
+      else if (s4 == SED_ENOMEM) ctx->last_error = kept;   // the calls read neb_tab
+      else st = s4;
+    }
     g->neb_a0 = dv.neb_a0 = neb_a0;
     g->neb_na = dv.neb_na = neb_na;
     // emission-line cube: per line the constants of the attenuation at its
@@ -1420,7 +1410,6 @@ sed_status run_forward_core(sed_ctx* ctx, Model* M, Workspace* w, const float* t
     w->have_stats = true;
     w->last_grad = false;
   }
-  if (M->dv.use_neb) ensure_neb4(ctx, g, s);
   if (sed_status ps = prof_mark(ctx, w, 0, s)) return ps;
   PrepArgs pa{};
   pa.theta = theta; pa.n = n; pa.ld = ld;
@@ -1548,7 +1537,7 @@ sed_status sed_forward(sed_ctx* ctx, sed_model_id id, const float* theta, int n,
   EpiArgs ea{};
   ea.n = n; ea.ldn = w->ldn; ea.Y = w->Y; ea.O = w->O; ea.rs = w->rs;
   ea.O2 = w->O2; ea.split = precision == SED_PREC_FP32 ? w->err + 8 : nullptr;   // the 3xTF32 launch's split choice
-  ea.md = M->dv; ea.g = grid_view(M->g);
+  ea.md = M->dv; ea.g = M->g->dv;
   ea.seg_stride = (size_t)w->cap_rows * w->ldn;
   ea.qneb = M->dv.use_neb && M->g->neb_na > 0 ? w->qneb : nullptr;
   reset_after(ea, w, n);
@@ -1578,7 +1567,7 @@ sed_status sed_line_fluxes(sed_ctx* ctx, sed_model_id id, const float* theta, in
   EpiArgs ea{};
   ea.n = n; ea.ldn = w->ldn; ea.Y = w->Y; ea.O = w->O; ea.rs = w->rs;
   ea.O2 = w->O2; ea.split = precision == SED_PREC_FP32 ? w->err + 8 : nullptr;   // the 3xTF32 launch's split choice
-  ea.md = M->dv; ea.g = grid_view(M->g);
+  ea.md = M->dv; ea.g = M->g->dv;
   ea.seg_stride = (size_t)w->cap_rows * w->ldn;
   ea.qneb = M->dv.use_neb && M->g->neb_na > 0 ? w->qneb : nullptr;
   reset_after(ea, w, n);
@@ -1607,7 +1596,7 @@ static sed_status loglike_impl(sed_ctx* ctx, sed_model_id id, const float* theta
   EpiArgs ea{};
   ea.n = n; ea.ldn = w->ldn; ea.Y = w->Y; ea.O = w->O; ea.rs = w->rs;
   ea.O2 = w->O2; ea.split = precision == SED_PREC_FP32 ? w->err + 8 : nullptr;   // the 3xTF32 launch's split choice
-  ea.md = M->dv; ea.g = grid_view(M->g);
+  ea.md = M->dv; ea.g = M->g->dv;
   ea.seg_stride = (size_t)w->cap_rows * w->ldn;
   ea.qneb = M->dv.use_neb && M->g->neb_na > 0 ? w->qneb : nullptr;
   reset_after(ea, w, n);
@@ -1726,7 +1715,7 @@ sed_status sed_loglike_grad(sed_ctx* ctx, sed_model_id id, const float* theta, i
   EpiBwdArgs eb{};
   eb.n = n; eb.ldn = w->ldn; eb.Y = w->Y; eb.O = w->O; eb.rs = w->rs;
   eb.O2 = w->O2; eb.o2_split = precision == SED_PREC_FP32 ? w->err + 8 : nullptr;
-  eb.md = M->dv; eb.g = grid_view(g); eb.split = f32 ? 1 : 0;
+  eb.md = M->dv; eb.g = g->dv; eb.split = f32 ? 1 : 0;
   eb.gy_hi = w->G_hi; eb.gy_lo = w->G_lo; eb.go_hi = w->GO_hi; eb.go_lo = w->GO_lo;
   eb.rgrad = w->rgrad; eb.lnl = lnl_out; eb.status = row_status; eb.err = w->err;
   eb.seg_stride = (size_t)w->cap_rows * w->ldn;

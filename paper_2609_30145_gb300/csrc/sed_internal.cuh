@@ -121,8 +121,9 @@ struct GridDev {
                            // [neb_na][nu][nz][n_lam], plane i the cube at SSP age neb_a0 + i
   const float4* neb4;      // the template's four corners {(u,z), (u,z+1), (u+1,z), (u+1,z+1)} of each cell of its
                            // axes (indices past an axis's end: its last), laid out as neb_tab's (u,z): a node's
-                           // corners in one load.  NULL in a grid's own view (grid_view() fills it in); where it is
-                           // NULL neb_tab is read instead
+                           // corners in one load.  NULL under a memory budget or a precision mask, past
+                           // NEB4_MAX_BYTES, with an age axis or where the device had no room: neb_tab is read
+                           // instead (the same values)
   int neb_nu, neb_nz;
   int neb_a0, neb_na;      // nebular age axis: the SSP ages [neb_a0, neb_a0 + neb_na) (neb_na = 0: none)
   // emission-line cube: per line {ln(lam/5500), k'/4.05, Drude/4.05, lam},
@@ -296,8 +297,6 @@ struct Grid {
   GridDev dv{};
   int neb_nu = 0, neb_nz = 0;
   int neb_a0 = 0, neb_na = 0;  // nebular age axis: the SSP ages it spans (neb_na = 0: none)
-  std::atomic<const float4*> neb4{nullptr};   // GridDev::neb4, built by the first call that reads it
-  std::atomic<bool> neb4_tried{false};
   std::vector<double> neb_logu, neb_logz;
   std::vector<Layout*> layouts;
   std::vector<void*> allocs;
@@ -731,17 +730,6 @@ struct PrepBwdArgs {
   int mask_words;
 };
 cudaError_t launch_prep_bwd(const PrepBwdArgs& a, cudaStream_t s);
-
-// The table of nebular template corners (GridDev::neb4), built on the first call
-// of a model with nebular emission: kept to NEB4_MAX_BYTES, left out for an age
-// axis, under stream capture, or where memory or the budget is short (a call
-// then reads neb_tab; the results are the same).
-void ensure_neb4(sed_ctx* ctx, Grid* g, cudaStream_t s);
-inline GridDev grid_view(const Grid* g) {
-  GridDev d = g->dv;
-  d.neb4 = g->neb4.load(std::memory_order_acquire);
-  return d;
-}
 
 // Build the FP8 copy of a layout (caller holds ctx->mu).
 sed_status ensure_f8_layout_shared(sed_ctx* ctx, Grid* g, Layout* L);

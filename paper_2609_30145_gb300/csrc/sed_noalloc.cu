@@ -181,7 +181,7 @@ extern "C" sed_status sed_loglike_noalloc(sed_ctx* ctx, sed_model_id id, const f
   if (e == cudaSuccess) {
     EpiArgs ea{};
     ea.n = n; ea.ldn = ldn; ea.Y = Y; ea.O = O; ea.rs = rs;
-    ea.md = M->dv; ea.g = grid_view(g);
+    ea.md = M->dv; ea.g = g->dv;
     ea.lnl = lnl_out; ea.status = row_status; ea.err = err;
     e = launch_epilogue(ea, s);
   }

@@ -220,7 +220,7 @@ cudaError_t issue_launch(sed_server* sv, SrvSlot& sl) {
   EpiArgs ea{};
   ea.n = n; ea.ldn = sv->ldn; ea.Y = sl.Y; ea.O = sl.O; ea.rs = sl.rs;
   ea.O2 = sl.O2; ea.split = sv->prec == SED_PREC_FP32 ? sl.err + 8 : nullptr;   // same choice as sed_loglike
-  ea.g = grid_view(g);
+  ea.g = g->dv;
   ea.mtab = sv->mtab; ea.row_model = sl.rowm;
   ea.smem_samp = sv->max_samp; ea.smem_pix = sv->max_pix; ea.smem_win = sv->max_win;
   ea.lnl = sl.lnl; ea.status = sl.st; ea.err = sl.err;
@@ -344,7 +344,6 @@ sed_status sed_server_create(sed_ctx* ctx, const sed_server_desc* d, sed_server*
     ok = ensure_f8_layout_shared(ctx, sv->g, sv->L) == SED_OK;
   }
   ok = ok && cudaStreamCreateWithFlags(&sv->up, cudaStreamNonBlocking) == cudaSuccess;
-  if (ok && M0->dv.use_neb) ensure_neb4(ctx, sv->g, sv->up);
   ok = ok && dmalloc(sv, sv->dev, &sv->mtab, sizeof(ModelDev) * SRV_MAX_MODELS);
   sv->mtab_loaded.assign(SRV_MAX_MODELS, 0);
   const size_t R = (size_t)sv->max_rows, K = (size_t)sv->L->Kpad, N = (size_t)sv->ldn;
