@@ -69,8 +69,10 @@ constexpr int EPI_FLAT = 512;
 
 // dynamic shared memory: lam, F/lam^2 and F over the row's window, the
 // included pixels' mu/sigma for the calibration moments, with emission lines,
-// per line ln(lam_obs) (an FP32 pair), F_l, A_l and 1/s_l, the pixels' residuals
-// and, from EPI_FLAT threads on, the samples' values
+// per line ln(lam_obs) (an FP32 pair), F_l, A_l and 1/s_l and, from EPI_FLAT threads
+// on, the samples' values.  The pixels' residuals pass through lam's and F/lam^2's
+// places, which the spectrum does not read, as many pixels at a time as fit there:
+// no number of pixels needs more.
 size_t epilogue_lines_off(const EpiArgs& a) {   // in floats, even (float2 alignment)
   const int np = a.row_model ? a.smem_pix : a.md.n_pix;
   const size_t W = (size_t)(a.row_model ? a.smem_win : a.md.win_max);
@@ -82,15 +84,9 @@ size_t epilogue_samp_off(const EpiArgs& a) {   // in floats
   const bool lines = a.row_model ? a.g.n_line > 0 : a.md.use_lines != 0;
   return epilogue_lines_off(a) + (lines ? (size_t)5 * a.g.n_line : 0);
 }
-// the pixels' residuals: over lam and F/lam^2, which the spectrum does not read,
-// where they fit there
-bool epilogue_res_alias(const EpiArgs& a) {
-  return (a.row_model ? a.smem_pix : a.md.n_pix) <= 2 * (a.row_model ? a.smem_win : a.md.win_max);
-}
 size_t epilogue_smem(const EpiArgs& a, int nt) {
-  const size_t pix = epilogue_res_alias(a) ? 0 : (size_t)(a.row_model ? a.smem_pix : a.md.n_pix);
   const size_t samp = 32 * (size_t)(a.row_model ? a.smem_samp : a.md.n_samp32);
-  return (epilogue_samp_off(a) + pix + (nt >= EPI_FLAT ? samp : 0)) * sizeof(float);
+  return (epilogue_samp_off(a) + (nt >= EPI_FLAT ? samp : 0)) * sizeof(float);
 }
 
 // a / b by the hardware's reciprocal, subnormals as zero (a and b here are
@@ -295,7 +291,7 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
       mb_s[b] = mb;
     }
   };
-  float* rn_s = reinterpret_cast<float*>(smem4) + a.res_off;    // the pixels' residuals
+  float* rn_s = reinterpret_cast<float*>(smem4);                // the pixels' residuals, 2 WIN at a time
   float* v_s = reinterpret_cast<float*>(smem4) + a.samp_off;    // NT >= EPI_FLAT: the samples' values
   if constexpr (NT < EPI_FLAT) {
     // one band per warp: consecutive lanes take consecutive samples (coalesced
@@ -371,11 +367,11 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
   //      -1/2 ln(2 pi sigma^2) in FP64.
   double part = 0.0;
   float chi = 0.f;
-  if (md.n_pix > 0) {
-    if (a.res_off < 2 * WIN) __syncthreads();   // the residuals go over lam and F/lam^2
+  for (int c0 = 0; c0 < md.n_pix; c0 += 2 * WIN) {   // pixels [c0, last]
+    __syncthreads();   // lam and F/lam^2, or the residuals before these, have been read
     const float ll0 = g.lnl_hi[0], llN = g.lnl_hi[N - 1];
-    const int last = md.n_pix - 1;
-    for (int ib = 2 * 32 * warp; ib < md.n_pix; ib += 2 * NT) {
+    const int last = min(c0 + 2 * WIN, md.n_pix) - 1;
+    for (int ib = c0 + 2 * 32 * warp; ib <= last; ib += 2 * NT) {
       float2 pl[2];
       float v[2], xh[2], xl[2], inv_s[2], sw[2] = {0.f, 0.f}, sf[2] = {0.f, 0.f};
       bool gauss[2], valid[2];
@@ -450,16 +446,16 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
           const float qf = floor_q(rs.fl[1], ms, dn, rs.fl[1][3] * isf);
           t = t * t / qf + logf(qf);
         }
-        rn_s[i] = inc ? t : __uint_as_float(EPI_MISSED);
+        rn_s[i - c0] = inc ? t : __uint_as_float(EPI_MISSED);
         if (md.calib_n) mu_s[i] = ms;
       }
     }
     __syncthreads();
     if (NT == EPI_THREADS || tid < EPI_THREADS)
-      for (int i = tid; i < md.n_pix; i += EPI_THREADS) {
+      for (int i = c0 + ((tid - c0) & (EPI_THREADS - 1)); i <= last; i += EPI_THREADS) {   // the pixels tid, tid + 128, ...
         // an included pixel's term: the residual squared, or twice minus the term
         // with the noise floor
-        const float t = rn_s[i];
+        const float t = rn_s[i - c0];
         if (__float_as_uint(t) == EPI_MISSED) continue;
         if (md.floor_bits[1]) chi -= 0.5f * t;
         else chi = fmaf(-0.5f * t, t, chi);
@@ -548,7 +544,6 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
 template <int NT>
 cudaError_t launch_epilogue_nt(EpiArgs a, cudaStream_t s) {
   const size_t smem = epilogue_smem(a, NT);
-  if (!epilogue_res_alias(a)) a.res_off = a.samp_off + (NT >= EPI_FLAT ? 32 * (a.row_model ? a.smem_samp : a.md.n_samp32) : 0);
   static DynSmemCache set_for[6];
   const bool lines = a.row_model ? a.g.n_line > 0 : a.md.use_lines != 0;
   // age-binned dust and the nebular age axis: neither served nor with lines
@@ -568,7 +563,6 @@ cudaError_t launch_epilogue(const EpiArgs& a_in, cudaStream_t s) {
   EpiArgs a = a_in;
   a.lines_off = (int)epilogue_lines_off(a);
   a.samp_off = (int)epilogue_samp_off(a);
-  a.res_off = 0;
   // Threads per row: as many as keep every row of the launch resident at once
   // (1024 threads per SM at 64 registers), where their shared memory fits.
   const int sm = device_sm_count();
