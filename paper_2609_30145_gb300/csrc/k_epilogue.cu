@@ -69,10 +69,11 @@ constexpr int EPI_FLAT = 512;
 
 // dynamic shared memory: lam, F/lam^2 and F over the row's window, the
 // included pixels' mu/sigma for the calibration moments, with emission lines,
-// per line ln(lam_obs) (an FP32 pair), F_l, A_l and 1/s_l and, from EPI_FLAT threads
-// on, the samples' values.  The pixels' residuals pass through lam's and F/lam^2's
-// places, which the spectrum does not read, as many pixels at a time as fit there:
-// no number of pixels needs more.
+// per line ln(lam_obs) (an FP32 pair), F_l, A_l and 1/s_l, from EPI_FLAT threads on
+// the samples' values, and the bands' extents and data where there is room for
+// them (a window of some 19,000 nodes with a spectrum leaves none).  The pixels'
+// residuals pass through lam's and F/lam^2's places, which the spectrum does not
+// read, as many pixels at a time as fit there: no number of pixels needs more.
 size_t epilogue_lines_off(const EpiArgs& a) {   // in floats, even (float2 alignment)
   const int np = a.row_model ? a.smem_pix : a.md.n_pix;
   const size_t W = (size_t)(a.row_model ? a.smem_win : a.md.win_max);
@@ -84,9 +85,16 @@ size_t epilogue_samp_off(const EpiArgs& a) {   // in floats
   const bool lines = a.row_model ? a.g.n_line > 0 : a.md.use_lines != 0;
   return epilogue_lines_off(a) + (lines ? (size_t)5 * a.g.n_line : 0);
 }
-size_t epilogue_smem(const EpiArgs& a, int nt) {
-  const size_t samp = 32 * (size_t)(a.row_model ? a.smem_samp : a.md.n_samp32);
-  return (epilogue_samp_off(a) + (nt >= EPI_FLAT ? samp : 0)) * sizeof(float);
+size_t epilogue_samp_end(const EpiArgs& a, int nt) {   // in floats
+  return epilogue_samp_off(a) + (nt >= EPI_FLAT ? 32 * (size_t)(a.row_model ? a.smem_samp : a.md.n_samp32) : 0);
+}
+size_t epilogue_band_off(const EpiArgs& a, int nt) {   // in floats, even (double alignment)
+  return (epilogue_samp_end(a, nt) + 1) & ~(size_t)1;
+}
+size_t epilogue_smem(const EpiArgs& a, int nt, bool bands) {
+  if (!bands) return epilogue_samp_end(a, nt) * sizeof(float);
+  const size_t nb = a.row_model ? MAX_BANDS : a.md.n_filt;
+  return epilogue_band_off(a, nt) * sizeof(float) + nb * sizeof(double3) + (nb + 1) * sizeof(int);
 }
 
 // a / b by the hardware's reciprocal, subnormals as zero (a and b here are
@@ -122,11 +130,14 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
   __shared__ double cal_fix;                       // the row's lnL terms that do not sum over pixels
 
   // the bands' extents and data, read in the shadow of the kernel before
-  __shared__ int b32_s[MAX_BANDS + 1];
-  __shared__ double3 band_s[MAX_BANDS];   // {datum, 1/sigma, -ln(2 pi sigma^2)/2}
-  for (int b = tid; b <= md.n_filt && md.n_filt > 0; b += NT) {
+  double3* band_s = reinterpret_cast<double3*>(reinterpret_cast<float*>(smem4) + a.band_off);
+  int* b32_s = reinterpret_cast<int*>(band_s + (MULTI ? MAX_BANDS : md.n_filt));
+  auto band_data = [&](int b) { return make_double3(md.phot_d[b], md.phot_isig[b], md.phot_nlog[b]); };
+  auto band = [&](int b) { return a.band_off ? band_s[b] : band_data(b); };   // {datum, 1/sigma, -ln(2 pi sigma^2)/2}
+  auto b32 = [&](int b) { return a.band_off ? b32_s[b] : __ldg(md.band32 + b); };
+  for (int b = tid; a.band_off && b <= md.n_filt && md.n_filt > 0; b += NT) {
     b32_s[b] = md.band32[b];
-    if (b < md.n_filt) band_s[b] = make_double3(md.phot_d[b], md.phot_isig[b], md.phot_nlog[b]);
+    if (b < md.n_filt) band_s[b] = band_data(b);
   }
   if constexpr (!MULTI) pdl_enter();
 
@@ -298,8 +309,9 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
     // loads, eight in flight per lane); a sample outside the grid adds zero
     for (int b = warp; b < md.n_filt; b += NT / 32) {
       float acc = 0.f;
-      const float2* s2 = md.samp32 + 32 * b32_s[b] + lane;
-      for (int n32 = b32_s[b + 1] - b32_s[b]; n32 > 0; n32 -= 8, s2 += 256) {
+      const int s0 = b32(b);
+      const float2* s2 = md.samp32 + 32 * s0 + lane;
+      for (int n32 = b32(b + 1) - s0; n32 > 0; n32 -= 8, s2 += 256) {
         if (pick) {
           float2 sp[8];
           int kg[8];
@@ -351,8 +363,9 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
     __syncthreads();
     for (int b = warp; b < md.n_filt; b += NT / 32) {
       float acc = 0.f;
+      const int j1 = 32 * b32(b + 1);
 #pragma unroll 8
-      for (int j = 32 * b32_s[b] + lane; j < 32 * b32_s[b + 1]; j += 32) acc = fmaf(__ldg(&md.samp32[j].y), v_s[j], acc);
+      for (int j = 32 * b32(b) + lane; j < j1; j += 32) acc = fmaf(__ldg(&md.samp32[j].y), v_s[j], acc);
       band_finish(b, acc);
     }
   }
@@ -512,15 +525,16 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
   if (warp == 0) {
     double pv = 0.0;
     for (int b = lane; b < md.n_filt; b += 32) {
-      const double is = band_s[b].y;
+      const double3 bd = band(b);
+      const double is = bd.y;
       if (is != 0.0) {
-        const double mn = (double)mb_s[b] * is, dn = band_s[b].x * is;
+        const double mn = (double)mb_s[b] * is, dn = bd.x * is;
         const double rr = phot_resid(md, b, dn, mn);
         if (md.floor_bits[0]) {   // sigma_eff of Eq. app_noise_floor
           const double q = floor_q(rs.fl[0], mn, dn, (double)rs.fl[0][3] * is);
-          pv += -0.5 * (rr * rr / q + log(q)) + band_s[b].z;
+          pv += -0.5 * (rr * rr / q + log(q)) + bd.z;
         } else {
-          pv += -0.5 * rr * rr + band_s[b].z;
+          pv += -0.5 * rr * rr + bd.z;
         }
       }
     }
@@ -543,7 +557,8 @@ __global__ void __launch_bounds__(NT, NT == EPI_THREADS ? 7 : 1024 / NT) k_epilo
 
 template <int NT>
 cudaError_t launch_epilogue_nt(EpiArgs a, cudaStream_t s) {
-  const size_t smem = epilogue_smem(a, NT);
+  size_t smem = epilogue_smem(a, NT, true);
+  a.band_off = (int)epilogue_band_off(a, NT);
   static DynSmemCache set_for[6];
   const bool lines = a.row_model ? a.g.n_line > 0 : a.md.use_lines != 0;
   // age-binned dust and the nebular age axis: neither served nor with lines
@@ -555,6 +570,11 @@ cudaError_t launch_epilogue_nt(EpiArgs a, cudaStream_t s) {
          : m == 3 ? k_epilogue<true, true, 0, NT>
          : m == 4 ? k_epilogue<false, false, 1, NT> : k_epilogue<false, false, 2, NT>;
   cudaError_t e = ensure_dyn_smem(k, smem, &set_for[m]);
+  if (e == cudaErrorInvalidConfiguration) {   // no room for the bands: they are read where the model keeps them
+    a.band_off = 0;
+    smem = epilogue_smem(a, NT, false);
+    e = ensure_dyn_smem(k, smem, &set_for[m]);
+  }
   if (e != cudaSuccess) return e;
   return launch_pdl(k, dim3(a.n), dim3(NT), smem, s, a);
 }
@@ -567,8 +587,8 @@ cudaError_t launch_epilogue(const EpiArgs& a_in, cudaStream_t s) {
   // (1024 threads per SM at 64 registers), where their shared memory fits.
   const int sm = device_sm_count();
   const size_t room = (size_t)220 * 1024;
-  if (a.n <= 2 * sm && 2 * epilogue_smem(a, 512) <= room) return launch_epilogue_nt<512>(a, s);
-  if (a.n <= 4 * sm && 4 * epilogue_smem(a, 256) <= room) return launch_epilogue_nt<256>(a, s);
+  if (a.n <= 2 * sm && 2 * epilogue_smem(a, 512, true) <= room) return launch_epilogue_nt<512>(a, s);
+  if (a.n <= 4 * sm && 4 * epilogue_smem(a, 256, true) <= room) return launch_epilogue_nt<256>(a, s);
   return launch_epilogue_nt<EPI_THREADS>(a, s);
 }
 

@@ -677,7 +677,8 @@ struct EpiArgs {
   const int* err;      // device error word of the contraction (row status SED_ROW_DEVICE_TIMEOUT)
   const float* lam8;   // FP8 path: [n_lam] 2^-f_l multiplying Y and O; NULL otherwise
   int lines_off;       // set by launch_epilogue: float offsets of the emission lines' shared arrays and of
-  int samp_off;        //   the samples' values
+  int samp_off;        //   the samples' values and of the bands' extents and data (0: not in shared memory)
+  int band_off;
   size_t seg_stride;   // age-binned dust: Y of attenuated block s at Y + s seg_stride
   const float* qneb;   // nebular age axis: [n][MAX_NEB_AGE] (k_prep's), or NULL
   int* win_reset;      // [win_mt][2] per-tile windows set back to empty by CTA 0 (the contraction,
