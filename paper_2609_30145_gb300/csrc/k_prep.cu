@@ -1195,7 +1195,7 @@ __global__ void __launch_bounds__(PREP_BWD_THREADS) k_prep_bwd(const __grid_cons
       out[md.offs[SED_KEY_SFH] + k] = (k < NT ? gps0[k] : 0.f) + (k > 0 ? gps1[k - 1] : 0.f);
   } else
   for (int i = tid; i < NT; i += blockDim.x) {
-    const float Ti = T[i], Ti1 = T[i + 1], r_dT = 1.f / (Ti1 - Ti), mi = m[i];
+    const float Ti = T[i], Ti1 = T[i + 1], dT = Ti1 - Ti, mi = m[i], rate = mi / dT;
     // first age whose cell reaches above T_i
     int a0 = 0, a1 = NA;
     while (a0 < a1) {
@@ -1211,15 +1211,15 @@ __global__ void __launch_bounds__(PREP_BWD_THREADS) k_prep_bwd(const __grid_cons
       const float lo = cell_lo[ag], hi = cell_hi[ag];
       const float ov = fminf(Ti1, hi) - fmaxf(Ti, lo);
       if (ov <= 0.f) continue;
-      const float f = ov * r_dT;   // the bin's share in the age's cell
+      const float f = ov / dT;   // the bin's share in the age's cell
       const float g0 = gWs[ag * NZ + j0];
       const float g1 = NZ > 1 ? gWs[ag * NZ + j0 + 1] : 0.f;
       const float gA = g0 * (1.f - t) + g1 * t;
       gz += mi * f * (g0 * d0 + g1 * d1);
       gm += gA * f;
-      const float gm_r = gA * mi * r_dT;
-      ghi += gm_r * ((Ti1 < hi ? 1.f : 0.f) - f);
-      glo += gm_r * (f - (Ti > lo ? 1.f : 0.f));
+      const float gr = gA * rate;
+      ghi += gr * ((Ti1 < hi ? 1.f : 0.f) - f);
+      glo += gr * (f - (Ti > lo ? 1.f : 0.f));
     }
     out[md.offs[SED_KEY_SFH] + i] = gm;
     gzeta[i] = gz;
