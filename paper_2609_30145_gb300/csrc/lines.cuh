@@ -77,23 +77,12 @@ __device__ __forceinline__ void line_setup(const ModelDev& md, const GridDev& g,
   is_s[l] = inv_s;
 }
 
-// Sum of the line profiles at pixel i (cgs F_nu), lines in index order, each
-// truncated at 5 s_l (Eq. app_line_profile, not renormalised).
-__device__ __forceinline__ float lines_at_pixel(const ModelDev& md, int i, int NLn, const float* A_s, const float* is_s,
-                                                const float2* x_s) {
-  const float2 p = md.pix_ln2[i];
-  float acc = 0.f;
-  for (int l = 0; l < NLn; ++l) {
-    const float u = ((p.x - x_s[l].x) + (p.y - x_s[l].y)) * is_s[l];
-    if (fabsf(u) <= 5.f) acc = fmaf(A_s[l], __expf(-0.5f * u * u), acc);
-  }
-  return acc * md.pix_lamc[i];
-}
-
-// The same sum for a warp's two pixels per lane (ln(lambda) in p0, p1; the
-// warp's pixels ascend from xmin to xmax): most lines reach none of them, so
-// each lane first tests one line against the warp's range, and only the lines
-// found are gone through, in index order.
+// Sums of the line profiles (without the pixels' conversion to cgs F_nu, pix_lamc)
+// at a warp's two pixels per lane, lines in index order, each truncated at 5 s_l
+// (Eq. app_line_profile, not renormalised); ln(lambda) in p0, p1, the warp's
+// pixels ascending from xmin to xmax.  Most lines reach none of them, so each
+// lane first tests one line against the warp's range, and only the lines found
+// are gone through.
 __device__ __forceinline__ void lines_at_pixels(int NLn, const float* A_s, const float* is_s, const float2* x_s,
                                                 float2 p0, float2 p1, float xmin, float xmax, int lane, float& a0,
                                                 float& a1) {
