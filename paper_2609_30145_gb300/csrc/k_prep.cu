@@ -505,9 +505,6 @@ constexpr int PREP_KWARPS = PREP_THREADS / 32 - 1;   // warps writing W; the las
 // Largest launch that orders itself (PrepArgs::self_order): each CTA reads
 // every row's redshift, so the cost grows with n^2
 constexpr int SELF_ORDER_MAX = 1024;
-// ... and one with K-tile masks, whose keys hold two brackets per row (301 rows
-// on the [a/Fe] grid: the call 134 us ordering itself, 113 us with k_order)
-constexpr int SELF_PAIR_MAX = 128;
 static_assert(SELF_ORDER_MAX <= 2 * MAX_SFH + 1, "the redshifts are staged in the edge and rate arrays");
 
 // Row p of the launch processes the caller's row r = perm[p] and records r in
@@ -541,7 +538,6 @@ __global__ void __launch_bounds__(PREP_THREADS, 8) k_prep(const __grid_constant_
   float* T = s_trate;
   float* rate = s_trate + MAX_SFH + 1;
   __shared__ int s_pos;
-  __shared__ uint8_t s_pair[SELF_PAIR_MAX];   // self-ordered launch with K-tile masks: the rows' bracket pairs
   __shared__ int zb[MAX_SFH];
   __shared__ float zt[MAX_SFH];
   __shared__ float s_red[PREP_THREADS / 32];
@@ -577,7 +573,7 @@ __global__ void __launch_bounds__(PREP_THREADS, 8) k_prep(const __grid_constant_
     const TmaxRow t = row_tmax(md, theta_col(md, th, md.offs[SED_KEY_ZRED]), theta_col(md, th, md.offs[SED_KEY_LOGMASS]));
     if (lane == 0) { s_tmax = t.tmax; s_lrat = t.lrat; s_zst = t.status; }
   } else if (rank_warp) {
-    // the row's place in the launch's order: the valid redshifts (z in [0, z_f),
+    // the row's place in the redshift order: the valid redshifts (z in [0, z_f),
     // others -1) and their range, then the keys of k_order's bins over that range
     // (invalid rows in the last bin) and the count of rows whose (key, index) is
     // below this row's
@@ -591,27 +587,16 @@ __global__ void __launch_bounds__(PREP_THREADS, 8) k_prep(const __grid_constant_
       zs[j] = zv;
       if (zv >= 0.f) { lo = min(lo, __float_as_int(zv)); hi = max(hi, __float_as_int(zv)); }
     }
-    if (a.by_pair)
-#pragma unroll 4
-      for (int j = lane; j < a.n; j += 32) s_pair[j] = (uint8_t)row_pair(md, a.theta + (size_t)j * a.ld);
     lo = __reduce_min_sync(0xffffffffu, lo);
     hi = __reduce_max_sync(0xffffffffu, hi);
     __syncwarp();
     const float zlo = __int_as_float(lo), zr = fmaxf(__int_as_float(hi) - zlo, 1e-6f);
-    const int halves = a.by_pair ? order_halves(md, zlo, zlo + zr) : 1;
-    const int nf = a.by_pair ? ORDER_BINS / (halves * a.n_pairs) : ORDER_BINS;
-    const float fscale = (float)nf / zr;
-    auto key = [&](int j) {
-      const float z = zs[j];
-      if (!(z >= 0.f)) return ORDER_BINS;
-      int k = min(nf - 1, (int)((z - zlo) * fscale));
-      if (a.by_pair) k += ((halves == 2 && (z - zlo) * 2.f >= zr ? a.n_pairs : 0) + s_pair[j]) * nf;
-      return k;
-    };
-    const int kb = key(b);
+    const float fscale = (float)ORDER_BINS / zr;
+    auto key = [&](float z) { return z >= 0.f ? min(ORDER_BINS - 1, (int)((z - zlo) * fscale)) : ORDER_BINS; };
+    const int kb = key(zs[b]);
     int below = 0;
     for (int j = lane; j < a.n; j += 32) {
-      const int kj = key(j);
+      const int kj = key(zs[j]);
       below += kj < kb || (kj == kb && j < b);
     }
     below = __reduce_add_sync(0xffffffffu, below);
@@ -1304,19 +1289,22 @@ cudaError_t launch_prep_bwd(const PrepBwdArgs& p, cudaStream_t s) {
 
 cudaError_t launch_prep(const PrepArgs& p, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
-  // a fixed redshift (no column) needs no redshift order, but rows of K-tile masks
-  // are ordered by their bracket pair all the same; else the caller's order is kept
+  // a fixed redshift (no column) needs no redshift order: the caller's is kept.  Rows
+  // with K-tile masks are ordered by their bracket pair all the same, unless
+  // they are one tile, whose window and mask are the same in any order (128 rows
+  // with a spectrum on the [a/Fe] grid: the call 92 us, 99 ordering itself, 95 with
+  // k_order; 64 rows without one on the paper-scale grid 35, 37 and 40)
   const bool z_col = p.md.offs[SED_KEY_ZRED] < p.md.n_param;
   const int mt = (p.n + 127) / 128;
   // bracket pair major when the contraction skips K tiles (the host gives
   // masks only to models with one [Fe/H], and [a/Fe], per row)
   const int pairs = std::max(p.md.n_feh - 1, 1) * (p.md.use_afe ? std::max(p.md.n_afe - 1, 1) : 1);
   const bool by_pair = !p.row_model && p.kmask && pairs > 1 && pairs <= ORDER_BINS / 4;
-  const bool ordered = p.row_model || z_col || by_pair;
+  const bool ordered = p.row_model || (by_pair ? p.n > 128 : z_col);
   // a small single-fit launch orders itself; its windows and masks start empty
   // because the last kernel of every call that filled them empties them again,
   // and the workspace starts them empty
-  const bool self = ordered && p.self_order && !p.row_model && p.n <= (by_pair ? SELF_PAIR_MAX : SELF_ORDER_MAX);
+  const bool self = ordered && p.self_order && !p.row_model && !by_pair && p.n <= SELF_ORDER_MAX;
   const bool order = ordered && !self && p.perm;
   if (!order && !p.self_order) {   // nothing before this kernel to start the windows and masks empty
     if (p.tile_win) e = cudaMemsetAsync(p.tile_win, WIN_EMPTY_BYTE, 2 * mt * sizeof(int), s);
@@ -1339,8 +1327,6 @@ cudaError_t launch_prep(const PrepArgs& p, cudaStream_t s) {
   PrepKernelArgs ka;
   ka.p = p;
   ka.p.self_order = self ? 1 : 0;
-  ka.p.by_pair = by_pair ? 1 : 0;
-  ka.p.n_pairs = pairs;
   if (!order) ka.p.perm = nullptr;
   // Ws [n_age][n_feh], the FP8 row scratch, the row's parameters (n_param <= ld
   // and n_param <= 2 MAX_SFH + SED_NKEYS + 2 MAX_DUST_BIN for every model)

@@ -478,8 +478,8 @@ struct PrepArgs {
   float* qneb;         // nebular age axis: [n][MAX_NEB_AGE] Q-weighted weight of each nebular SSP age, or NULL
   int self_order;      // 1: tile_win and kmask are already empty, and the prep kernel may find each
                        // row's place in the order itself (no k_order launch): theta in device memory
-                       // (each CTA reads every row's keys); done for one fit of n <= SELF_ORDER_MAX
-  int by_pair, n_pairs;   // set by launch_prep: rows ordered by bracket pair, and the pairs there are
+                       // (each CTA reads every row's redshift); done for one fit of n <= SELF_ORDER_MAX
+                       // without masks that order it by bracket pair
 };
 // A 128-row tile's node window is two words side by side, its first node and the
 // complement of its last one, both taken as minima over the tile's rows and both
