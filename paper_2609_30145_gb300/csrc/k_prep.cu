@@ -582,7 +582,7 @@ __global__ void __launch_bounds__(PREP_THREADS, 8) k_prep(const __grid_constant_
     int lo = 0x7f7fffff, hi = 0;
 #pragma unroll 8
     for (int j = lane; j < a.n; j += 32) {
-      const float z = theta_col(md, a.theta + (size_t)j * a.ld, zoff);
+      const float z = a.theta[(size_t)j * a.ld + zoff];   // a column: launch_prep orders no fixed redshift here
       const float zv = z >= 0.f && z < (float)md.zf ? z : -1.f;
       zs[j] = zv;
       if (zv >= 0.f) { lo = min(lo, __float_as_int(zv)); hi = max(hi, __float_as_int(zv)); }
