@@ -4,16 +4,16 @@
 // birth-cloud age (Eq. app_attn with a two-bin age-to-bin matrix):
 //     Y[theta][lam] = sum_{k in young} W[theta][k] SSP[k][lam]
 //     O[theta][lam] = sum_{k in old}   W[theta][k] SSP[k][lam]
-// W (A operand, [n][Kpad]) and SSP^T (B operand, [n_lam][Kpad]) are both
-// K-major; K is ordered [young block | old block], each padded to 64.
+// W ([n][Kpad], the row operand) and SSP^T ([n_lam][Kpad]) are both K-major; K is
+// ordered [young block | old block], each padded to 64.
 //
 // Adjoint (GRAD = true): the same contraction transposed, reducing over lambda,
 //     dW[theta][k] = sum_lam G[theta][lam] SSP[k][lam]
-// with G = dlnL/dY for young columns k and dlnL/dO for old ones; A = G
-// ([n][ldn], lambda-major), B = SSP ([Kpad][ldn], lambda-major).  The column
-// tiles of the young block start at 0 and those of the old block at Ky_pad, so
-// every tile reads one A operand; the columns of a tile past the end of its
-// block are computed but not stored.
+// with G = dlnL/dY for young columns k and dlnL/dO for old ones: G ([n][ldn]) is the
+// row operand, beside SSP ([Kpad][ldn]), both lambda-major.  The column tiles of
+// the young block start at 0 and those of the old block at Ky_pad, so every tile
+// reads one G; the columns of a tile past the end of its block are computed
+// but not stored.
 //
 // One CTA computes a tile of 128 wavelengths (columns of Y and O, or of dW) by up
 // to 128 rows (theta): the SSP is the MMA's M operand, the rows its N operand, so
@@ -22,13 +22,15 @@
 // warp's store touched 32 rows: without the stores the 4096-row BF16 contraction
 // took 37 us instead of 55.)  The row operand is loaded in boxes of 32 rows, so a
 // small launch or a piece of a tile loads and multiplies only its own.  Warp roles:
-//   warp 0 lane 0 : TMA producer (128B-swizzled K tiles into a STAGES-deep ring)
-//   warp 1 lane 0 : MMA issuer (tcgen05.mma into a ping-pong pair of tensor-memory
-//                   accumulators; a commit frees a smem stage / hands over a buffer)
-//   warps 2-5     : drain the accumulators into FP32 registers and store the tile
-//   warp 2        : also allocates / frees tensor memory
+//   warp 0   : TMA producer (128B-swizzled K tiles into a ring of as many stages as
+//              the launch's rows leave room for, up to 8; one elected lane issues)
+//   warp 1   : MMA issuer (tcgen05.mma, likewise, into a ping-pong pair of tensor-memory
+//              accumulators; a commit frees a smem stage / hands over a buffer)
+//   warps 2-5: drain the accumulators into FP32 registers and store the tile
+//   warp 2   : also allocates / frees tensor memory
 // Precision:
-//   SED_PREC_FP32 : 3xTF32 split, D += A_lo B_hi + A_hi B_lo + A_hi B_hi
+//   SED_PREC_FP32 : 3xTF32 split of the SSP S and the rows R,
+//                   D += S_hi R_lo + S_lo R_hi + S_hi R_hi
 //                   (each operand x = hi + lo, hi = TF32(x)), FP32 accumulate
 //   SED_PREC_BF16 : BF16 operands, FP32 accumulate
 //   SED_PREC_FP8  : FP8 E4M3 operands (kind::f8f6f4), FP32 accumulate
@@ -268,12 +270,12 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 // [K0, KT) -> dW.  A persistent 3xTF32 launch may instead split each tile
 // three ways (kinds 0, 1: the old part's halves [KY, KH) -> O and [KH, KT) ->
 // O2; kind 2: the young blocks), when that shortens its longest CTA (see
-// split_pays): one unit per tile has less overhead (1024-row photometric
-// step 0.0927 against 0.0948 ms split, 4096 rows 0.2960 against 0.3125 ms, the
-// 2048-row [a/Fe] spectro-photometric forward 0.3648 against 0.3865 ms), but
-// with a few tiles more than SMs its leftover tiles leave a few CTAs a second
-// unit (154 tiles on 152 SMs: 0.109 against 0.099 ms split); and 51 tiles of
-// K = 6528 (301 rows) take 135 us as units against 70 us split.
+// split_pays): one unit per tile has less overhead (the call of 1024 photometric
+// rows 73.5 us against 75.8 split, of 4096 rows 233 against 243, of 2048 rows with a
+// spectrum on the [a/Fe] grid 310 against 327), but few tiles leave SMs idle (64
+// rows 42.4 against 33.9 split, 200 rows on the [a/Fe] grid 164 against 133), and
+// with a few tiles more than SMs some CTAs get a second unit (1100 rows 91.2
+// against 83.2).
 //  - Grid schedule (p.tile_win NULL): one unit per CTA from blockIdx; the CTA
 //    exits at once when the tile lies outside the union of its rows' windows.
 //  - Persistent schedule (forward, p.tile_win set): one CTA per SM; every CTA
@@ -282,8 +284,9 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 //    then the wavelength tiles of its window) are cut into full waves -- the
 //    largest multiple of gridDim.x, run as whole units -- and a remainder whose
 //    tiles are split along the rows into up to four pieces of BN/npc rows (an
-//    MMA of N = BN/npc), so the last partial wave costs a fraction of a unit.  Tensor memory, barriers and the smem ring are set up
-//    once, and one unit's drain overlaps the next unit's MMAs.
+//    MMA of N = BN/npc), so the last partial wave costs a fraction of a unit.
+//    Tensor memory, barriers and the smem ring are set up once, and one unit's
+//    drain overlaps the next unit's MMAs.
 //  - Clusters (adjoint, p.cz > 1): a launch with few tiles (200 rows of the
 //    paper-scale grid: 22 on 152 SMs) gives each to a cluster of cz CTAs along
 //    blockIdx.z, which share the groups of its reduction over wavelength: CTA 0
@@ -366,10 +369,13 @@ __device__ __forceinline__ float sched_longest(int tiles, int P, int nz, int kt,
 }
 // Whether the 3-way split shortens the launch by more than 5 % once the
 // epilogue's extra reads are counted: it then reads O2 beside O, a 128 x 128
-// FP32 tile more per tile, about 0.04 of one K tile of a CTA's MMA time per
-// tile of the launch (measured on the photometric fit: 4096 rows split gave a
-// 16 us longer epilogue for no shorter contraction; at 1024 rows, 154 tiles,
-// the split step took 0.099 against 0.109 ms unsplit).
+// FP32 tile more per tile, taken as 0.04 of one K tile of a CTA's MMA time per
+// tile of the launch (at 4096 photometric rows the split call is 10 us longer for
+// no shorter contraction, about 0.02).  Measured both ways at 26 sizes (64 to 4096
+// photometric rows, 64 to 2048 with a spectrum on the [a/Fe] grid, wide and
+// narrow redshift ranges), the call is within about 1 us of the faster side (what
+// the choice itself costs) but for 512 rows on the [a/Fe] grid with z in
+// [0.9, 1.3]: split, as chosen, 122.5 us against 114.3.
 constexpr float SPLIT_EPI_KT_PER_TILE = 0.04f;
 __device__ __forceinline__ bool split_pays(int tiles, int P, int ky, int kt, int rt) {
   const int ko = kt - ky, kh = (ko + 1) / 2;

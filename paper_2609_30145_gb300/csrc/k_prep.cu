@@ -372,8 +372,13 @@ __device__ __forceinline__ int row_pair(const ModelDev& md, const float* row) {
 // Redshift ranges the bracket pairs are ordered within: two halves of the
 // launch's range, which keeps a tile's node window narrow, unless half the range
 // moves a row's window by less than a quarter of its width; one range then puts
-// half as many pairs into a tile (301 rows with z in [0.9, 1.3] on the [a/Fe]
-// grid: the call 117 -> 113 us).
+// half as many pairs into a tile.  Measured with one range and with two, [a/Fe]
+// grid with a spectrum: z in [0.9, 1.3], 301 rows 112 and 117 us, 700 rows 143 and
+// 168, 2048 rows 234 and 258; past the line, z in [0, 12], two are faster for the gradient of 2048 rows (674 against 685: the dW
+// contraction reduces over a tile's whole window) and for 160 rows (109 against
+// 122), one for forward calls of 1024 and 2048 rows (182 and 281 against 204 and
+// 296).  So the line is right for narrow ranges and the gradients of large
+// batches, and leaves up to a tenth of a large forward call over a wide range.
 __device__ __forceinline__ int order_halves(const ModelDev& md, float zlo, float zhi) {
   float width = 0.f;
   if (md.n_filt > 0) width = logf(md.samp_lam_max / md.samp_lam_min);

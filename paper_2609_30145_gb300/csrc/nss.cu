@@ -16,9 +16,10 @@
 //
 // Prior volume: removing the j-th lowest of n live points shrinks the volume
 // by exp(-1 / (n - j)), the expectation of its log shrinkage; the removed
-// point's weight is the volume it leaves behind.  Evidence and information
-// are accumulated in FP64 by one thread in removal order (Skilling's
-// recurrence for H), so a run is deterministic for a given seed.
+// point's weight is the volume it leaves behind.  Evidence and information take
+// an iteration's points at once: FP64 sums over the block in a fixed order, every
+// term scaled by the largest (Skilling's recurrence for H after all of them), so
+// a run is deterministic for a given seed.
 #include <math.h>
 #include <string.h>
 

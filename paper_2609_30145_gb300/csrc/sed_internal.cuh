@@ -512,10 +512,13 @@ __device__ __forceinline__ void ln_rest(float2 p, float z_hi, float z_lo, float&
   x_lo = t - (x_hi - s);
 }
 
-// Programmatic dependent launch.  Every kernel of the library begins with
-// pdl_enter(): it waits until the kernel before it on the stream has completed
-// and its writes are visible, then lets the next kernel be scheduled.  Launched
-// directly on a stream, a kernel carries programmatic stream serialisation, so
+// Programmatic dependent launch.  Every kernel of the library calls pdl_enter()
+// before it touches anything that another kernel writes or reads: it waits until
+// the kernel before it on the stream has completed and its writes are visible,
+// then lets the next kernel be scheduled.  Most begin with it; the epilogue reads
+// the bands, the persistent contraction sets up its barriers and tensor memory
+// and k_prep_bwd reads the ages' cells before it.  Launched directly on a stream,
+// a kernel carries programmatic stream serialisation, so
 // its launch and scheduling overlap the previous kernel's work; results are
 // those of plain stream order.  Under stream capture the attribute is left off:
 // a graph replay already launches back to back, and measured slower with it.

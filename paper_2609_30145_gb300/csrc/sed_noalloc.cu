@@ -20,9 +20,10 @@
 // calls whose kernels can overlap on the GPU (different streams, or
 // different host threads) race on it and must be serialised by the caller.
 // Each call overwrites what it uses.  What must start from a known value is
-// set on the call's stream before its kernels: the per-tile window bounds
-// (two memsets, as in sed_loglike); the device error word of the
-// contraction is cleared by the first kernel of every call.
+// set on the call's stream: the per-tile windows and K-tile masks by the
+// ordering kernel, or by memsets where the rows keep the caller's order (a call
+// finds nothing left by the one before it, unlike sed_loglike's workspace); the
+// device error word of the contraction by the preparation kernel.
 //
 // FP8 is refused (SED_EUNSUPPORTED): its operand copy of the grid is built
 // with cudaMalloc on the first FP8 call of sed_loglike, so an allocation-free
