@@ -96,16 +96,6 @@ size_t epi_bwd_smem(const EpiBwdArgs& a) {
   return epi_bwd_lines_off(a) + lines;
 }
 
-// a / d from d's rounded reciprocal rd: the quotient's remainder, exact by FMA, times
-// rd corrects it to the rounded quotient (Markstein 1990, "Computation of elementary
-// functions on the IBM RISC System/6000 processor").  Two quotients by one d then
-// take one reciprocal: the gradient of 2048 rows with a spectrum takes 671.5 us so,
-// 689.5 with two divisions.
-__device__ __forceinline__ float div_rn(float a, float d, float rd) {
-  const float q = a * rd;
-  return fmaf(fmaf(-q, d, a), rd, q);
-}
-
 // LINES: an instance with the emission lines (the one without keeps its code free of them);
 // VAR: 1 the age-binned attenuation (one Y and one dlnL/dY per attenuated
 // block), 2 the nebular age axis (per-age ionising weights); 0 neither

@@ -1185,7 +1185,7 @@ __global__ void __launch_bounds__(PREP_BWD_THREADS) k_prep_bwd(const __grid_cons
       out[md.offs[SED_KEY_SFH] + k] = (k < NT ? gps0[k] : 0.f) + (k > 0 ? gps1[k - 1] : 0.f);
   } else
   for (int i = tid; i < NT; i += blockDim.x) {
-    const float Ti = T[i], Ti1 = T[i + 1], dT = Ti1 - Ti, mi = m[i], rate = mi / dT;
+    const float Ti = T[i], Ti1 = T[i + 1], dT = Ti1 - Ti, r_dT = __frcp_rn(dT), mi = m[i], rate = mi / dT;
     // first age whose cell reaches above T_i
     int a0 = 0, a1 = NA;
     while (a0 < a1) {
@@ -1201,7 +1201,7 @@ __global__ void __launch_bounds__(PREP_BWD_THREADS) k_prep_bwd(const __grid_cons
       const float lo = cell_lo[ag], hi = cell_hi[ag];
       const float ov = fminf(Ti1, hi) - fmaxf(Ti, lo);
       if (ov <= 0.f) continue;
-      const float f = ov / dT;   // the bin's share in the age's cell
+      const float f = div_rn(ov, dT, r_dT);   // the bin's share in the age's cell
       const float g0 = gWs[ag * NZ + j0];
       const float g1 = NZ > 1 ? gWs[ag * NZ + j0 + 1] : 0.f;
       const float gA = g0 * (1.f - t) + g1 * t;
