@@ -147,7 +147,10 @@ typedef struct {
    * SED_EUNSUPPORTED -- and a requested FP8 copy is built at load.  Per
    * layout the copies take 8 (3xTF32), 4 (FP32), 2 (BF16) and 1 (FP8) bytes
    * x Kpad x n_lam: a server that runs BF16 only keeps a fifth of the default
-   * footprint.  The gradient needs the copy of its precision (3xTF32 or FP32). */
+   * footprint.  The gradient needs the copy of its precision (3xTF32 or FP32).
+   * Without a mask and without a memory budget the grid also keeps its nebular
+   * template's cell corners side by side (16 bytes x n_logu x n_logz x n_lam, up to
+   * 64 MB), which the calls of nebular models then read (the same results). */
   unsigned precision_mask;
   /* Emission-line cube of the nebular grid (App. C): line luminosity per
    * ionising photon on the same (log U, log Z_gas) axes as the continuum
